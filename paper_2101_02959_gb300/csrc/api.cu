@@ -57,6 +57,8 @@ struct DevMem {
   }
 };
 
+constexpr size_t kWs64Cap = (size_t)1 << 30;  // workspace of the FP64 tensor-core updates
+
 inline int pad8(int n) { return (n + 7) & ~7; }
 inline long long pad32(long long n) { return (n + 31) & ~31LL; }
 
@@ -275,6 +277,7 @@ struct bd_handle {
   // FP32 with tensor cores: the inverse of every matrix's current 128 x 128 diagonal block
   // (128 x 128 floats per matrix of the largest batch), for the panel solves
   float *d_pinv = nullptr;
+  Slice64 ws64;  // FP64: digit planes of the tensor-core updates, panel inverses
   GemmTask *d_gemm = nullptr;
   int n_gemm = 0;
   int *d_ext_idx = nullptr;
@@ -833,6 +836,16 @@ void setup_handle(bd_handle &h) {
     if (h.mixed()) {  // the autotuner may turn the tensor cores on
       const int most = std::max({h.shK.count, h.shA.count, h.shC.count, 1});
       h.d_pinv = m.alloc<float>((size_t)most * 128 * 128);
+    } else {
+      // digit planes of the batch's largest update, at most kWs64Cap bytes (and one matrix)
+      size_t want = 0, one = 0;
+      for (const EngineShape *q : {&h.shK, &h.shA, &h.shC, &h.shCo}) {
+        want = std::max(want, slice64_bytes(q->count, q->max_m, q->max_e));
+        one = std::max(one, slice64_bytes(1, q->max_m, q->max_e));
+      }
+      h.ws64.bytes = std::max(one, std::min(want, kWs64Cap));
+      h.ws64.mem = m.alloc<unsigned char>(h.ws64.bytes);
+      h.ws64.pinv = m.alloc<double>((size_t)std::max({h.shK.count, h.shA.count, h.shC.count, 1}) * kPanel64 * kPanel64);
     }
     // sparse pattern of S_PP: the (p, q) pairs that some subdomain couples, with the
     // offsets of their local contributions in the augmented matrices (subdomain order)
@@ -1087,7 +1100,7 @@ void run_engine_groups(bd_handle &h, const EngineShape &all, const MatDesc *d_de
       g.max_e = std::max(g.max_e, all.e[q]);
     }
     engine_partial_cholesky<T>(g, d_desc + a, base, h.d_err, h.s, linv, &h.prof, h.opt.use_tensor_cores != 0,
-                               h.tune_panel_tc ? h.d_pinv : nullptr);
+                               h.tune_panel_tc ? h.d_pinv : nullptr, &h.ws64);
   }
 }
 
@@ -1113,7 +1126,7 @@ void linearize_t(bd_handle &h, Dense<T> &D, bool precond) {
   launch_copy<T, T>(h.cp_zx.n, h.cp_zx.max_elems, h.cp_zx.d, D.Aug, D.Z, s);
   launch_class_aug<T>(h.ncls, h.max_nc, h.d_cls, h.d_pairs, D.Blk, h.d_Cdesc, D.CA, s);
   engine_partial_cholesky<T>(h.shC, h.d_Cdesc, D.CA, h.d_err, s, D.Linv, &h.prof, h.opt.use_tensor_cores != 0,
-                             h.tune_panel_tc ? h.d_pinv : nullptr);
+                             h.tune_panel_tc ? h.d_pinv : nullptr, &h.ws64);
   launch_copy<T, T>(h.cp_sinv.n, h.cp_sinv.max_elems, h.cp_sinv.d, D.CA, D.Sinv, s);
   if (h.opt.scaling == BD_SCALING_RHO) {
     const double si = std::max({h.fp.sigma_i[0], h.fp.sigma_i[1], h.fp.sigma_i[2]});
@@ -1131,7 +1144,7 @@ void linearize_t(bd_handle &h, Dense<T> &D, bool precond) {
     EngineShape co = h.shCo;
     co.ob = h.tune_ob;
     engine_partial_cholesky<T>(co, h.d_Codesc, D.Co, h.d_err, s, D.LdCo, &h.prof, h.opt.use_tensor_cores != 0,
-                               h.tune_panel_tc ? h.d_pinv : nullptr);
+                               h.tune_panel_tc ? h.d_pinv : nullptr, &h.ws64);
   }
   launch_copy<T, T>(h.cp_coinv.n, h.cp_coinv.max_elems, h.cp_coinv.d, D.Co, D.CoInv, s);
   if (h.d_CoInv64) coarse_refine64<T>(h.np, D.CoInv, pad8(h.np), h.d_Co64d, h.d_CoInv64, h.d_CoW, h.d_CoY, s);
@@ -1875,6 +1888,10 @@ int bidomain_setup(const bd_mesh *mesh, const bd_conductivity *cond, const bd_io
     h->tune_panel_tc = h->opt.use_tensor_cores == 2 ? 1 : 0;
     if (h->opt.learned_guess && !gemm_tc_configure()) {
       g_last_error = "tensor-core GEMM configuration failed";
+      return BD_ERR_CUDA;
+    }
+    if (!tc64_configure()) {
+      g_last_error = "FP64 tensor-core kernel configuration failed";
       return BD_ERR_CUDA;
     }
     if (!dense_configure()) {

@@ -17,14 +17,6 @@
 
 namespace bd {
 
-template <typename T> __device__ inline T dsqrt(T v);
-template <> __device__ inline float dsqrt<float>(float v) { return sqrtf(v); }
-template <> __device__ inline double dsqrt<double>(double v) { return sqrt(v); }
-// 1 / sqrt(v): the hardware estimate for float (relative error a few units in the
-// last place, the level of FP32 rounding in the factors), the library routine for double
-template <typename T> __device__ inline T drsqrt(T v);
-template <> __device__ inline float drsqrt<float>(float v) { return rsqrtf(v); }
-template <> __device__ inline double drsqrt<double>(double v) { return rsqrt(v); }
 
 // 16-byte vectors of T (row starts of the batched matrices are 32-byte aligned).
 template <typename T> struct Vec16;
@@ -61,7 +53,9 @@ __device__ __forceinline__ void warp_chol32(T (&a)[32], int lane, int wb, bool &
     if (c < wb) {  // uniform across the warp
       T piv = __shfl_sync(0xffffffffu, a[c], c);
       if (!(piv > T(0))) { bad = true; piv = T(1); }
-      const T inv = drsqrt(piv), sd = piv * inv;
+      // the hardware estimate: relative error a few units in the last place, the level of
+      // FP32 rounding in the factors
+      const T inv = rsqrtf(piv), sd = piv * inv;
       a[c] = (lane == c) ? sd : a[c] * inv;  // rows above c hold 0 here
 #pragma unroll
       for (int t = c + 1; t < 32; ++t) {
@@ -87,7 +81,6 @@ constexpr int kPW = kEnginePanel;  // outer panel width
 constexpr int kLDP = kPW + 4;      // row stride of the staged panel (16-byte aligned rows)
 template <typename T> struct PanelRows;
 template <> struct PanelRows<float> { static constexpr int RB = 128; };
-template <> struct PanelRows<double> { static constexpr int RB = 16; };
 
 template <typename T, bool ROWS>
 constexpr size_t bigpanel_smem() {
@@ -376,103 +369,18 @@ __global__ void __launch_bounds__(256, 1) k_diag_inverse(const MatDesc *__restri
   }
 }
 
-// ---- rank-k update of lower tiles --------------------------------------------
-// Two-level right-looking blocking: inner panels of kNB columns inside outer
-// panels [K0, K1) of kOB columns.
-// mode 0 (inner): rows [k0+w, m), cols [k0+w, min(K1, e)), K = [k0, k0+w), w = one engine panel
-// mode 2 (outer): rows [K1, m),   cols [K1, e),            K = [K0, K1)
-// mode 1 (final): rows [e, m),    cols [e, m),             K = [0, e)
-// C[r][c] -= sum_k A[r][k] A[c][k]; 64x64 tiles, 256 threads, 4x4 per thread.
-constexpr int kTB = 64, kKC = 32;
-
-template <typename T>
-__global__ void __launch_bounds__(256) k_rankk(const MatDesc *__restrict__ desc, T *__restrict__ base, int mode,
-                                               int k0, int K0, int K1, int nct) {
-  const MatDesc d = desc[blockIdx.y];
-  int row0, colend, kb, ke;
-  if (mode == 0) {
-    if (k0 >= d.e) return;
-    const int w = min(kEnginePanel, d.e - k0);
-    row0 = k0 + w;
-    colend = min(K1, d.e);
-    kb = k0;
-    ke = k0 + w;
-  } else if (mode == 2) {
-    if (K1 >= d.e) return;
-    row0 = K1;
-    colend = d.e;
-    kb = K0;
-    ke = K1;
-  } else {
-    row0 = d.e;
-    colend = d.m;
-    kb = 0;
-    ke = d.e;
-  }
-  const BandRows br = band_rows(d, row0, ke);  // rows past the band hold zeros in K = [kb, ke)
-  if (mode != 1) colend = min(colend, band_limit(d, ke));
-  const int ti = blockIdx.x / nct, tj = blockIdx.x % nct;
-  if (tj > ti) return;
-  const int v0 = ti * kTB, c0 = row0 + tj * kTB;
-  if (mode == 1 && d.ifirst && v0 < br.nv) kb = max(kb, d.ifirst[v0] & ~3);  // rows' L starts there
-  if (v0 >= br.nv || c0 >= colend || ke <= kb) return;
-  T *A = base + d.off;
-  __shared__ T As[kKC][kTB + 1];  // row pad 65: the strided stores below hit distinct banks
-  __shared__ T Bs[kKC][kTB + 1];
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  T acc[4][4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = T(0);
-  const int lr = tid >> 2, lk = (tid & 3) * 8;
-  for (int kk = kb; kk < ke; kk += kKC) {
-    {
-      const bool va = v0 + lr < br.nv;
-      const int ra = va ? br.row(v0 + lr) : 0, rb = c0 + lr;
-#pragma unroll
-      for (int q = 0; q < 8; ++q) {
-        const int k = kk + lk + q;
-        As[lk + q][lr] = (va && k < ke) ? A[(long long)ra * d.ld + k] : T(0);
-        Bs[lk + q][lr] = (rb < colend && k < ke) ? A[(long long)rb * d.ld + k] : T(0);
-      }
-    }
-    __syncthreads();
-#pragma unroll 8
-    for (int k = 0; k < kKC; ++k) {
-      T av[4], bv[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) av[i] = As[k][ty + 16 * i];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) bv[j] = Bs[k][tx + 16 * j];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] += av[i] * bv[j];
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int v = v0 + ty + 16 * i;
-    if (v >= br.nv) continue;
-    const int r = br.row(v);
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int c = c0 + tx + 16 * j;
-      if (c < colend) A[(long long)r * d.ld + c] -= acc[i][j];
-    }
-  }
-}
-
 std::atomic<long long> g_launches{0};
 void count_launch(int n) { g_launches += n; }
 long long launch_count() { return g_launches.load(); }
 
 
-// ---- FP32 rank-k update: 128x128 CTA tiles, 8x8 outputs per thread ----------
-// Same modes and index ranges as k_rankk.  K is consumed in chunks of 16 with
-// the next chunk prefetched into registers while the current one is used.
+// ---- FP32 rank-k update of lower tiles: 128x128 CTA tiles, 8x8 outputs per thread ----------
+// C[r][c] -= sum_k A[r][k] A[c][k] with
+// mode 0 (in-block): rows [k0+w, m), cols [k0+w, min(K1, e)), K = [k0, k0+w), w = one panel
+// mode 2 (outer):    rows [K1, m),   cols [K1, e),            K = [K0, K1)
+// mode 1 (final):    rows [e, m),    cols [e, m),             K = [0, e)
+// K is consumed in chunks of 16 with the next chunk prefetched into registers while the
+// current one is used.  (The FP64 updates run on the tensor cores, tc64.cu.)
 constexpr int kTB2 = 128, kKC2 = 16;
 
 __global__ void __launch_bounds__(256) k_rankk128(const MatDesc *__restrict__ desc, float *__restrict__ base,
@@ -577,16 +485,7 @@ __global__ void __launch_bounds__(256) k_rankk128(const MatDesc *__restrict__ de
   }
 }
 
-template <typename T>
-static void launch_rankk(const MatDesc *d_desc, T *base, int mode, int k0, int K0, int K1, int max_rows, int max_cols,
-                         int count, cudaStream_t s) {
-  const int nrt = ceil_div(max_rows, kTB), nct = ceil_div(max_cols, kTB);
-  if (nrt == 0 || nct == 0) return;
-  k_rankk<T><<<dim3(nrt * nct, count), 256, 0, s>>>(d_desc, base, mode, k0, K0, K1, nct);
-  count_launch();
-}
-template <>
-void launch_rankk<float>(const MatDesc *d_desc, float *base, int mode, int k0, int K0, int K1, int max_rows,
+static void launch_rankk(const MatDesc *d_desc, float *base, int mode, int k0, int K0, int K1, int max_rows,
                          int max_cols, int count, cudaStream_t s) {
   const int nrt = ceil_div(max_rows, kTB2), nct = ceil_div(max_cols, kTB2);
   if (nrt == 0 || nct == 0) return;
@@ -609,9 +508,10 @@ static double band_entries(const MatDesc &hd, int t0, int ke, int cend) {
 
 template <typename T>
 void engine_partial_cholesky(const EngineShape &sh, const MatDesc *d_desc, T *base, int *d_err, cudaStream_t s,
-                             T *store, ProfHook *prof, bool tc, float *pinv) {
+                             T *store, ProfHook *prof, bool tc, float *pinv, const Slice64 *ws64) {
   if (sh.count == 0) return;
-  constexpr int RB = PanelRows<T>::RB;
+  constexpr bool f64 = std::is_same<T, double>::value;
+  constexpr int PW = f64 ? kPanel64 : kPW;
   const int ob = std::max(kPW, (sh.ob / kPW) * kPW);  // outer block: columns per long-K trailing update
   // host copies of the descriptors' sizes and bands: the grids cover the rows and columns
   // the band lets an update reach (the kernels apply the same limits per matrix)
@@ -625,12 +525,12 @@ void engine_partial_cholesky(const EngineShape &sh, const MatDesc *d_desc, T *ba
   }
   for (int K0 = 0; K0 < sh.max_e; K0 += ob) {
     const int K1 = K0 + ob;
-    for (int k0 = K0; k0 < std::min(K1, sh.max_e); k0 += kPW) {
+    for (int k0 = K0; k0 < std::min(K1, sh.max_e); k0 += PW) {
       int max_below = 0, max_cols = 0;
       double fl_panel = 0.0, fl_in = 0.0;
       for (int b = 0; b < sh.count; ++b) {
         if (k0 >= sh.e[b]) continue;
-        const int w = std::min(kPW, sh.e[b] - k0);
+        const int w = std::min(PW, sh.e[b] - k0);
         const int below = band_rows(hd[b], k0 + w, k0 + w).nv;
         const int cend = std::min({K1, sh.e[b], band_limit(hd[b], k0 + w)});
         max_below = std::max(max_below, below);
@@ -639,21 +539,19 @@ void engine_partial_cholesky(const EngineShape &sh, const MatDesc *d_desc, T *ba
         fl_in += 2.0 * w * band_entries(hd[b], k0 + w, k0 + w, cend);
       }
       if (prof) prof->begin(PROF_PANEL, s);
-      k_bigpanel<T, false><<<dim3(1, sh.count), 256, bigpanel_smem<T, false>(), s>>>(d_desc, base, k0, d_err, store);
-      count_launch();
-      if (max_below > 0) {
-        bool done_rows = false;
-        if constexpr (std::is_same<T, float>::value) {
-          if (tc && pinv) {  // L_21 = A_21 L_11^-T as one tensor-core product with the block's inverse
-            k_diag_inverse<<<dim3(1, sh.count), 256, kInvSmem, s>>>(d_desc, base, k0, pinv);
-            count_launch();
-            launch_rankk_tc(d_desc, base, 3, k0, 0, max_below, kPW, sh.count, d_err, s, pinv);
-            done_rows = true;
-          }
-        }
-        if (!done_rows) {
-          k_bigpanel<T, true><<<dim3(ceil_div(max_below, RB), sh.count), 256, bigpanel_smem<T, true>(), s>>>(
-              d_desc, base, k0, d_err, store);
+      if constexpr (f64) {
+        launch_diag64(d_desc, base, k0, sh.count, d_err, store, ws64->pinv, s);
+        launch_update64(d_desc, base, Upd64{3, k0, 0, PW, 0, 0}, max_below, PW, sh.count, *ws64, d_err, s, ws64->pinv);
+      } else {
+        k_bigpanel<T, false><<<dim3(1, sh.count), 256, bigpanel_smem<T, false>(), s>>>(d_desc, base, k0, d_err, store);
+        count_launch();
+        if (max_below > 0 && tc && pinv) {  // L_21 = A_21 L_11^-T as one tensor-core product with the block's inverse
+          k_diag_inverse<<<dim3(1, sh.count), 256, kInvSmem, s>>>(d_desc, base, k0, pinv);
+          count_launch();
+          launch_rankk_tc(d_desc, base, 3, k0, 0, max_below, kPW, sh.count, d_err, s, pinv);
+        } else if (max_below > 0) {
+          k_bigpanel<T, true><<<dim3(ceil_div(max_below, PanelRows<T>::RB), sh.count), 256, bigpanel_smem<T, true>(),
+                                s>>>(d_desc, base, k0, d_err, store);
           count_launch();
         }
       }
@@ -662,12 +560,12 @@ void engine_partial_cholesky(const EngineShape &sh, const MatDesc *d_desc, T *ba
       // with the panels (the long-K class holds only the trailing updates)
       if (max_below > 0 && max_cols > 0) {
         if (prof) prof->begin(PROF_PANEL, s);
-        if constexpr (std::is_same<T, float>::value) {
+        if constexpr (f64) {
+          launch_update64(d_desc, base, Upd64{0, k0, K1, PW, 0, 0}, max_below, max_cols, sh.count, *ws64, d_err, s);
+        } else {
           static_assert(kPW == 128, "the tensor-core in-block update takes 128-column panels");
           if (tc) launch_rankk_tc(d_desc, base, 0, k0, K1, max_below, max_cols, sh.count, d_err, s);
-          else launch_rankk<T>(d_desc, base, 0, k0, K0, K1, max_below, max_cols, sh.count, s);
-        } else {
-          launch_rankk<T>(d_desc, base, 0, k0, K0, K1, max_below, max_cols, sh.count, s);
+          else launch_rankk(d_desc, base, 0, k0, K0, K1, max_below, max_cols, sh.count, s);
         }
         if (prof) prof->end(PROF_PANEL, s, fl_in, 0.0);
       }
@@ -688,9 +586,9 @@ void engine_partial_cholesky(const EngineShape &sh, const MatDesc *d_desc, T *ba
       if (prof) prof->begin(PROF_RANKK, s);
       if constexpr (std::is_same<T, float>::value) {
         if (tc) launch_rankk_tc(d_desc, base, 2, K0, K1, max_rows, max_cols, sh.count, d_err, s);
-        else launch_rankk<T>(d_desc, base, 2, 0, K0, K1, max_rows, max_cols, sh.count, s);
+        else launch_rankk(d_desc, base, 2, 0, K0, K1, max_rows, max_cols, sh.count, s);
       } else {
-        launch_rankk<T>(d_desc, base, 2, 0, K0, K1, max_rows, max_cols, sh.count, s);
+        launch_update64(d_desc, base, Upd64{2, K0, K1, PW, K0, K1}, max_rows, max_cols, sh.count, *ws64, d_err, s);
       }
       if (prof) prof->end(PROF_RANKK, s, fl, by);
     }
@@ -717,9 +615,9 @@ void engine_partial_cholesky(const EngineShape &sh, const MatDesc *d_desc, T *ba
     if (prof) prof->begin(PROF_RANKK, s);
     if constexpr (std::is_same<T, float>::value) {
       if (tc) launch_rankk_tc(d_desc, base, 1, 0, 0, max_t, max_t, sh.count, d_err, s);
-      else launch_rankk<T>(d_desc, base, 1, 0, 0, 0, max_t, max_t, sh.count, s);
+      else launch_rankk(d_desc, base, 1, 0, 0, 0, max_t, max_t, sh.count, s);
     } else {
-      launch_rankk<T>(d_desc, base, 1, 0, 0, 0, max_t, max_t, sh.count, s);
+      launch_update64(d_desc, base, Upd64{1, 0, 0, PW, 0, sh.max_e}, max_t, max_t, sh.count, *ws64, d_err, s);
     }
     if (prof) prof->end(PROF_RANKK, s, fl, by);
   }
@@ -1344,10 +1242,6 @@ bool dense_configure() {
                              (int)bigpanel_smem<float, false>()) == cudaSuccess;
   ok &= cudaFuncSetAttribute(k_bigpanel<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)bigpanel_smem<float, true>()) == cudaSuccess;
-  ok &= cudaFuncSetAttribute(k_bigpanel<double, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)bigpanel_smem<double, false>()) == cudaSuccess;
-  ok &= cudaFuncSetAttribute(k_bigpanel<double, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)bigpanel_smem<double, true>()) == cudaSuccess;
   ok &= cudaFuncSetAttribute(k_trsv<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim) == cudaSuccess;
   ok &= cudaFuncSetAttribute(k_trsv<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim) == cudaSuccess;
   ok &= cudaFuncSetAttribute(k_gemv<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim) == cudaSuccess;
@@ -1368,7 +1262,7 @@ bool dense_configure() {
 
 #define BD_INST(T)                                                                                              \
   template void engine_partial_cholesky<T>(const EngineShape &, const MatDesc *, T *, int *, cudaStream_t,    \
-                                           T *, ProfHook *, bool, float *);                                    \
+                                           T *, ProfHook *, bool, float *, const Slice64 *);                                    \
   template void launch_gemv<T>(int, int, int, const GemvDesc *, const T *, const double *, const int *,        \
                                double *, double, const int *, cudaStream_t);                                   \
   template void launch_symv_rows<T>(int, const T *, int, const double *, double *, int, const int *,           \

@@ -72,6 +72,18 @@ void launch_dot3(int n, const double *a0, const double *b0, const double *a1, co
 void launch_gauge_shift(int n, double *ui, double *ue, const double *scal, cudaStream_t s);
 void launch_sum_partials(int nblk, const double *partial, double *out, cudaStream_t s);
 
+// tc64.cu -- FP64 rank-k updates and panel solves on the tensor cores (exact digit products).
+constexpr int kPanel64 = 64;   // panel width of the FP64 engine
+constexpr int kSliceK = 1024;  // columns whose digit planes the workspace holds at a time
+struct Upd64 {                 // one update over a batch (modes as in tc64.cu)
+  int mode, K0, K1, pw, ka, kz;
+};
+struct Slice64 {               // workspace: digit planes, row exponents; pinv: a panel inverse per matrix
+  unsigned char *mem = nullptr;
+  size_t bytes = 0;
+  double *pinv = nullptr;
+};
+
 // dense.cu -- batched partial Cholesky: eliminates the first e columns of every
 // matrix; afterwards the trailing (m-e) x (m-e) lower triangle holds the Schur
 // complement A22 - A21 A11^-1 A12 and the first e columns hold L11 and L21.
@@ -95,10 +107,20 @@ constexpr int kEnginePanel = 128;
 // every panel are solved as one tensor-core product with the inverse of the diagonal block.
 template <typename T>
 void engine_partial_cholesky(const EngineShape &sh, const MatDesc *d_desc, T *base, int *d_err, cudaStream_t s,
-                             T *store, ProfHook *prof = nullptr, bool tc = false, float *pinv = nullptr);
+                             T *store, ProfHook *prof = nullptr, bool tc = false, float *pinv = nullptr,
+                             const Slice64 *ws64 = nullptr);
 
 bool dense_configure();
 size_t dense_smem_limit();  // bytes of shared memory the dense kernels may stage per CTA
+
+// tc64.cu
+bool tc64_configure();
+// workspace of `count` matrices of max_rows rows and max_e eliminated columns at once
+size_t slice64_bytes(int count, int max_rows, int max_e);
+void launch_update64(const MatDesc *d_desc, double *base, Upd64 u, int max_rows, int max_cols, int count,
+                     const Slice64 &ws, int *err, cudaStream_t s, const double *pinv = nullptr);
+void launch_diag64(const MatDesc *d_desc, double *base, int K0, int count, int *err, double *store, double *pinv,
+                   cudaStream_t s);
 
 // tc.cu
 bool tc_configure();
