@@ -57,7 +57,8 @@ struct DevMem {
   }
 };
 
-constexpr size_t kWs64Cap = (size_t)1 << 30;  // workspace of the FP64 tensor-core updates
+// workspace of the tensor-core updates
+constexpr size_t kWsCap64 = (size_t)1 << 30, kWsCap32 = (size_t)512 << 20;
 
 inline int pad8(int n) { return (n + 7) & ~7; }
 inline long long pad32(long long n) { return (n + 31) & ~31LL; }
@@ -274,10 +275,8 @@ struct bd_handle {
   // the operator S_Gamma and the local solve [X; Psi^T] as symmetric products (X, S_Gamma
   // symmetric: each lower tile read once); used instead of gv_schur / gv_local when set
   SymvSet sv_schur, sv_local;
-  // FP32 with tensor cores: the inverse of every matrix's current 128 x 128 diagonal block
-  // (128 x 128 floats per matrix of the largest batch), for the panel solves
-  float *d_pinv = nullptr;
-  Slice64 ws64;  // FP64: digit planes of the tensor-core updates, panel inverses
+  // tensor-core factorisation: digit planes of the updates, inverses of the panels' diagonal blocks
+  SliceWs ws;
   GemmTask *d_gemm = nullptr;
   int n_gemm = 0;
   int *d_ext_idx = nullptr;
@@ -318,12 +317,13 @@ struct bd_handle {
   double rtol_scale = 1.0;
   // factorisation tuning (bidomain_autotune): outer panel width, batch groups, tensor cores
   int tune_ob = 256, tune_groups = 1;
-  int tune_panel_tc = 0;  // 1: panel solves on the tensor cores too (with d_pinv; tensor cores on)
+  int tune_panel_tc = 0;  // 1: panel solves on the tensor cores too (tensor cores on)
   cudaGraphExec_t pcg_exec[2] = {nullptr, nullptr};  // captured PCG chunk per method
   size_t pcg_nodes[2] = {0, 0};
   double gemv_schur_flops = 0, gemv_schur_bytes = 0, gemv_local_flops = 0, gemv_local_bytes = 0;
 
   bool mixed() const { return opt.precision == BD_MIXED; }
+  int tc() const { return opt.use_tensor_cores ? 1 + tune_panel_tc : 0; }
   int check_err() {
     int e = 0;
     ck(cudaMemcpyAsync(&e, d_err, sizeof(int), cudaMemcpyDeviceToHost, s), "read error flag");
@@ -833,19 +833,20 @@ void setup_handle(bd_handle &h) {
     h.d_Codesc = m.upload(std::vector<MatDesc>{co}, s);
     h.shCo = EngineShape{1, np, 2 * np, {2 * np}, {np}};
     h.shCo.id0 = {np};
-    if (h.mixed()) {  // the autotuner may turn the tensor cores on
-      const int most = std::max({h.shK.count, h.shA.count, h.shC.count, 1});
-      h.d_pinv = m.alloc<float>((size_t)most * 128 * 128);
-    } else {
-      // digit planes of the batch's largest update, at most kWs64Cap bytes (and one matrix)
+    {  // (in mixed precision the autotuner may turn the tensor cores on)
       size_t want = 0, one = 0;
+      int most = 1;
       for (const EngineShape *q : {&h.shK, &h.shA, &h.shC, &h.shCo}) {
-        want = std::max(want, slice64_bytes(q->count, q->max_m, q->max_e));
-        one = std::max(one, slice64_bytes(1, q->max_m, q->max_e));
+        auto need = [&](int n) {
+          return h.mixed() ? slice_bytes<float>(n, q->max_m, q->max_e) : slice_bytes<double>(n, q->max_m, q->max_e);
+        };
+        want = std::max(want, need(q->count));
+        one = std::max(one, need(1));
+        most = std::max(most, q->count);
       }
-      h.ws64.bytes = std::max(one, std::min(want, kWs64Cap));
-      h.ws64.mem = m.alloc<unsigned char>(h.ws64.bytes);
-      h.ws64.pinv = m.alloc<double>((size_t)std::max({h.shK.count, h.shA.count, h.shC.count, 1}) * kPanel64 * kPanel64);
+      h.ws.bytes = std::max(one, std::min(want, h.mixed() ? kWsCap32 : kWsCap64));
+      h.ws.mem = m.alloc<unsigned char>(h.ws.bytes);
+      h.ws.pinv = m.alloc<unsigned char>((size_t)most * kPanel64 * kPanel64 * (h.mixed() ? sizeof(float) : sizeof(double)));
     }
     // sparse pattern of S_PP: the (p, q) pairs that some subdomain couples, with the
     // offsets of their local contributions in the augmented matrices (subdomain order)
@@ -1099,8 +1100,7 @@ void run_engine_groups(bd_handle &h, const EngineShape &all, const MatDesc *d_de
       g.max_m = std::max(g.max_m, all.m[q]);
       g.max_e = std::max(g.max_e, all.e[q]);
     }
-    engine_partial_cholesky<T>(g, d_desc + a, base, h.d_err, h.s, linv, &h.prof, h.opt.use_tensor_cores != 0,
-                               h.tune_panel_tc ? h.d_pinv : nullptr, &h.ws64);
+    engine_partial_cholesky<T>(g, d_desc + a, base, h.d_err, h.s, linv, &h.prof, h.tc(), h.ws);
   }
 }
 
@@ -1125,8 +1125,7 @@ void linearize_t(bd_handle &h, Dense<T> &D, bool precond) {
   run_engine_groups<T>(h, h.shA, h.d_Adesc, D.Aug, D.Linv);
   launch_copy<T, T>(h.cp_zx.n, h.cp_zx.max_elems, h.cp_zx.d, D.Aug, D.Z, s);
   launch_class_aug<T>(h.ncls, h.max_nc, h.d_cls, h.d_pairs, D.Blk, h.d_Cdesc, D.CA, s);
-  engine_partial_cholesky<T>(h.shC, h.d_Cdesc, D.CA, h.d_err, s, D.Linv, &h.prof, h.opt.use_tensor_cores != 0,
-                             h.tune_panel_tc ? h.d_pinv : nullptr, &h.ws64);
+  engine_partial_cholesky<T>(h.shC, h.d_Cdesc, D.CA, h.d_err, s, D.Linv, &h.prof, h.tc(), h.ws);
   launch_copy<T, T>(h.cp_sinv.n, h.cp_sinv.max_elems, h.cp_sinv.d, D.CA, D.Sinv, s);
   if (h.opt.scaling == BD_SCALING_RHO) {
     const double si = std::max({h.fp.sigma_i[0], h.fp.sigma_i[1], h.fp.sigma_i[2]});
@@ -1143,8 +1142,7 @@ void linearize_t(bd_handle &h, Dense<T> &D, bool precond) {
   {  // one large matrix: its trailing updates go to the tensor cores like the local ones
     EngineShape co = h.shCo;
     co.ob = h.tune_ob;
-    engine_partial_cholesky<T>(co, h.d_Codesc, D.Co, h.d_err, s, D.LdCo, &h.prof, h.opt.use_tensor_cores != 0,
-                               h.tune_panel_tc ? h.d_pinv : nullptr, &h.ws64);
+    engine_partial_cholesky<T>(co, h.d_Codesc, D.Co, h.d_err, s, D.LdCo, &h.prof, h.tc(), h.ws);
   }
   launch_copy<T, T>(h.cp_coinv.n, h.cp_coinv.max_elems, h.cp_coinv.d, D.Co, D.CoInv, s);
   if (h.d_CoInv64) coarse_refine64<T>(h.np, D.CoInv, pad8(h.np), h.d_Co64d, h.d_CoInv64, h.d_CoW, h.d_CoY, s);
@@ -1880,18 +1878,14 @@ int bidomain_setup(const bd_mesh *mesh, const bd_conductivity *cond, const bd_io
     ck(cudaStreamCreateWithFlags(&h->s2, cudaStreamNonBlocking), "stream");
     ck(cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming), "event");
     ck(cudaEventCreateWithFlags(&h->ev_join, cudaEventDisableTiming), "event");
-    if (h->opt.use_tensor_cores && h->opt.precision == BD_MIXED && !tc_configure()) {
-      g_last_error = "tensor-core kernel configuration failed";
-      return BD_ERR_CUDA;
-    }
     if (h->opt.precision != BD_MIXED) h->opt.use_tensor_cores = 0;
     h->tune_panel_tc = h->opt.use_tensor_cores == 2 ? 1 : 0;
     if (h->opt.learned_guess && !gemm_tc_configure()) {
       g_last_error = "tensor-core GEMM configuration failed";
       return BD_ERR_CUDA;
     }
-    if (!tc64_configure()) {
-      g_last_error = "FP64 tensor-core kernel configuration failed";
+    if (!digits_configure()) {
+      g_last_error = "tensor-core kernel configuration failed";
       return BD_ERR_CUDA;
     }
     if (!dense_configure()) {
@@ -2176,10 +2170,10 @@ int bidomain_autotune(bd_handle *h, bd_tune_result *out) {
     ck(cudaEventCreate(&e1), "event");
     const int prof_on = h->prof.on;
     h->prof.on = 0;
-    const int tc0 = h->opt.use_tensor_cores ? 1 + h->tune_panel_tc : 0, ob0 = h->tune_ob, g0 = h->tune_groups;
+    const int tc0 = h->tc(), ob0 = h->tune_ob, g0 = h->tune_groups;
     auto set_tc = [&](int tc) {  // 0 SIMT, 1 tensor-core updates, 2 also the panel solves
       h->opt.use_tensor_cores = tc > 0;
-      h->tune_panel_tc = tc == 2 && h->d_pinv;
+      h->tune_panel_tc = tc == 2;
     };
     auto time_it = [&]() {
       linearize(*h);  // warm
@@ -2200,7 +2194,6 @@ int bidomain_autotune(bd_handle *h, bd_tune_result *out) {
     int best_ob = ob0, best_g = g0, best_tc = tc0, n = 0;
     for (int tc : {0, 1, 2}) {
       if (tc && !h->mixed()) continue;
-      if (tc == 2 && !h->d_pinv) continue;
       for (int ob : {128, 256, 512})
         for (int g : {1, 2, 4}) {
           set_tc(tc);

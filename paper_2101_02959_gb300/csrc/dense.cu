@@ -297,82 +297,9 @@ __global__ void __launch_bounds__(256, 2) k_bigpanel(const MatDesc *__restrict__
   }
 }
 
-// ---- inverse of a factored diagonal block (tensor-core panel solve) -------------
-// L_11^-1 for the w x w factored diagonal block at [K0, K0 + w) of every matrix (one CTA
-// each), into pinv (128 x 128 per matrix, row-major, zero outside the lower w x w part), so
-// that the rows below the panel become one product L_21 = A_21 L_11^-T on the tensor cores.
-// 32 x 32 blocks: the four diagonal blocks by substitution (warp b, lane = column, the column
-// in registers), then the blocks at distance 1, 2, 3 below the diagonal,
-// Y_ij = -Y_ii (sum_{k=j}^{i-1} L_ik Y_kj), all threads over the entries of one distance.
-constexpr int kInvLD = kPW + 1;
-constexpr size_t kInvSmem = sizeof(float) * (2 * (size_t)kPW * kInvLD + 3 * 32 * 33);
-
-__global__ void __launch_bounds__(256, 1) k_diag_inverse(const MatDesc *__restrict__ desc,
-                                                         const float *__restrict__ base, int K0,
-                                                         float *__restrict__ pinv) {
-  const MatDesc d = desc[blockIdx.y];
-  if (K0 >= d.e) return;
-  const int w = min(kPW, d.e - K0), nbk = (w + 31) / 32;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  float *Ls = reinterpret_cast<float *>(smem_raw);  // [128][129] L_11, lower, identity past w
-  float *Ys = Ls + kPW * kInvLD;                      // [128][129] the inverse
-  float *Tm = Ys + kPW * kInvLD;                      // [3][32][33] sums of one distance
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const float *A = base + d.off + (long long)K0 * d.ld + K0;
-  for (int e = tid; e < kPW * kPW; e += 256) {
-    const int i = e / kPW, j = e % kPW;
-    float v = 0.f;
-    if (i < w && j < w) v = j <= i ? A[(long long)i * d.ld + j] : 0.f;
-    else if (i == j) v = 1.f;
-    Ls[i * kInvLD + j] = v;
-    Ys[i * kInvLD + j] = 0.f;
-  }
-  __syncthreads();
-  if (warp < 4) {  // diagonal block b = warp: lane = column j, forward substitution down the rows
-    const int b0 = 32 * warp;
-    float y[32];
-#pragma unroll
-    for (int i = 0; i < 32; ++i) {
-      float sacc = (i == lane) ? 1.f : 0.f;
-#pragma unroll
-      for (int k = 0; k < i; ++k) sacc -= Ls[(b0 + i) * kInvLD + b0 + k] * y[k];
-      y[i] = sacc / Ls[(b0 + i) * kInvLD + b0 + i];
-    }
-#pragma unroll
-    for (int i = 0; i < 32; ++i) Ys[(b0 + i) * kInvLD + b0 + lane] = i >= lane ? y[i] : 0.f;
-  }
-  __syncthreads();
-  for (int dist = 1; dist < nbk; ++dist) {
-    const int nblk = nbk - dist;  // output blocks (j + dist, j), j < nblk
-    for (int e = tid; e < nblk * 1024; e += 256) {
-      const int j = e / 1024, r = (e % 1024) / 32, c = e % 32, i = j + dist;
-      float t = 0.f;
-      for (int k = j; k < i; ++k)
-#pragma unroll 8
-        for (int q = 0; q < 32; ++q) t += Ls[(32 * i + r) * kInvLD + 32 * k + q] * Ys[(32 * k + q) * kInvLD + 32 * j + c];
-      Tm[(j * 32 + r) * 33 + c] = t;
-    }
-    __syncthreads();
-    for (int e = tid; e < nblk * 1024; e += 256) {
-      const int j = e / 1024, r = (e % 1024) / 32, c = e % 32, i = j + dist;
-      float t = 0.f;
-#pragma unroll 8
-      for (int q = 0; q < 32; ++q) t += Ys[(32 * i + r) * kInvLD + 32 * i + q] * Tm[(j * 32 + q) * 33 + c];
-      Ys[(32 * i + r) * kInvLD + 32 * j + c] = -t;
-    }
-    __syncthreads();
-  }
-  float *out = pinv + (long long)blockIdx.y * kPW * kPW;
-  for (int e = tid; e < kPW * kPW; e += 256) {
-    const int i = e / kPW, j = e % kPW;
-    out[e] = (i < w && j < w && j <= i) ? Ys[i * kInvLD + j] : 0.f;
-  }
-}
-
 std::atomic<long long> g_launches{0};
 void count_launch(int n) { g_launches += n; }
 long long launch_count() { return g_launches.load(); }
-
 
 // ---- FP32 rank-k update of lower tiles: 128x128 CTA tiles, 8x8 outputs per thread ----------
 // C[r][c] -= sum_k A[r][k] A[c][k] with
@@ -508,10 +435,12 @@ static double band_entries(const MatDesc &hd, int t0, int ke, int cend) {
 
 template <typename T>
 void engine_partial_cholesky(const EngineShape &sh, const MatDesc *d_desc, T *base, int *d_err, cudaStream_t s,
-                             T *store, ProfHook *prof, bool tc, float *pinv, const Slice64 *ws64) {
+                             T *store, ProfHook *prof, int tc, const SliceWs &ws) {
   if (sh.count == 0) return;
   constexpr bool f64 = std::is_same<T, double>::value;
-  constexpr int PW = f64 ? kPanel64 : kPW;
+  const bool narrow = f64 || tc == 2;  // 64-column panels solved on the tensor cores
+  const int PW = narrow ? kPanel64 : kPW;
+  T *pinv = static_cast<T *>(ws.pinv);
   const int ob = std::max(kPW, (sh.ob / kPW) * kPW);  // outer block: columns per long-K trailing update
   // host copies of the descriptors' sizes and bands: the grids cover the rows and columns
   // the band lets an update reach (the kernels apply the same limits per matrix)
@@ -539,17 +468,13 @@ void engine_partial_cholesky(const EngineShape &sh, const MatDesc *d_desc, T *ba
         fl_in += 2.0 * w * band_entries(hd[b], k0 + w, k0 + w, cend);
       }
       if (prof) prof->begin(PROF_PANEL, s);
-      if constexpr (f64) {
-        launch_diag64(d_desc, base, k0, sh.count, d_err, store, ws64->pinv, s);
-        launch_update64(d_desc, base, Upd64{3, k0, 0, PW, 0, 0}, max_below, PW, sh.count, *ws64, d_err, s, ws64->pinv);
-      } else {
+      if (narrow) {
+        launch_diag<T>(d_desc, base, k0, sh.count, d_err, store, pinv, s);
+        launch_update<T>(d_desc, base, Upd64{3, k0, 0, PW, 0, 0}, max_below, PW, sh.count, ws, d_err, s, pinv);
+      } else if constexpr (!f64) {
         k_bigpanel<T, false><<<dim3(1, sh.count), 256, bigpanel_smem<T, false>(), s>>>(d_desc, base, k0, d_err, store);
         count_launch();
-        if (max_below > 0 && tc && pinv) {  // L_21 = A_21 L_11^-T as one tensor-core product with the block's inverse
-          k_diag_inverse<<<dim3(1, sh.count), 256, kInvSmem, s>>>(d_desc, base, k0, pinv);
-          count_launch();
-          launch_rankk_tc(d_desc, base, 3, k0, 0, max_below, kPW, sh.count, d_err, s, pinv);
-        } else if (max_below > 0) {
+        if (max_below > 0) {
           k_bigpanel<T, true><<<dim3(ceil_div(max_below, PanelRows<T>::RB), sh.count), 256, bigpanel_smem<T, true>(),
                                 s>>>(d_desc, base, k0, d_err, store);
           count_launch();
@@ -561,10 +486,9 @@ void engine_partial_cholesky(const EngineShape &sh, const MatDesc *d_desc, T *ba
       if (max_below > 0 && max_cols > 0) {
         if (prof) prof->begin(PROF_PANEL, s);
         if constexpr (f64) {
-          launch_update64(d_desc, base, Upd64{0, k0, K1, PW, 0, 0}, max_below, max_cols, sh.count, *ws64, d_err, s);
+          launch_update<T>(d_desc, base, Upd64{0, k0, K1, PW, 0, 0}, max_below, max_cols, sh.count, ws, d_err, s);
         } else {
-          static_assert(kPW == 128, "the tensor-core in-block update takes 128-column panels");
-          if (tc) launch_rankk_tc(d_desc, base, 0, k0, K1, max_below, max_cols, sh.count, d_err, s);
+          if (tc) launch_update<T>(d_desc, base, Upd64{0, k0, K1, PW, 0, 0}, max_below, max_cols, sh.count, ws, d_err, s);
           else launch_rankk(d_desc, base, 0, k0, K0, K1, max_below, max_cols, sh.count, s);
         }
         if (prof) prof->end(PROF_PANEL, s, fl_in, 0.0);
@@ -584,11 +508,11 @@ void engine_partial_cholesky(const EngineShape &sh, const MatDesc *d_desc, T *ba
     }
     if (max_rows > 0 && max_cols > 0) {
       if (prof) prof->begin(PROF_RANKK, s);
-      if constexpr (std::is_same<T, float>::value) {
-        if (tc) launch_rankk_tc(d_desc, base, 2, K0, K1, max_rows, max_cols, sh.count, d_err, s);
-        else launch_rankk(d_desc, base, 2, 0, K0, K1, max_rows, max_cols, sh.count, s);
+      if constexpr (f64) {
+        launch_update<T>(d_desc, base, Upd64{2, K0, K1, PW, K0, K1}, max_rows, max_cols, sh.count, ws, d_err, s);
       } else {
-        launch_update64(d_desc, base, Upd64{2, K0, K1, PW, K0, K1}, max_rows, max_cols, sh.count, *ws64, d_err, s);
+        if (tc) launch_update<T>(d_desc, base, Upd64{2, K0, K1, PW, K0, K1}, max_rows, max_cols, sh.count, ws, d_err, s);
+        else launch_rankk(d_desc, base, 2, 0, K0, K1, max_rows, max_cols, sh.count, s);
       }
       if (prof) prof->end(PROF_RANKK, s, fl, by);
     }
@@ -613,11 +537,11 @@ void engine_partial_cholesky(const EngineShape &sh, const MatDesc *d_desc, T *ba
   }
   if (max_t > 0) {
     if (prof) prof->begin(PROF_RANKK, s);
-    if constexpr (std::is_same<T, float>::value) {
-      if (tc) launch_rankk_tc(d_desc, base, 1, 0, 0, max_t, max_t, sh.count, d_err, s);
-      else launch_rankk(d_desc, base, 1, 0, 0, 0, max_t, max_t, sh.count, s);
+    if constexpr (f64) {
+      launch_update<T>(d_desc, base, Upd64{1, 0, 0, PW, 0, sh.max_e}, max_t, max_t, sh.count, ws, d_err, s);
     } else {
-      launch_update64(d_desc, base, Upd64{1, 0, 0, PW, 0, sh.max_e}, max_t, max_t, sh.count, *ws64, d_err, s);
+      if (tc) launch_update<T>(d_desc, base, Upd64{1, 0, 0, PW, 0, sh.max_e}, max_t, max_t, sh.count, ws, d_err, s);
+      else launch_rankk(d_desc, base, 1, 0, 0, 0, max_t, max_t, sh.count, s);
     }
     if (prof) prof->end(PROF_RANKK, s, fl, by);
   }
@@ -1236,8 +1160,6 @@ size_t dense_smem_limit() { return 200 * 1024; }
 bool dense_configure() {
   const int lim = (int)dense_smem_limit();
   bool ok = true;
-  ok &= cudaFuncSetAttribute(k_diag_inverse, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kInvSmem) ==
-        cudaSuccess;
   ok &= cudaFuncSetAttribute(k_bigpanel<float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)bigpanel_smem<float, false>()) == cudaSuccess;
   ok &= cudaFuncSetAttribute(k_bigpanel<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1262,7 +1184,7 @@ bool dense_configure() {
 
 #define BD_INST(T)                                                                                              \
   template void engine_partial_cholesky<T>(const EngineShape &, const MatDesc *, T *, int *, cudaStream_t,    \
-                                           T *, ProfHook *, bool, float *, const Slice64 *);                                    \
+                                           T *, ProfHook *, int, const SliceWs &);                                              \
   template void launch_gemv<T>(int, int, int, const GemvDesc *, const T *, const double *, const int *,        \
                                double *, double, const int *, cudaStream_t);                                   \
   template void launch_symv_rows<T>(int, const T *, int, const double *, double *, int, const int *,           \

@@ -72,16 +72,16 @@ void launch_dot3(int n, const double *a0, const double *b0, const double *a1, co
 void launch_gauge_shift(int n, double *ui, double *ue, const double *scal, cudaStream_t s);
 void launch_sum_partials(int nblk, const double *partial, double *out, cudaStream_t s);
 
-// tc64.cu -- FP64 rank-k updates and panel solves on the tensor cores (exact digit products).
-constexpr int kPanel64 = 64;   // panel width of the FP64 engine
+// digits.cu -- rank-k updates and panel solves on the tensor cores by exact digit products.
+constexpr int kPanel64 = 64;   // panel width where the panels too are solved that way
 constexpr int kSliceK = 1024;  // columns whose digit planes the workspace holds at a time
-struct Upd64 {                 // one update over a batch (modes as in tc64.cu)
+struct Upd64 {                 // one update over a batch (modes as in digits.cu); pw: panel width
   int mode, K0, K1, pw, ka, kz;
 };
-struct Slice64 {               // workspace: digit planes, row exponents; pinv: a panel inverse per matrix
+struct SliceWs {               // workspace: digit planes and row exponents; a panel inverse per matrix
   unsigned char *mem = nullptr;
   size_t bytes = 0;
-  double *pinv = nullptr;
+  void *pinv = nullptr;
 };
 
 // dense.cu -- batched partial Cholesky: eliminates the first e columns of every
@@ -101,31 +101,26 @@ struct EngineShape {
 // one long-K (K = ob) update of the trailing columns.  store: block store
 // receiving the factored kNB x kNB diagonal blocks L_kk; matrix b uses slots
 // [desc[b].dblk, desc[b].dblk + ceil(e_b / kNB)) (row-major, identity outside the last
-// block's width).  tc: FP32 only, run the long-K updates on the tensor cores (tc.cu).
+// block's width).  tc: 0 SIMT (FP32 only), 1 the updates on the tensor cores (digits.cu), 2 also the
+// panels, 64 columns wide (always in FP64).
 constexpr int kEnginePanel = 128;
-// pinv (FP32 with tc only): 128 x 128 floats per matrix of scratch; with it, the rows below
-// every panel are solved as one tensor-core product with the inverse of the diagonal block.
 template <typename T>
 void engine_partial_cholesky(const EngineShape &sh, const MatDesc *d_desc, T *base, int *d_err, cudaStream_t s,
-                             T *store, ProfHook *prof = nullptr, bool tc = false, float *pinv = nullptr,
-                             const Slice64 *ws64 = nullptr);
+                             T *store, ProfHook *prof, int tc, const SliceWs &ws);
 
 bool dense_configure();
 size_t dense_smem_limit();  // bytes of shared memory the dense kernels may stage per CTA
 
-// tc64.cu
-bool tc64_configure();
+// digits.cu
+bool digits_configure();
 // workspace of `count` matrices of max_rows rows and max_e eliminated columns at once
-size_t slice64_bytes(int count, int max_rows, int max_e);
-void launch_update64(const MatDesc *d_desc, double *base, Upd64 u, int max_rows, int max_cols, int count,
-                     const Slice64 &ws, int *err, cudaStream_t s, const double *pinv = nullptr);
-void launch_diag64(const MatDesc *d_desc, double *base, int K0, int count, int *err, double *store, double *pinv,
-                   cudaStream_t s);
-
-// tc.cu
-bool tc_configure();
-void launch_rankk_tc(const MatDesc *d_desc, float *base, int mode, int K0, int K1, int max_rows, int max_cols,
-                     int count, int *err, cudaStream_t s, const float *pinv = nullptr);
+template <typename T>
+size_t slice_bytes(int count, int max_rows, int max_e);
+template <typename T>
+void launch_update(const MatDesc *d_desc, T *base, Upd64 u, int max_rows, int max_cols, int count, const SliceWs &ws,
+                   int *err, cudaStream_t s, const T *pinv = nullptr);
+template <typename T>
+void launch_diag(const MatDesc *d_desc, T *base, int K0, int count, int *err, T *store, T *pinv, cudaStream_t s);
 
 // The same products for many small matrices: one CTA per task over all its rows (columns)
 template <typename T>
