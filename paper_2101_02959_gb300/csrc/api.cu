@@ -527,7 +527,7 @@ void setup_handle(bd_handle &h) {
     *v = m.alloc<double>(N);
     ck(cudaMemsetAsync(*v, 0, sizeof(double) * N, s), "memset");
   }
-  h.d_partial = m.alloc<double>(3 * kRedBlocks);
+  h.d_partial = m.alloc<double>(3 * std::max(kRedBlocks, kResBlocks));
   h.d_scal = m.alloc<double>(64);
   h.d_err = m.alloc<int>(1);
   ck(cudaMemsetAsync(h.d_err, 0, sizeof(int), s), "memset");
@@ -1453,7 +1453,7 @@ int solve(bd_handle &h, const double *fi, const double *fe, double *si, double *
 
 StimParams stim_params(const bd_handle &h, const bd_stimulus *st, double t_next) {
   StimParams sp{};
-  for (int d = 0; d < 3; ++d) { sp.h[d] = h.plan.h[d]; sp.o[d] = h.plan.origin[d]; }
+  for (int d = 0; d < 3; ++d) { sp.h[d] = h.plan.h[d]; sp.o[d] = h.plan.origin[d]; sp.n[d] = h.plan.n[d]; }
   if (st) {
     sp.amp = st->amp;
     for (int k = 0; k < 6; ++k) sp.box[k] = st->box[k];

@@ -1,4 +1,6 @@
 // Q1 assembly, gating, residual and reductions (Sections 2, 3a, 3b).
+#include <algorithm>
+
 #include "kernels.cuh"
 
 namespace bd {
@@ -254,14 +256,12 @@ __global__ void k_stencil_gather(int nrows, const int *__restrict__ row_node, co
 // ---------------------------------------------------------------------------
 // Rogers-McCulloch model (Section 2) and Step 1 (Section 3b).
 // ---------------------------------------------------------------------------
-__device__ inline double rmc_iion(double v, double w, const FemParams &p) {
-  return p.G * v * (1.0 - v / p.vth) * (1.0 - v / p.vp) + p.eta1 * v * w;
-}
-__device__ inline double rmc_diion(double v, double w, const FemParams &p) {
-  // derivative of G v (1 - v a)(1 - v b) + eta1 v w with a = 1/vth, b = 1/vp
-  const double a = 1.0 / p.vth, b = 1.0 / p.vp;
-  return p.G * (1.0 - 2.0 * (a + b) * v + 3.0 * a * b * v * v) + p.eta1 * w;
-}
+// The residual's parameters: reciprocals 1 / vth, 1 / vp, the derivative's coefficients, and the
+// stimulus box as node index ranges.
+struct ResParams {
+  double G, eta1, a, b, chi_cm, tau, g1, g2, amp;
+  int active, lo[3], hi[3];
+};
 
 __global__ void k_gating(int n, const double *__restrict__ ui, const double *__restrict__ ue,
                          const double *__restrict__ w, double *__restrict__ wn, FemParams p) {
@@ -272,54 +272,74 @@ __global__ void k_gating(int n, const double *__restrict__ ui, const double *__r
   wn[x] = (w[x] + te * v / p.vp) / (1.0 + te);
 }
 
+// u + lam s, both media (line-search trial point).
+__global__ void k_trial(int n, const double *__restrict__ ui0, const double *__restrict__ ue0,
+                        const double *__restrict__ si, const double *__restrict__ se, double lam,
+                        double *__restrict__ ui, double *__restrict__ ue) {
+  const int x = blockIdx.x * blockDim.x + threadIdx.x;
+  if (x >= n) return;
+  ui[x] = ui0[x] + lam * si[x];
+  ue[x] = ue0[x] + lam * se[x];
+}
+
 // F(u) - G (Step 2) with the Jacobian factor chi Cm + tau dI/dv, and per-block
-// partial sums of ||F - G||^2.  u = x + lam * s when s != nullptr (line search).
-__global__ void k_residual(int n, const double *__restrict__ stencil, const int *__restrict__ nbr,
-                           const double *__restrict__ mass, const int *__restrict__ node_ijk,
-                           const double *__restrict__ ui0, const double *__restrict__ ue0,
-                           const double *__restrict__ si, const double *__restrict__ se, double lam,
-                           const double *__restrict__ wn, const double *__restrict__ uin,
-                           const double *__restrict__ uen, FemParams p, StimParams st,
-                           double *__restrict__ ri, double *__restrict__ re, double *__restrict__ factor,
-                           double *__restrict__ ui_out, double *__restrict__ ue_out, double *__restrict__ partial) {
+// partial sums of ||F - G||^2.  One node per thread; the stencil's 27 slots in three batches of nine,
+// all loads of a batch in flight (a missing neighbour reads the node itself against its zero
+// coefficient).  Bound by FP64 instructions (64 clocks each per warp and scheduler: 54 stencil
+// multiply-adds and about 25 others) and HBM (656 bytes a node): 549,153 nodes take 120 us, 235 us
+// with divisions by the ionic parameters in the kernel, the trial point formed at every neighbour
+// and a grid that held a few loads in flight.
+__global__ void __launch_bounds__(256, 3) k_residual(
+    int n, const double *__restrict__ stencil, const int *__restrict__ nbr, const double *__restrict__ mass,
+    const int *__restrict__ node_ijk, const double *__restrict__ ui, const double *__restrict__ ue,
+    const double *__restrict__ wn, const double *__restrict__ uin, const double *__restrict__ uen, ResParams p,
+    double *__restrict__ ri, double *__restrict__ re, double *__restrict__ factor, double *__restrict__ ui_out,
+    double *__restrict__ ue_out, double *__restrict__ partial) {
   __shared__ double sh[32];
   double acc = 0.0;
   for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < n; x += gridDim.x * blockDim.x) {
-    double Au_i = 0.0, Au_e = 0.0;
-#pragma unroll 3
-    for (int sl = 0; sl < 27; ++sl) {
-      const int y = nbr[(long long)sl * n + x];
-      if (y < 0) continue;
-      double yi = ui0[y], ye = ue0[y];
-      if (si) { yi += lam * si[y]; ye += lam * se[y]; }
-      Au_i += stencil[(long long)sl * n + x] * yi;
-      Au_e += stencil[(long long)(27 + sl) * n + x] * ye;
+    double Ai = 0.0, Ae = 0.0;
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      int y[9];
+      double ci[9], ce[9], vi[9], ve[9];
+#pragma unroll
+      for (int q = 0; q < 9; ++q) {
+        y[q] = nbr[(long long)(9 * b + q) * n + x];
+        ci[q] = stencil[(long long)(9 * b + q) * n + x];
+        ce[q] = stencil[(long long)(27 + 9 * b + q) * n + x];
+      }
+#pragma unroll
+      for (int q = 0; q < 9; ++q) {
+        const int z = y[q] < 0 ? x : y[q];
+        vi[q] = ui[z];
+        ve[q] = ue[z];
+      }
+#pragma unroll
+      for (int q = 0; q < 9; ++q) {
+        Ai += ci[q] * vi[q];
+        Ae += ce[q] * ve[q];
+      }
     }
-    double xi = ui0[x], xe = ue0[x];
-    if (si) { xi += lam * si[x]; xe += lam * se[x]; }
+    const double xi = ui[x], xe = ue[x], w = wn[x], M = mass[x];
     const double v = xi - xe, vn = uin[x] - uen[x];
-    const double M = mass[x];
-    const double cap = p.chi_cm * M * (v - vn);
-    const double ion = p.tau * M * rmc_iion(v, wn[x], p);
-    double app = 0.0;
-    if (st.active) {
-      const double cx = st.o[0] + node_ijk[3 * x] * st.h[0], cy = st.o[1] + node_ijk[3 * x + 1] * st.h[1],
-                   cz = st.o[2] + node_ijk[3 * x + 2] * st.h[2];
-      const double eps = 1e-12;
-      if (cx >= st.box[0] - eps && cx <= st.box[1] + eps && cy >= st.box[2] - eps && cy <= st.box[3] + eps &&
-          cz >= st.box[4] - eps && cz <= st.box[5] + eps)
-        app = p.tau * M * st.amp;
-    }
-    const double a = cap + p.tau * Au_i + ion - app;
-    const double b = -cap + p.tau * Au_e - ion + app;
+    // ion = tau M (G v (1 - v / vth)(1 - v / vp) + eta1 v w) - tau M I_app
+    double ion = v * (p.G * fma(-v, p.a, 1.0) * fma(-v, p.b, 1.0) + p.eta1 * w);
+    if (p.active && node_ijk[3 * x] >= p.lo[0] && node_ijk[3 * x] <= p.hi[0] && node_ijk[3 * x + 1] >= p.lo[1] &&
+        node_ijk[3 * x + 1] <= p.hi[1] && node_ijk[3 * x + 2] >= p.lo[2] && node_ijk[3 * x + 2] <= p.hi[2])
+      ion -= p.amp;
+    const double q = M * fma(p.tau, ion, p.chi_cm * (v - vn));
+    const double a = fma(p.tau, Ai, q), c = fma(p.tau, Ae, -q);
     ri[x] = a;
-    re[x] = b;
-    if (factor) factor[x] = p.chi_cm + p.tau * rmc_diion(v, wn[x], p);
+    re[x] = c;
+    // d/dv (G v (1 - a v)(1 - b v) + eta1 v w) = G + v (2 g1 + 3 g2 v) + eta1 w
+    if (factor) factor[x] = fma(p.tau, fma(v, fma(v, p.g2, p.g1), p.G) + p.eta1 * w, p.chi_cm);
     if (ui_out) { ui_out[x] = xi; ue_out[x] = xe; }
-    acc += a * a + b * b;
+    acc += a * a + c * c;
   }
+  if (!partial) return;
   acc = block_sum(acc, sh);
-  if (threadIdx.x == 0 && partial) partial[blockIdx.x] = acc;
+  if (threadIdx.x == 0) partial[blockIdx.x] = acc;
 }
 
 // Partial sums of up to three dot products over the same index range.
@@ -398,16 +418,41 @@ void launch_gating(int n, const double *ui, const double *ue, const double *w, d
   count_launch();
 }
 
+// The node indices i with box[0] - eps <= o + i h <= box[1] + eps, as a range (empty: lo > hi).
+static void stim_range(double o, double h, double b0, double b1, int n, int &lo, int &hi) {
+  const double eps = 1e-12;
+  lo = 0;
+  hi = n;
+  while (lo <= n && !(o + lo * h >= b0 - eps)) ++lo;
+  while (hi >= 0 && !(o + hi * h <= b1 + eps)) --hi;
+}
+
 void launch_residual(int n, const double *stencil, const int *nbr, const double *mass, const int *node_ijk,
                      const double *ui0, const double *ue0, const double *si, const double *se, double lam,
                      const double *wn, const double *uin, const double *uen, const FemParams &p,
                      const StimParams &st, double *ri, double *re, double *factor, double *ui_out,
                      double *ue_out, double *partial, double *norm2, cudaStream_t s) {
-  k_residual<<<kRedBlocks, 256, 0, s>>>(n, stencil, nbr, mass, node_ijk, ui0, ue0, si, se, lam, wn, uin, uen, p, st,
-                                        ri, re, factor, ui_out, ue_out, partial);
+  if (si) {  // the trial point is an output too: form it once, then evaluate there
+    k_trial<<<ceil_div(n, 256), 256, 0, s>>>(n, ui0, ue0, si, se, lam, ui_out, ue_out);
+    count_launch();
+    ui0 = ui_out;
+    ue0 = ue_out;
+    ui_out = ue_out = nullptr;
+  }
+  ResParams r{};
+  r.G = p.G; r.eta1 = p.eta1; r.a = 1.0 / p.vth; r.b = 1.0 / p.vp; r.chi_cm = p.chi_cm; r.tau = p.tau;
+  r.g1 = -2.0 * p.G * (r.a + r.b);
+  r.g2 = 3.0 * p.G * r.a * r.b;
+  r.active = st.active;
+  r.amp = st.amp;
+  if (st.active)
+    for (int d = 0; d < 3; ++d) stim_range(st.o[d], st.h[d], st.box[2 * d], st.box[2 * d + 1], st.n[d], r.lo[d], r.hi[d]);
+  const int blocks = std::max(1, std::min(ceil_div(n, 256), kResBlocks));
+  k_residual<<<blocks, 256, 0, s>>>(n, stencil, nbr, mass, node_ijk, ui0, ue0, wn, uin, uen, r, ri, re, factor, ui_out,
+                                    ue_out, norm2 ? partial : nullptr);
   count_launch();
   if (norm2) {
-    k_finalize<<<1, 256, 0, s>>>(kRedBlocks, 1, partial, norm2);
+    k_finalize<<<1, 256, 0, s>>>(blocks, 1, partial, norm2);
     count_launch();
   }
 }

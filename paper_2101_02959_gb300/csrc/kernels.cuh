@@ -7,6 +7,7 @@
 namespace bd {
 
 constexpr int kRedBlocks = 304;  // fixed reduction grid (2 x 152 SMs): deterministic sums
+constexpr int kResBlocks = 456;  // most blocks of the residual (3 per SM): its partial sums
 constexpr int kNB = 32;          // panel width of the partial Cholesky
 
 // Per-launch timing hook (CUDA events recorded on the launch stream) and
@@ -37,6 +38,7 @@ struct StimParams {
   double box[6];
   double h[3];
   double o[3];  // grid origin in the parametric coordinates
+  int n[3];     // elements per direction
 };
 
 // Element geometry: kind 0 = box (spacing h, slab depth lz), 1 = truncated
