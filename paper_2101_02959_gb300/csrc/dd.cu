@@ -256,32 +256,57 @@ void coarse_refine64(int np, const T *x0, int ld0, const double *C, double *X, d
   count_launch(5);
 }
 
-// The whole coarse solve of a small coarse problem in one CTA: c (as k_coarse_rhs),
+// The whole coarse solve of a small coarse problem in one launch: c (as k_coarse_rhs),
 // z = X c with the FP64 explicit inverse X, then nref steps of iterative refinement
 // z += X (c - S_PP z) with the FP64 sparse S_PP.  The refinement makes the solve
 // backward stable (the explicit inverse alone is not: its error grows with cond(S_PP)
 // times the size of X, and the (u_i, u_e) constant mode that the gauge alone holds is
 // where it shows).
-__global__ void __launch_bounds__(1024) k_coarse_solve_small(
+//
+// One cluster of eight CTAs, each with an eighth of the rows, one warp per row; every CTA keeps whole
+// copies of the vectors, which the owners write into all of them.  On one SM the products are bound by
+// its FP64 rate (2 multiply-adds a clock: 35 us for np = 270); spread over eight SMs the launch takes
+// COARSE_AFTER.
+constexpr int kCoCta = 8;
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// v into entry i of the double array at shared address `addr`, in every CTA of the cluster (lanes < 8)
+__device__ __forceinline__ void cluster_store(uint32_t addr, int i, double v, int lane) {
+  if (lane < kCoCta) {
+    uint32_t remote;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(addr + 8 * i), "r"(lane));
+    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(remote), "d"(v) : "memory");
+  }
+}
+
+__global__ void __cluster_dims__(kCoCta, 1, 1) __launch_bounds__(1024) k_coarse_solve_small(
     int np, int gauge, const int *__restrict__ pl_ptr, const int *__restrict__ pl_idx,
     const double *__restrict__ yprim, const double *__restrict__ rP, const CsrIn rPc, const double *__restrict__ X,
     const int *__restrict__ sptr, const int *__restrict__ scol, const double *__restrict__ sval, int nref,
     double *__restrict__ z_out, const int *__restrict__ done) {
-  if (done && *done) return;
+  if (done && *done) return;  // the same in every CTA of the cluster
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  double *c = reinterpret_cast<double *>(smem_raw);
-  double *z = c + np;
-  double *r = z + np;
-  for (int q = threadIdx.x; q < np; q += blockDim.x) {
-    c[q] = coarse_rhs_row(q, gauge, pl_ptr, pl_idx, yprim, rP, rPc);
-    r[q] = c[q];
-    z[q] = 0.0;
-  }
-  __syncthreads();
+  double *c = reinterpret_cast<double *>(smem_raw), *z = c + np, *r = z + np;
+  const uint32_t zs = (uint32_t)__cvta_generic_to_shared(z), rs = (uint32_t)__cvta_generic_to_shared(r);
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int q0 = (int)((long long)np * blockIdx.x / kCoCta), q1 = (int)((long long)np * (blockIdx.x + 1) / kCoCta);
+  for (int q = threadIdx.x; q < np; q += blockDim.x) z[q] = 0.0;
+  cluster_sync();  // every CTA runs and has cleared its copy
+  for (int q = q0 + wid; q < q1; q += nw) {  // right-hand side: c of the own rows, r = c everywhere
+    double acc = 0.0;
+    for (int k = pl_ptr[q] + lane; k < pl_ptr[q + 1]; k += 32) acc -= yprim[pl_idx[k]];
+    if (!rP && rPc.ptr)
+      for (int k = rPc.ptr[q] + lane; k < rPc.ptr[q + 1]; k += 32) acc += rPc.val[k] * rPc.v[rPc.col[k]];
+    acc = warp_sum(acc);
+    if (rP) acc += rP[q];
+    if (q == gauge) acc = 0.0;
+    if (lane == 0) c[q] = acc;
+    cluster_store(rs, q, acc, lane);
+  }
+  cluster_sync();
   for (int pass = 0; pass <= nref; ++pass) {
-    // z += X r (r = c on the first pass)
-    for (int q = wid; q < np; q += nw) {
+    for (int q = q0 + wid; q < q1; q += nw) {  // z += X r (r = c on the first pass)
       const double *row = X + (long long)q * np;
       double a0 = 0.0, a1 = 0.0;
       int k = lane;
@@ -290,19 +315,24 @@ __global__ void __launch_bounds__(1024) k_coarse_solve_small(
         a1 += row[k + 32] * r[k + 32];
       }
       if (k < np) a0 += row[k] * r[k];
-      const double v = warp_sum(a0 + a1);
-      if (lane == 0) z[q] += v;
+      const double v = warp_sum(a0 + a1) + z[q];
+      if (pass == nref) {
+        if (lane == 0) z_out[q] = v;
+      } else {
+        __syncwarp();  // every lane has read the old z[q]
+        cluster_store(zs, q, v, lane);
+      }
     }
-    __syncthreads();
     if (pass == nref) break;
-    for (int q = threadIdx.x; q < np; q += blockDim.x) {
+    cluster_sync();
+    for (int q = q0 + wid; q < q1; q += nw) {
       double acc = 0.0;
-      for (int k = sptr[q]; k < sptr[q + 1]; ++k) acc += sval[k] * z[scol[k]];
-      r[q] = c[q] - acc;
+      for (int k = sptr[q] + lane; k < sptr[q + 1]; k += 32) acc += sval[k] * z[scol[k]];
+      acc = c[q] - warp_sum(acc);
+      cluster_store(rs, q, acc, lane);
     }
-    __syncthreads();
+    cluster_sync();
   }
-  for (int q = threadIdx.x; q < np; q += blockDim.x) z_out[q] = z[q];
 }
 
 // ---- rho-scaling (Section 4.2) --------------------------------------------------
@@ -793,7 +823,7 @@ void launch_coarse_solve(const CoarseSolve &cs, const T *X, const double *yprim,
   if (cs.np == 0) return;
   const CsrIn rc = rPc ? *rPc : CsrIn{};
   if (cs.X64) {
-    k_coarse_solve_small<<<1, 1024, 3 * sizeof(double) * cs.np, s>>>(
+    k_coarse_solve_small<<<kCoCta, 1024, 3 * sizeof(double) * cs.np, s>>>(
         cs.np, cs.gauge, cs.pl_ptr, cs.pl_idx, yprim, rP, rc, cs.X64, cs.sptr, cs.scol, cs.sval, cs.nref, z, done);
     count_launch();
     return;
