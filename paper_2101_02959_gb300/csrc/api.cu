@@ -1359,6 +1359,13 @@ int gmres(bd_handle &h, int n, const double *b, double *x, Op A, Pc M, bd_solve_
       A(h.d_gV + (long long)j * n, h.d_gt, stop);
       M(h.d_gt, h.d_gz, stop);
       launch_gmres_step(n, j, h.d_gV, h.d_gz, h.d_gpart, h1, h2, zz, h.d_gs, s);
+      // launches past the stop return at once but still cost their launch time: look every kChunk steps
+      if (j % kChunk == kChunk - 1 && j + 1 < m) {
+        int stopped = 0;
+        ck(cudaMemcpyAsync(&stopped, stop, sizeof(int), cudaMemcpyDeviceToHost, s), "gmres stop");
+        ck(cudaStreamSynchronize(s), "gmres sync");
+        if (stopped) break;
+      }
     }
     launch_gmres_end(n, h.d_gV, x, h.d_gs, s);
     ck(cudaGetLastError(), "gmres launch");
