@@ -87,16 +87,30 @@ static inline long long sym_tile_entries(int n) {
 }
 struct SymvSet {  // batched symmetric GEMV tasks; n = 0 when their shared memory does not fit
   SymvTask *d = nullptr;
-  int n = 0, max_n = 0;
-  int split = 1, ld_scr = 0;  // CTAs per task; partial-sum rows (split > 1)
-  void *scratch = nullptr;    // n x split x ld_scr values of the local precision
-  int *counter = nullptr;     // n zeroed ints
+  int n = 0, max_n = 0;       // CTAs; largest order
+  int ld_scr = 0;             // row stride of the partial sums of split matrices
+  void *scratch = nullptr;    // their rows, in the local precision
+  int *counter = nullptr;     // a zeroed int per split matrix
+  // FP64: the matrices' lower tiles in fixed point, packed from the FP64 matrices once per Jacobian
+  FixTask *fix = nullptr;
+  int nfix = 0;
+  int2 *tiles = nullptr;
+  int *ex = nullptr;
 };
-template <class T>
-void launch_symv(const SymvSet &g, const T *A, const double *x, const int *xidx, double *y, const int *done,
+void launch_symv(const SymvSet &g, const float *A, const double *x, const int *xidx, double *y, const int *done,
                  cudaStream_t s) {
-  launch_symv_batched<T>(g.n, g.max_n, g.split, g.d, A, x, xidx, y, 1.0, done, static_cast<T *>(g.scratch),
-                         g.counter, g.ld_scr, s);
+  launch_symv_batched(g.n, g.max_n, g.d, A, x, xidx, y, 1.0, done, static_cast<float *>(g.scratch), g.counter,
+                      g.ld_scr, s);
+}
+void launch_symv(const SymvSet &g, const double *, const double *x, const int *xidx, double *y, const int *done,
+                 cudaStream_t s) {
+  launch_symv_fix(g.n, g.max_n, g.d, g.tiles, g.ex, x, xidx, y, 1.0, done, static_cast<double *>(g.scratch),
+                  g.counter, g.ld_scr, s);
+}
+// the fixed-point tiles of a set from its matrices (FP64 only)
+void pack_symv(const SymvSet &, const float *, cudaStream_t) {}
+void pack_symv(const SymvSet &g, const double *A, cudaStream_t s) {
+  launch_fix_tiles(g.nfix, g.max_n, g.fix, A, g.tiles, g.ex, s);
 }
 struct CopySet {
   CopyTask *d = nullptr;
@@ -274,7 +288,7 @@ struct bd_handle {
   GemvSet gv_psi;  // Psi^T r_Delta alone (the coarse right-hand side's local parts)
   // the operator S_Gamma and the local solve [X; Psi^T] as symmetric products (X, S_Gamma
   // symmetric: each lower tile read once); used instead of gv_schur / gv_local when set
-  SymvSet sv_schur, sv_local;
+  SymvSet sv_schur, sv_local, sv_sdd;  // sv_sdd: the FETI-DP preconditioner's S_DeltaDelta
   // tensor-core factorisation: digit planes of the updates, inverses of the panels' diagonal blocks
   SliceWs ws;
   GemmTask *d_gemm = nullptr;
@@ -905,13 +919,14 @@ void setup_handle(bd_handle &h) {
     return c;
   };
   std::vector<GemvDesc> g_schur, g_local, g_psit, g_sdd, g_lgi, g_lgit;
-  std::vector<SymvTask> s_schur, s_local;
+  std::vector<SymvTask> s_schur, s_local, s_sdd;
   std::vector<GemvDesc> g_psi;
   std::vector<CopyTask> c_sorig, c_sdd, c_zx;
   for (int j = 0; j < S; ++j) {
     const int ng = h.nG[j], ni = h.nI[j], nd = h.nD[j], npj = h.nP[j];
     g_schur.push_back(GemvDesc{so_off[j], ldg[j], ng, ng, h.giff_off[j], h.giff_off[j], 1});
     s_schur.push_back(SymvTask{so_off[j], 0, ldg[j], ng, 0, h.giff_off[j], h.giff_off[j], 0, 1});
+    s_sdd.push_back(SymvTask{sdd_off[j], 0, ldx[j], nd, 0, h.ldual_off[j], h.ldual_off[j], 0, 0});
     s_local.push_back(SymvTask{zx_off[j], 0, ldx[j], nd, 0, h.ldual_off[j], h.ldual_off[j], 0, 0});
     g_psi.push_back(GemvDesc{zp_off[j], ldx[j], npj, nd, h.ldual_off[j], h.nD_tot + h.lprim_off[j], 0});
     g_local.push_back(GemvDesc{zx_off[j], ldx[j], nd, nd, h.ldual_off[j], h.ldual_off[j], 0});
@@ -947,26 +962,41 @@ void setup_handle(bd_handle &h) {
     const size_t el = h.mixed() ? sizeof(float) : sizeof(double);
     int sms = 0;
     ck(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h.device), "SM count");
-    auto sset = [&](const std::vector<SymvTask> &v) {
+    auto sset = [&](const std::vector<SymvTask> &in) {
       SymvSet g;
-      for (auto &t : v) g.max_n = std::max(g.max_n, t.n);
+      for (auto &t : in) g.max_n = std::max(g.max_n, t.n);
       const size_t np = (size_t)ceil_div(g.max_n, 32) * 32;
-      if (el * (9 * np + 8 * 32 * 33) > dense_smem_limit()) return SymvSet{};  // the full GEMV then
-      g.n = (int)v.size();
-      g.d = m.upload(v, s);
-      // split every matrix over enough CTAs to fill the resident slots evenly
-      const int occ = h.mixed() ? symv_occupancy<float>(g.max_n) : symv_occupancy<double>(g.max_n);
-      g.split = symv_split(g.n, g.max_n, sms * occ);
-      if (g.split > 1) {
-        g.ld_scr = (int)np;
-        g.scratch = m.alloc<unsigned char>(el * (size_t)g.n * g.split * g.ld_scr);
-        g.counter = m.alloc<int>(g.n);
-        ck(cudaMemsetAsync(g.counter, 0, sizeof(int) * g.n, s), "memset counters");
+      if ((h.mixed() ? symv_smem<float>(g.max_n) : symv_smem<double>(g.max_n)) > dense_smem_limit())
+        return SymvSet{};  // the full GEMV then
+      std::vector<SymvTask> v = in;
+      if (!h.mixed()) {
+        std::vector<FixTask> fix;
+        long long off = 0;
+        for (SymvTask &t : v) {
+          const long long nb = ceil_div(t.n, 32);
+          t.f_off = off;
+          fix.push_back(FixTask{t.a_off, off, t.ld, t.n});
+          off += nb * (nb + 1) / 2;
+        }
+        g.fix = m.upload(fix, s);
+        g.nfix = (int)fix.size();
+        g.tiles = m.alloc<int2>((size_t)off * 1024);
+        g.ex = m.alloc<int>(off);
       }
+      const int occ = h.mixed() ? symv_occupancy<float>(g.max_n) : symv_occupancy<double>(g.max_n);
+      int rows = 0, ctrs = 0;
+      const std::vector<SymvTask> plan = symv_plan(v, sms * occ, &rows, &ctrs);
+      g.n = (int)plan.size();
+      g.d = m.upload(plan, s);
+      g.ld_scr = (int)np;
+      g.scratch = m.alloc<unsigned char>(el * (size_t)rows * g.ld_scr);
+      g.counter = m.alloc<int>(ctrs);
+      ck(cudaMemsetAsync(g.counter, 0, sizeof(int) * std::max(ctrs, 1), s), "memset counters");
       return g;
     };
     h.sv_schur = sset(s_schur);
     h.sv_local = sset(s_local);
+    h.sv_sdd = sset(s_sdd);
     // bytes read by the products of one application (the profile's library bytes)
     if (h.sv_schur.n) {
       h.gemv_schur_bytes = 0.0;
@@ -1114,6 +1144,7 @@ void linearize_t(bd_handle &h, Dense<T> &D, bool precond) {
                            h.tau, h.d_Kdesc, D.K, s);
   run_engine_groups<T>(h, h.shK, h.d_Kdesc, D.K, D.LdK);
   launch_copy<T, T>(h.cp_sorig.n, h.cp_sorig.max_elems, h.cp_sorig.d, D.K, D.Sorig, s);
+  pack_symv(h.sv_schur, D.Sorig, s);
   if (!precond) return;
   const T *tval;
   if constexpr (std::is_same<T, float>::value) tval = h.d_tl_valf;
@@ -1121,9 +1152,11 @@ void linearize_t(bd_handle &h, Dense<T> &D, bool precond) {
   launch_build_aug<T>(h.nsub, h.shA.max_m, h.d_Sdesc, D.Sorig, h.d_Adesc, D.Aug, h.d_nD, h.d_tl_off, h.d_tl_ptr,
                       h.d_tl_row, tval, s);
   launch_copy<T, T>(h.cp_sdd.n, h.cp_sdd.max_elems, h.cp_sdd.d, D.Aug, D.SDD, s);
+  pack_symv(h.sv_sdd, D.SDD, s);
   launch_copy<T, T>(h.cp_blk.n, h.cp_blk.max_elems, h.cp_blk.d, D.Aug, D.Blk, s);
   run_engine_groups<T>(h, h.shA, h.d_Adesc, D.Aug, D.Linv);
   launch_copy<T, T>(h.cp_zx.n, h.cp_zx.max_elems, h.cp_zx.d, D.Aug, D.Z, s);
+  pack_symv(h.sv_local, D.Z, s);
   launch_class_aug<T>(h.ncls, h.max_nc, h.d_cls, h.d_pairs, D.Blk, h.d_Cdesc, D.CA, s);
   engine_partial_cholesky<T>(h.shC, h.d_Cdesc, D.CA, h.d_err, s, D.Linv, &h.prof, h.tc(), h.ws);
   launch_copy<T, T>(h.cp_sinv.n, h.cp_sinv.max_elems, h.cp_sinv.d, D.CA, D.Sinv, s);
@@ -1169,7 +1202,7 @@ template <class T>
 void schur_t(bd_handle &h, Dense<T> &D, const double *x, double *y, const int *done, const DotFuse *f = nullptr) {
   h.prof.begin(PROF_GEMV, h.s);
   if (h.sv_schur.n)
-    launch_symv<T>(h.sv_schur, D.Sorig, x, h.d_R, h.d_yloc, done, h.s);
+    launch_symv(h.sv_schur, D.Sorig, x, h.d_R, h.d_yloc, done, h.s);
   else
     launch_gemv<T>(h.gv_schur.n, h.gv_schur.max_rows, h.gv_schur.max_cols, h.gv_schur.d, D.Sorig, x, h.d_R,
                    h.d_yloc, 1.0, done, h.s);
@@ -1194,7 +1227,7 @@ void st_inv_t(bd_handle &h, Dense<T> &D, const double *rP, const double *rD, con
     launch_coarse_solve<T>(h.cs, D.CoInv, h.d_ydc + h.nD_tot, rP_csr ? nullptr : rP, rP_csr, h.d_zbar + h.nd,
                            h.d_co_c, h.d_co_rho, done, h.s2);
     ck(cudaEventRecord(h.ev_join, h.s2), "record");
-    launch_symv<T>(h.sv_local, D.Z, rD, nullptr, h.d_ydc, done, h.s);
+    launch_symv(h.sv_local, D.Z, rD, nullptr, h.d_ydc, done, h.s);
     h.prof.end(PROF_GEMV, h.s, h.gemv_local_flops, h.gemv_local_bytes * sizeof(T));
     ck(cudaStreamWaitEvent(h.s, h.ev_join, 0), "wait");
   } else {
@@ -1238,8 +1271,11 @@ void feti_F_t(bd_handle &h, Dense<T> &D, const double *lam, double *y, const int
 template <class T>
 void feti_M_t(bd_handle &h, Dense<T> &D, const double *mu, double *y, const int *done) {
   launch_jump_dt<T>(h.nwt, h.max_nc, h.d_wt, h.d_went, D.Blk, D.Sinv, mu, h.d_w1, done, h.s);
-  launch_gemv<T>(h.gv_sdd.n, h.gv_sdd.max_rows, h.gv_sdd.max_cols, h.gv_sdd.d, D.SDD, h.d_w1, nullptr, h.d_w2, 1.0,
-                 done, h.s);
+  if (h.sv_sdd.n)
+    launch_symv(h.sv_sdd, D.SDD, h.d_w1, nullptr, h.d_w2, done, h.s);
+  else
+    launch_gemv<T>(h.gv_sdd.n, h.gv_sdd.max_rows, h.gv_sdd.max_cols, h.gv_sdd.d, D.SDD, h.d_w1, nullptr, h.d_w2, 1.0,
+                   done, h.s);
   launch_jump_d<T>(h.nlt, h.max_nc, h.d_lt, h.d_pairs, D.Blk, D.Sinv, h.d_w2, y, done, h.s);
 }
 
@@ -1711,7 +1747,7 @@ int noalloc_scratch(int dev, double **out) {
 template <class T>
 void schur_noalloc_t(bd_handle &h, Dense<T> &D, const double *x, double *y, double *scratch) {
   if (h.sv_schur.n)
-    launch_symv<T>(h.sv_schur, D.Sorig, x, h.d_R, scratch, nullptr, h.s);
+    launch_symv(h.sv_schur, D.Sorig, x, h.d_R, scratch, nullptr, h.s);
   else
     launch_gemv<T>(h.gv_schur.n, h.gv_schur.max_rows, h.gv_schur.max_cols, h.gv_schur.d, D.Sorig, x, h.d_R,
                    scratch, 1.0, nullptr, h.s);

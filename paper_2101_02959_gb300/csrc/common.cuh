@@ -107,9 +107,18 @@ __host__ __device__ inline BandRows band_rows(const MatDesc &d, int row0, int ke
 // Batched symmetric GEMV task: y = alpha A x for a symmetric n x n matrix stored in full
 // (row-major, ld a multiple of 8, 16-byte aligned), plus optional plain rows yb = alpha B x
 // (B: nb x n at b_off, same ld).  flags bit0: x gathered through xidx; bit1: accumulate.
+// One CTA takes part `part` of `nparts` of the matrix's tiles; with nparts > 1 the parts' sums
+// meet in scratch rows scr .. scr + nparts - 1 and counter ctr.
 struct SymvTask {
   long long a_off, b_off;
   int ld, n, nb, x_off, y_off, yb_off, flags;
+  int part = 0, nparts = 1, scr = 0, ctr = 0;
+  long long f_off = 0;  // FP64: first packed tile
+};
+// A symmetric matrix to be packed as fixed-point tiles (its lower block triangle).
+struct FixTask {
+  long long a_off, f_off;
+  int ld, n;
 };
 
 // Generic batched GEMV task: y[y_idx?] = alpha * op(A) x + beta * y.

@@ -596,7 +596,7 @@ __global__ void __launch_bounds__(256) k_gemv(const GemvDesc *__restrict__ tasks
   }
 }
 
-// ---- batched symmetric GEMV: S CTAs (8 warps each) per matrix ---------------
+// ---- batched symmetric GEMV: S = nparts CTAs (8 warps each) per matrix -------
 // The matrix is read as 32 x 32 tiles of its lower block triangle, each once: tile (I, J),
 // J < I, serves both y_I += A_IJ x_J and y_J += A_IJ^T x_I; a diagonal tile serves
 // y_I += A_II x_I.  CTA s of a matrix takes the s-th of S contiguous runs of the row-major
@@ -619,8 +619,8 @@ __global__ void __launch_bounds__(256) k_symv_batched(const SymvTask *__restrict
   constexpr int LPR = 32 / VN;       // lanes per 32-wide tile row
   constexpr int RPI = 32 / LPR;      // tile rows per warp instruction
   constexpr int TPL = 32 / RPI;      // vectors per lane per tile
-  const SymvTask t = tasks[blockIdx.y];
-  const int S = gridDim.x, sidx = blockIdx.x;
+  const SymvTask t = tasks[blockIdx.x];
+  const int S = t.nparts, sidx = t.part;
   const int n = t.n, nb = (n + 31) >> 5, np = nb * 32;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T *xs = reinterpret_cast<T *>(smem_raw);  // [np]
@@ -699,7 +699,7 @@ __global__ void __launch_bounds__(256) k_symv_batched(const SymvTask *__restrict
     }
     return;
   }
-  T *mysum = scratch + ((long long)blockIdx.y * S + sidx) * ld_scr;
+  T *mysum = scratch + ((long long)t.scr + sidx) * ld_scr;
   for (int r = tid; r < n; r += 256) {
     T v = part[r];
 #pragma unroll
@@ -708,51 +708,306 @@ __global__ void __launch_bounds__(256) k_symv_batched(const SymvTask *__restrict
   }
   __threadfence();
   __syncthreads();
-  if (tid == 0) last = (atomicAdd(&counter[blockIdx.y], 1) == S - 1);
+  if (tid == 0) last = (atomicAdd(&counter[t.ctr], 1) == S - 1);
   __syncthreads();
   if (!last) return;
   __threadfence();
-  const T *sums = scratch + (long long)blockIdx.y * S * ld_scr;
+  const T *sums = scratch + (long long)t.scr * ld_scr;
   for (int r = tid; r < n; r += 256) {
     T v = __ldcg(sums + r);
     for (int q = 1; q < S; ++q) v += __ldcg(sums + (long long)q * ld_scr + r);
     const double o = alpha * (double)v;
     y[t.y_off + r] = (t.flags & 2) ? y[t.y_off + r] + o : o;
   }
-  if (tid == 0) counter[blockIdx.y] = 0;  // ready for the next launch
+  if (tid == 0) counter[t.ctr] = 0;  // ready for the next launch
 }
 
+static size_t symv_fix_smem(int max_n) {
+  const size_t nb = (max_n + 31) / 32;
+  return nb * 32 * (8 * sizeof(double) + sizeof(int2)) + ((nb + 3) & ~(size_t)3) * sizeof(int) + 8 * 32 * 33 * sizeof(int2);
+}
 template <typename T>
 size_t symv_smem(int max_n) {
   const size_t np = (size_t)((max_n + 31) / 32) * 32;
-  return sizeof(T) * (9 * np + 8 * 32 * 33);
+  return std::is_same<T, double>::value ? symv_fix_smem(max_n) : sizeof(T) * (9 * np + 8 * 32 * 33);
 }
 
-// CTAs per matrix: one while the matrices alone fill the resident slots (a split costs a
-// partial-sum round trip and shorter prefetch runs), else enough to fill one wave, with at
-// least 8 tiles per CTA (one per warp) and at most 16.  slots = 0: one CTA per matrix.
-int symv_split(int ntasks, int max_n, int slots) {
-  if (slots <= 0 || ntasks <= 0 || ntasks >= slots) return 1;
-  const long long nb = (max_n + 31) / 32, ntiles = nb * (nb + 1) / 2;
-  const int smax = (int)std::max<long long>(1, std::min<long long>(16, ntiles / 8));
-  return std::max(1, std::min(smax, (slots + ntasks - 1) / ntasks));
+// The CTAs of a launch: whole matrices while they fill the resident slots (a split costs a
+// partial-sum round trip and shorter prefetch runs), largest first, and the ones that would make up
+// a last, part-empty wave split over several CTAs.  Which ones and into how many parts is decided by
+// scheduling the CTAs on the slots with a cost of their tiles plus a fixed part (staging, reduction),
+// for every candidate.  1,024 matrices of order 772 on 456 slots: 3 waves of whole matrices, 2.3 so.
+std::vector<SymvTask> symv_plan(const std::vector<SymvTask> &tasks, int slots, int *scratch_rows, int *counters) {
+  constexpr double kFix = 24.0, kSplitFix = 20.0;  // in tiles of 32 x 32
+  const int n = (int)tasks.size();
+  auto tiles = [](const SymvTask &t) { const double b = (t.n + 31) / 32; return b * (b + 1) / 2; };
+  std::vector<int> order(n);
+  for (int i = 0; i < n; ++i) order[i] = i;
+  std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return tasks[a].n > tasks[b].n; });
+  double total = 0.0;
+  for (const SymvTask &t : tasks) total += tiles(t);
+  slots = std::max(1, slots);
+  auto parts_of = [&](int i, int tail, int p) {  // parts of the i-th matrix of the order
+    const double w = tiles(tasks[order[i]]);
+    const int most = (int)std::max(1.0, std::min(16.0, w / 8.0));  // one tile per warp at least
+    int q = i >= n - tail ? p : 1;
+    if (w > total / slots) q = std::max(q, (int)std::ceil(w * slots / total));
+    return std::min(q, most);
+  };
+  auto makespan = [&](int tail, int p) {
+    std::vector<double> load(slots, 0.0);  // a heap of the slots' finishing times
+    auto later = [](double a, double b) { return a > b; };
+    for (int i = 0; i < n; ++i) {
+      const int q = parts_of(i, tail, p);
+      const double c = tiles(tasks[order[i]]) / q + kFix + (q > 1 ? kSplitFix : 0.0);
+      for (int k = 0; k < q; ++k) {
+        std::pop_heap(load.begin(), load.end(), later);
+        load.back() += c;
+        std::push_heap(load.begin(), load.end(), later);
+      }
+    }
+    return *std::max_element(load.begin(), load.end());
+  };
+  int best_tail = 0, best_p = 1;
+  double best = makespan(0, 1);
+  for (int tail : {n % slots, n % slots + slots, n / 2, n})
+    for (int p : {2, 3, 4, 5, 6, 8, 12, 16}) {
+      if (tail <= 0 || tail > n) continue;
+      const double m = makespan(tail, p);
+      if (m < 0.98 * best) { best = m; best_tail = tail; best_p = p; }
+    }
+  std::vector<SymvTask> out;
+  int rows = 0, ctrs = 0;
+  for (int i = 0; i < n; ++i) {
+    SymvTask t = tasks[order[i]];
+    t.nparts = parts_of(i, best_tail, best_p);
+    if (t.nparts > 1) {
+      t.scr = rows;
+      t.ctr = ctrs++;
+      rows += t.nparts;
+    }
+    for (t.part = 0; t.part < t.nparts; ++t.part) out.push_back(t);
+  }
+  *scratch_rows = rows;
+  *counters = ctrs;
+  return out;
+}
+
+
+void launch_symv_batched(int ntasks, int max_n, const SymvTask *d_tasks, const float *A, const double *x,
+                         const int *xidx, double *y, double alpha, const int *done, float *scratch, int *counter,
+                         int ld_scr, cudaStream_t s) {
+  if (ntasks == 0 || max_n == 0) return;
+  k_symv_batched<float><<<ntasks, 256, symv_smem<float>(max_n), s>>>(d_tasks, A, x, xidx, y, alpha, done, scratch,
+                                                                    counter, ld_scr);
+  count_launch();
+}
+
+// ---- FP64 symmetric products in integer arithmetic --------------------------------
+// The FP64 pipe (2 multiply-adds per SM and clock) cannot keep up with HBM: a symmetric product needs
+// 5.4 of them per SM and clock at the copy rate.  So the operators' lower block triangles are kept a
+// second time as 32 x 32 tiles of fixed-point numbers: every tile is scaled by a power of two and
+// rounded once to 55 bits, X = 2^28 h + l with |h|, |l| <= 2^27 (8 bytes, as the FP64 entry, error below
+// 2^-56 of the tile's largest entry); x likewise by segments of 32.  A tile's product with a segment is
+// then four 32 x 32 -> 64-bit integer multiply-adds per entry, exact, and two FP64 instructions per
+// row and tile.  Packed tiles in the order of k_symv_batched; the same parts, partial vectors
+// and fixed orders.
+__device__ __forceinline__ int2 fix_split(double x, double scale) {  // scale = 2^(55 - e), |x| < 2^e
+  const long long X = __double2ll_rn(x * scale);
+  const int lo = (int)(X & ((1 << 28) - 1)), l = lo - ((lo >> 27) << 28);
+  return make_int2((int)((X - l) >> 28), l);
+}
+__device__ __forceinline__ double pow2(int e) {  // 2^e, e clamped to the normal range
+  return __hiloint2double((max(min(e, 1023), -1022) + 1023) << 20, 0);
+}
+constexpr int kFixNan = 1 << 20;  // exponent of a tile or segment that holds an infinity or a NaN
+constexpr int kFixMin = -900;     // smallest exponent (keeps the scale factor finite)
+__device__ __forceinline__ int fix_exp(int mag) {  // from the largest top word of the magnitudes
+  return mag >= 0x7ff00000 ? kFixNan : max((mag >> 20) - 1022, kFixMin);
+}
+
+// One tile per CTA, grid-stride over a matrix's tiles: task.a_off -> packed tile task.f_off + s.
+__global__ void __launch_bounds__(256) k_fix_tiles(const FixTask *__restrict__ tasks, const double *__restrict__ A,
+                                                   int2 *__restrict__ tiles, int *__restrict__ ex) {
+  const FixTask t = tasks[blockIdx.y];
+  const int nb = (t.n + 31) >> 5, ntiles = nb * (nb + 1) / 2;
+  __shared__ int smax[8];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for (int s = blockIdx.x; s < ntiles; s += gridDim.x) {
+    int I = (int)((sqrtf(8.f * s + 1.f) - 1.f) * 0.5f);
+    while ((I + 1) * (I + 2) / 2 <= s) ++I;
+    while (I * (I + 1) / 2 > s) --I;
+    const int J = s - I * (I + 1) / 2;
+    double v[4];
+    int mag = 0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int r = 32 * I + warp + 8 * q, c = 32 * J + lane;
+      v[q] = r < t.n && c < t.n ? A[t.a_off + (long long)r * t.ld + c] : 0.0;
+      mag = max(mag, __double2hiint(v[q]) & 0x7fffffff);
+    }
+    mag = __reduce_max_sync(0xffffffffu, mag);
+    if (lane == 0) smax[warp] = mag;
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < 8; ++q) mag = max(mag, smax[q]);
+    __syncthreads();
+    const int e = fix_exp(mag);
+    const double scale = e == kFixNan ? 0.0 : pow2(55 - e);
+    if (tid == 0) ex[t.f_off + s] = e;
+    int2 *out = tiles + (t.f_off + s) * 1024;
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      out[(warp + 8 * q) * 32 + lane] = e == kFixNan ? make_int2(0, 0) : fix_split(v[q], scale);
+  }
+}
+
+__device__ __forceinline__ void mad_wide(long long &acc, int a, int b) { acc += (long long)a * b; }
+
+__global__ void __launch_bounds__(256) k_symv_fix(const SymvTask *__restrict__ tasks, const int2 *__restrict__ tiles,
+                                                  const int *__restrict__ ex, const double *__restrict__ x,
+                                                  const int *__restrict__ xidx, double *__restrict__ y, double alpha,
+                                                  const int *__restrict__ done, double *__restrict__ scratch,
+                                                  int *__restrict__ counter, int ld_scr) {
+  if (done && *done) return;
+  const SymvTask t = tasks[blockIdx.x];
+  const int S = t.nparts, sidx = t.part;
+  const int n = t.n, nb = (n + 31) >> 5, np = nb * 32;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  double *part = reinterpret_cast<double *>(smem_raw);       // [8][np]
+  int2 *xs = reinterpret_cast<int2 *>(part + 8 * np);        // [np] the segments of x, split
+  int *xe = reinterpret_cast<int *>(xs + np);                // [nb] their exponents
+  int2 *stage = reinterpret_cast<int2 *>(xe + ((nb + 3) & ~3));  // [8][32][33]
+  __shared__ int last;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for (int b = warp; b < nb; b += 8) {
+    const int c = 32 * b + lane;
+    const double v = c < n ? ((t.flags & 1) ? x[xidx[t.x_off + c]] : x[t.x_off + c]) : 0.0;
+    const int e = fix_exp(__reduce_max_sync(0xffffffffu, __double2hiint(v) & 0x7fffffff));
+    xs[c] = e == kFixNan ? make_int2(0, 0) : fix_split(v, pow2(55 - e));
+    if (lane == 0) xe[b] = e;
+  }
+  for (int c = tid; c < 8 * np; c += 256) part[c] = 0.0;
+  __syncthreads();
+  const long long ntiles = (long long)nb * (nb + 1) / 2;
+  const long long c0 = ntiles * sidx / S, c1 = ntiles * (sidx + 1) / S;  // this CTA's run
+  const int s0 = (int)(c0 + (c1 - c0) * warp / 8), s1 = (int)(c0 + (c1 - c0) * (warp + 1) / 8);
+  int2 *tile = stage + warp * 32 * 33;
+  double *mine = part + warp * np;
+  int I = 0;
+  while ((I + 1) * (I + 2) / 2 <= s0) ++I;
+  int J = s0 - I * (I + 1) / 2;
+  const int4 *src = reinterpret_cast<const int4 *>(tiles + t.f_off * 1024) + lane;
+  const int *et = ex + t.f_off;
+  int4 buf[16];
+  int e1 = 0;
+  auto load = [&](int s) {
+#pragma unroll
+    for (int i = 0; i < 16; ++i) buf[i] = src[(long long)s * 512 + 32 * i];
+    e1 = et[s];
+  };
+  // sum of 32 products as FP64: (h h) 2^56 + (h l + l h) 2^28 + l l, the low part rounded to 2^28
+  auto value = [](long long hh, long long m, long long ll, int ea, int eb) {
+    m += (ll + (1 << 27)) >> 28;
+    const double v = fma(__ll2double_rn(hh), 268435456.0, __ll2double_rn(m));
+    return (ea == kFixNan || eb == kFixNan) ? __hiloint2double(0x7ff80000, 0) : v * pow2(ea + eb - 82);
+  };
+  if (s0 < s1) load(s0);
+  double racc = 0.0;  // row sums of the current block row
+  for (int s = s0; s < s1; ++s) {
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {  // entries 64 i + 2 lane, + 1 of the tile
+      int2 *p = tile + (2 * i + (lane >> 4)) * 33 + 2 * (lane & 15);
+      p[0] = make_int2(buf[i].x, buf[i].y);
+      p[1] = make_int2(buf[i].z, buf[i].w);
+    }
+    __syncwarp();
+    const int ci = I, cj = J, e = e1;
+    if (++J > I) { ++I; J = 0; }
+    if (s + 1 < s1) load(s + 1);  // in flight while this tile is multiplied
+    long long hh = 0, m = 0, ll = 0;
+#pragma unroll 8
+    for (int c = 0; c < 32; ++c) {
+      const int2 a = tile[lane * 33 + c], b = xs[32 * cj + c];
+      mad_wide(hh, a.x, b.x);
+      mad_wide(m, a.x, b.y);
+      mad_wide(m, a.y, b.x);
+      mad_wide(ll, a.y, b.y);
+    }
+    racc += value(hh, m, ll, e, xe[cj]);
+    if (cj < ci) {
+      hh = m = ll = 0;
+#pragma unroll 8
+      for (int r = 0; r < 32; ++r) {
+        const int2 a = tile[r * 33 + lane], b = xs[32 * ci + r];
+        mad_wide(hh, a.x, b.x);
+        mad_wide(m, a.x, b.y);
+        mad_wide(m, a.y, b.x);
+        mad_wide(ll, a.y, b.y);
+      }
+      mine[32 * cj + lane] += value(hh, m, ll, e, xe[ci]);
+    }
+    if (I != ci || s + 1 == s1) {
+      mine[32 * ci + lane] += racc;
+      racc = 0.0;
+    }
+    __syncwarp();
+  }
+  __syncthreads();
+  auto column = [&](int r) {
+    double v = part[r];
+#pragma unroll
+    for (int w = 1; w < 8; ++w) v += part[w * np + r];
+    return v;
+  };
+  if (S == 1) {
+    for (int r = tid; r < n; r += 256) {
+      const double o = alpha * column(r);
+      y[t.y_off + r] = (t.flags & 2) ? y[t.y_off + r] + o : o;
+    }
+    return;
+  }
+  double *mysum = scratch + ((long long)t.scr + sidx) * ld_scr;
+  for (int r = tid; r < n; r += 256) mysum[r] = column(r);
+  __threadfence();
+  __syncthreads();
+  if (tid == 0) last = (atomicAdd(&counter[t.ctr], 1) == S - 1);
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  const double *sums = scratch + (long long)t.scr * ld_scr;
+  for (int r = tid; r < n; r += 256) {
+    double v = __ldcg(sums + r);
+    for (int q = 1; q < S; ++q) v += __ldcg(sums + (long long)q * ld_scr + r);
+    const double o = alpha * v;
+    y[t.y_off + r] = (t.flags & 2) ? y[t.y_off + r] + o : o;
+  }
+  if (tid == 0) counter[t.ctr] = 0;  // ready for the next launch
 }
 
 template <typename T>
 int symv_occupancy(int max_n) {
   int occ = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_symv_batched<T>, 256, symv_smem<T>(max_n)) != cudaSuccess)
-    return 0;
+  const cudaError_t e =
+      std::is_same<T, double>::value
+          ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_symv_fix, 256, symv_smem<T>(max_n))
+          : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_symv_batched<float>, 256, symv_smem<T>(max_n));
+  if (e != cudaSuccess) return 0;
   return occ;
 }
 
-template <typename T>
-void launch_symv_batched(int ntasks, int max_n, int split, const SymvTask *d_tasks, const T *A, const double *x,
-                         const int *xidx, double *y, double alpha, const int *done, T *scratch, int *counter,
-                         int ld_scr, cudaStream_t s) {
+void launch_fix_tiles(int n, int max_n, const FixTask *d_tasks, const double *A, int2 *tiles, int *ex, cudaStream_t s) {
+  if (n == 0 || max_n == 0) return;
+  const int nb = ceil_div(max_n, 32);
+  k_fix_tiles<<<dim3(std::min(nb * (nb + 1) / 2, 64), n), 256, 0, s>>>(d_tasks, A, tiles, ex);
+  count_launch();
+}
+void launch_symv_fix(int ntasks, int max_n, const SymvTask *d_tasks, const int2 *tiles, const int *ex, const double *x,
+                     const int *xidx, double *y, double alpha, const int *done, double *scratch, int *counter,
+                     int ld_scr, cudaStream_t s) {
   if (ntasks == 0 || max_n == 0) return;
-  k_symv_batched<T><<<dim3(split, ntasks), 256, symv_smem<T>(max_n), s>>>(d_tasks, A, x, xidx, y, alpha, done,
-                                                                          scratch, counter, ld_scr);
+  k_symv_fix<<<ntasks, 256, symv_fix_smem(max_n), s>>>(d_tasks, tiles, ex, x, xidx, y, alpha, done, scratch, counter,
+                                                       ld_scr);
   count_launch();
 }
 
@@ -1172,8 +1427,7 @@ bool dense_configure() {
   ok &= cudaFuncSetAttribute(k_gemv_t<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim) == cudaSuccess;
   ok &= cudaFuncSetAttribute(k_symv_rows<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim) == cudaSuccess;
   ok &= cudaFuncSetAttribute(k_symv_batched<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim) == cudaSuccess;
-  ok &= cudaFuncSetAttribute(k_symv_batched<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim) ==
-        cudaSuccess;
+  ok &= cudaFuncSetAttribute(k_symv_fix, cudaFuncAttributeMaxDynamicSharedMemorySize, lim) == cudaSuccess;
   ok &= cudaFuncSetAttribute(k_symv_rows<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim) == cudaSuccess;
   ok &= cudaFuncSetAttribute(k_gemv_task<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim) == cudaSuccess;
   ok &= cudaFuncSetAttribute(k_gemv_task<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim) == cudaSuccess;
@@ -1191,8 +1445,6 @@ bool dense_configure() {
                                     cudaStream_t);                                                             \
   template size_t symv_smem<T>(int);                                                                           \
   template int symv_occupancy<T>(int);                                                                         \
-  template void launch_symv_batched<T>(int, int, int, const SymvTask *, const T *, const double *, const int *,\
-                                       double *, double, const int *, T *, int *, int, cudaStream_t);          \
   template void launch_gemv_task<T>(int, int, int, const GemvDesc *, const T *, const double *, const int *,   \
                                     double *, double, const int *, cudaStream_t);                              \
   template void launch_gemv_t_task<T>(int, int, int, const GemvDesc *, const T *, const double *, const int *, \

@@ -132,20 +132,24 @@ template <typename T>
 void launch_gemv_t_task(int ntasks, int max_rows, int max_cols, const GemvDesc *d_tasks, const T *A,
                         const double *x, const int *xidx, double *y, double alpha, const int *done, cudaStream_t s,
                         const CsrIn *csr = nullptr);
-// Batched symmetric GEMV over SymvTask (split CTAs per task, lower block triangle read once);
+// Batched symmetric GEMV, one CTA per SymvTask (lower block triangle read once);
 // symv_smem: its shared memory for matrices up to max_n (above dense_smem_limit: not usable);
-// symv_occupancy: resident CTAs per SM at that size; symv_split: CTAs per task for a number of
-// resident slots.  With split > 1, scratch holds ntasks x split rows of ld_scr >= max_n values
-// and counter ntasks zeroed ints (left zeroed by every launch).
+// symv_occupancy: resident CTAs per SM at that size; symv_plan: the CTAs (parts of matrices) for a
+// number of resident slots, with the scratch rows (of ld_scr >= max_n values) and zeroed counters
+// (left zeroed by every launch) that the split matrices use.
 template <typename T>
 size_t symv_smem(int max_n);
 template <typename T>
 int symv_occupancy(int max_n);
-int symv_split(int ntasks, int max_n, int slots);
-template <typename T>
-void launch_symv_batched(int ntasks, int max_n, int split, const SymvTask *d_tasks, const T *A, const double *x,
-                         const int *xidx, double *y, double alpha, const int *done, T *scratch, int *counter,
+std::vector<SymvTask> symv_plan(const std::vector<SymvTask> &tasks, int slots, int *scratch_rows, int *counters);
+void launch_symv_batched(int ntasks, int max_n, const SymvTask *d_tasks, const float *A, const double *x,
+                         const int *xidx, double *y, double alpha, const int *done, float *scratch, int *counter,
                          int ld_scr, cudaStream_t s);
+// FP64: the tiles packed in fixed point (1024 int2 and an exponent each), and the product with them
+void launch_fix_tiles(int n, int max_n, const FixTask *d_tasks, const double *A, int2 *tiles, int *ex, cudaStream_t s);
+void launch_symv_fix(int ntasks, int max_n, const SymvTask *d_tasks, const int2 *tiles, const int *ex, const double *x,
+                     const int *xidx, double *y, double alpha, const int *done, double *scratch, int *counter,
+                     int ld_scr, cudaStream_t s);
 // y (+)= A x for one large symmetric n x n row-major matrix (ld a multiple of 8, zero padding
 // columns), reading only its lower block triangle
 template <typename T>
