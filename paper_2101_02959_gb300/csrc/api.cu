@@ -58,7 +58,11 @@ struct DevMem {
 };
 
 // workspace of the tensor-core updates
-constexpr size_t kWsCap64 = (size_t)1 << 30, kWsCap32 = (size_t)512 << 20;
+constexpr size_t kWsCap64 = (size_t)1 << 30, kWsCap32 = (size_t)512 << 20, kWsCapCls = (size_t)256 << 20;
+
+// order from which a deluxe product runs on the tensor cores: FP64 n = 242 took 10.2 ms per Jacobian in
+// SIMT and about 1 ms so; below, a 128 x 64 tile is mostly padding
+constexpr int kProductMin = 48;
 
 inline int pad8(int n) { return (n + 7) & ~7; }
 inline long long pad32(long long n) { return (n + 31) & ~31LL; }
@@ -66,7 +70,7 @@ inline long long pad32(long long n) { return (n + 31) & ~31LL; }
 template <class T>
 struct Dense {
   T *K = nullptr, *Aug = nullptr, *Sorig = nullptr, *Z = nullptr, *SDD = nullptr, *Blk = nullptr, *CA = nullptr,
-    *Sinv = nullptr, *Dd = nullptr, *Linv = nullptr, *LdK = nullptr;  // Linv: block store scratch; LdK: K's
+    *Sinv = nullptr, *Dd = nullptr, *Linv = nullptr, *LinvC = nullptr, *LdK = nullptr;  // Linv, LinvC: block store scratch; LdK: K's
   // coarse problem in the local precision: augmented matrix, its block store, S_PiPi^-1
   T *Co = nullptr, *LdCo = nullptr, *CoInv = nullptr;
 };
@@ -290,9 +294,11 @@ struct bd_handle {
   // symmetric: each lower tile read once); used instead of gv_schur / gv_local when set
   SymvSet sv_schur, sv_local, sv_sdd;  // sv_sdd: the FETI-DP preconditioner's S_DeltaDelta
   // tensor-core factorisation: digit planes of the updates, inverses of the panels' diagonal blocks
-  SliceWs ws;
-  GemmTask *d_gemm = nullptr;
-  int n_gemm = 0;
+  SliceWs ws, ws_cls;  // ws_cls: of the deluxe classes, factorised on the second stream
+  // D_C^(j) products: blocks of order kProductMin and more on the tensor cores (FP64, or tensor cores on)
+  GemmTask *d_gemm = nullptr, *d_gemm_small = nullptr;
+  int n_gemm = 0, n_gemm_small = 0, max_small = 0, n_prod = 0, max_prod = 0;
+  MatDesc *d_prod[3] = {nullptr, nullptr, nullptr};
   int *d_ext_idx = nullptr;
   MatDesc *d_Sdesc = nullptr;
   CopySet cp_sorig, cp_sdd, cp_blk, cp_zx, cp_sinv, cp_coinv;
@@ -827,6 +833,23 @@ void setup_handle(bd_handle &h) {
     }
     h.n_gemm = (int)gt.size();
     h.d_gemm = m.upload(gt, s);
+    std::vector<GemmTask> small;
+    std::vector<MatDesc> pd[3];
+    for (const GemmTask &g : gt) {
+      if (g.n < kProductMin) {
+        small.push_back(g);
+        h.max_small = std::max(h.max_small, g.n);
+        continue;
+      }
+      pd[0].push_back(MatDesc{g.a_off, g.n, g.n, g.n, 0});
+      pd[1].push_back(MatDesc{g.b_off, g.n, g.n, g.n, 0});
+      pd[2].push_back(MatDesc{g.c_off, g.ldc, g.n, g.n, 0});
+      h.max_prod = std::max(h.max_prod, g.n);
+    }
+    h.n_gemm_small = (int)small.size();
+    h.d_gemm_small = m.upload(small, s);
+    h.n_prod = (int)pd[0].size();
+    for (int k = 0; k < 3; ++k) h.d_prod[k] = m.upload(pd[k], s);
     h.d_ext_idx = m.upload(ext_idx, s);
     auto mk = [&](const std::vector<GemvDesc> &v) {
       GemvSet g;
@@ -850,7 +873,7 @@ void setup_handle(bd_handle &h) {
     {  // (in mixed precision the autotuner may turn the tensor cores on)
       size_t want = 0, one = 0;
       int most = 1;
-      for (const EngineShape *q : {&h.shK, &h.shA, &h.shC, &h.shCo}) {
+      for (const EngineShape *q : {&h.shK, &h.shA, &h.shCo}) {
         auto need = [&](int n) {
           return h.mixed() ? slice_bytes<float>(n, q->max_m, q->max_e) : slice_bytes<double>(n, q->max_m, q->max_e);
         };
@@ -860,7 +883,16 @@ void setup_handle(bd_handle &h) {
       }
       h.ws.bytes = std::max(one, std::min(want, h.mixed() ? kWsCap32 : kWsCap64));
       h.ws.mem = m.alloc<unsigned char>(h.ws.bytes);
-      h.ws.pinv = m.alloc<unsigned char>((size_t)most * kPanel64 * kPanel64 * (h.mixed() ? sizeof(float) : sizeof(double)));
+      const size_t inv = (size_t)kPanel64 * kPanel64 * (h.mixed() ? sizeof(float) : sizeof(double));
+      h.ws.pinv = m.alloc<unsigned char>(most * inv);
+      // the deluxe classes' factorisation and products run beside the local Neumann factorisation
+      auto cls = [&](int n) {
+        return h.mixed() ? std::max(slice_bytes<float>(n, h.shC.max_m, h.shC.max_e), product_bytes<float>(n, h.max_prod))
+                         : std::max(slice_bytes<double>(n, h.shC.max_m, h.shC.max_e), product_bytes<double>(n, h.max_prod));
+      };
+      h.ws_cls.bytes = std::max(cls(1), std::min(cls(std::max(h.shC.count, h.n_prod)), kWsCapCls));
+      h.ws_cls.mem = m.alloc<unsigned char>(h.ws_cls.bytes);
+      h.ws_cls.pinv = m.alloc<unsigned char>(std::max(h.shC.count, 1) * inv);
     }
     // sparse pattern of S_PP: the (p, q) pairs that some subdomain couples, with the
     // offsets of their local contributions in the augmented matrices (subdomain order)
@@ -1064,7 +1096,8 @@ void setup_handle(bd_handle &h) {
     D.CA = m.alloc<T>(h.CA_el);
     D.Sinv = m.alloc<T>(h.Sinv_el);
     D.Dd = m.alloc<T>(h.Dd_el);
-    D.Linv = m.alloc<T>((size_t)std::max({h.A_blk, h.C_blk, 1}) * kNB * kNB);
+    D.Linv = m.alloc<T>((size_t)std::max(h.A_blk, 1) * kNB * kNB);
+    D.LinvC = m.alloc<T>((size_t)std::max(h.C_blk, 1) * kNB * kNB);
     D.LdK = m.alloc<T>((size_t)std::max(h.K_blk, 1) * kNB * kNB);
     D.Co = m.alloc<T>((size_t)h.ld_co * 2 * h.np);
     D.LdCo = m.alloc<T>((size_t)std::max(1, ceil_div(h.np, kNB)) * kNB * kNB);
@@ -1154,18 +1187,29 @@ void linearize_t(bd_handle &h, Dense<T> &D, bool precond) {
   launch_copy<T, T>(h.cp_sdd.n, h.cp_sdd.max_elems, h.cp_sdd.d, D.Aug, D.SDD, s);
   pack_symv(h.sv_sdd, D.SDD, s);
   launch_copy<T, T>(h.cp_blk.n, h.cp_blk.max_elems, h.cp_blk.d, D.Aug, D.Blk, s);
-  run_engine_groups<T>(h, h.shA, h.d_Adesc, D.Aug, D.Linv);
-  launch_copy<T, T>(h.cp_zx.n, h.cp_zx.max_elems, h.cp_zx.d, D.Aug, D.Z, s);
-  pack_symv(h.sv_local, D.Z, s);
-  launch_class_aug<T>(h.ncls, h.max_nc, h.d_cls, h.d_pairs, D.Blk, h.d_Cdesc, D.CA, s);
-  engine_partial_cholesky<T>(h.shC, h.d_Cdesc, D.CA, h.d_err, s, D.Linv, &h.prof, h.tc(), h.ws);
-  launch_copy<T, T>(h.cp_sinv.n, h.cp_sinv.max_elems, h.cp_sinv.d, D.CA, D.Sinv, s);
+  // the deluxe classes need only the blocks just copied: their factorisation and the products D_C^(j)
+  // run on the second stream beside the local Neumann factorisation (each is a chain of short launches)
+  cudaStream_t s2 = h.s2;
+  ck(cudaEventRecord(h.ev_fork, s), "record");
+  ck(cudaStreamWaitEvent(s2, h.ev_fork, 0), "wait");
+  launch_class_aug<T>(h.ncls, h.max_nc, h.d_cls, h.d_pairs, D.Blk, h.d_Cdesc, D.CA, s2);
+  engine_partial_cholesky<T>(h.shC, h.d_Cdesc, D.CA, h.d_err, s2, D.LinvC, &h.prof, h.tc(), h.ws_cls);
+  launch_copy<T, T>(h.cp_sinv.n, h.cp_sinv.max_elems, h.cp_sinv.d, D.CA, D.Sinv, s2);
   if (h.opt.scaling == BD_SCALING_RHO) {
     const double si = std::max({h.fp.sigma_i[0], h.fp.sigma_i[1], h.fp.sigma_i[2]});
     const double se = std::max({h.fp.sigma_e[0], h.fp.sigma_e[1], h.fp.sigma_e[2]});
-    launch_rho_blocks<T>(h.ncls, h.d_cls, h.d_pairs, si, se, D.Sinv, D.Blk, s);
+    launch_rho_blocks<T>(h.ncls, h.d_cls, h.d_pairs, si, se, D.Sinv, D.Blk, s2);
   }
-  launch_small_gemm<T>(h.n_gemm, h.max_nc, h.d_gemm, D.Sinv, D.Blk, D.Dd, s);
+  if (!h.mixed() || h.tc()) {  // S_C^(j) is symmetric: Sinv S_C^(j) = Sinv (S_C^(j))^T
+    launch_small_gemm<T>(h.n_gemm_small, h.max_small, h.d_gemm_small, D.Sinv, D.Blk, D.Dd, s2);
+    launch_product<T>(h.d_prod[0], D.Sinv, h.d_prod[1], D.Blk, h.d_prod[2], D.Dd, h.n_prod, h.max_prod, h.ws_cls, h.d_err, s2);
+  } else {
+    launch_small_gemm<T>(h.n_gemm, h.max_nc, h.d_gemm, D.Sinv, D.Blk, D.Dd, s2);
+  }
+  ck(cudaEventRecord(h.ev_join, s2), "record");
+  run_engine_groups<T>(h, h.shA, h.d_Adesc, D.Aug, D.Linv);
+  launch_copy<T, T>(h.cp_zx.n, h.cp_zx.max_elems, h.cp_zx.d, D.Aug, D.Z, s);
+  pack_symv(h.sv_local, D.Z, s);
   // coarse: S_PiPi assembled in FP64 (sparse) and, in the local precision, into the augmented
   // matrix whose partial Cholesky leaves the explicit inverse; the solve refines against FP64
   ck(cudaMemsetAsync(D.Co, 0, sizeof(T) * (size_t)h.ld_co * 2 * h.np, s), "memset coarse");
@@ -1179,6 +1223,7 @@ void linearize_t(bd_handle &h, Dense<T> &D, bool precond) {
   }
   launch_copy<T, T>(h.cp_coinv.n, h.cp_coinv.max_elems, h.cp_coinv.d, D.Co, D.CoInv, s);
   if (h.d_CoInv64) coarse_refine64<T>(h.np, D.CoInv, pad8(h.np), h.d_Co64d, h.d_CoInv64, h.d_CoW, h.d_CoY, s);
+  ck(cudaStreamWaitEvent(s, h.ev_join, 0), "wait");
 }
 
 // counted = true for the Jacobian evaluations of the solve (Newton, bidomain_linearize):

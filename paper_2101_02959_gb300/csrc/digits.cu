@@ -70,7 +70,8 @@ struct Range {
 // mode 0: an outer block by its finished panel [K0, K0 + pw): rows [K0 + w, m), columns up to K1;
 // mode 1: rows and columns [e, m), K = [K0, min(K1, e)); mode 2: rows [K1, m), columns [K1, e),
 // K = [ka, kz) inside the outer block [K0, K1); mode 3: the panel solve, rows [K0 + w, m),
-// K = [K0, K0 + w), columns of the panel (B from the inverse of its diagonal block).
+// K = [K0, K0 + w), columns of the panel (B from the inverse of its diagonal block); mode 4: the plain
+// product C = A B^T of n x n matrices (desc.e = desc.m = n).
 __device__ inline bool upd_range(const MatDesc &d, const Upd64 &u, Range &r) {
   if (u.mode == 1) {
     r.row0 = d.e; r.colend = d.m; r.kb = u.ka; r.ke = min(u.kz, d.e); r.w = 0;
@@ -79,6 +80,10 @@ __device__ inline bool upd_range(const MatDesc &d, const Upd64 &u, Range &r) {
   if (u.mode == 2) {
     r.row0 = u.K1; r.colend = d.e; r.kb = u.ka; r.ke = min(u.kz, u.K1); r.w = 0;
     return u.K1 < d.e && r.kb < r.ke;
+  }
+  if (u.mode == 4) {
+    r.row0 = 0; r.colend = d.m; r.kb = u.ka; r.ke = min(u.kz, d.m); r.w = 0;
+    return r.kb < r.ke;
   }
   if (u.K0 >= d.e) return false;
   r.w = min(u.pw, d.e - u.K0);
@@ -90,7 +95,7 @@ __device__ inline bool upd_range(const MatDesc &d, const Upd64 &u, Range &r) {
 // Columns of the update as a count of leading virtual rows (row(v) = column of the update).
 __device__ inline int virt_cols(const MatDesc &d, const Upd64 &u, const Range &r, const BandRows &br) {
   if (u.mode == 3) return r.w;
-  if (u.mode == 1) return br.nv;
+  if (u.mode == 1 || u.mode == 4) return br.nv;
   return max(0, min(r.colend, band_limit(d, r.ke)) - r.row0);
 }
 
@@ -155,7 +160,7 @@ __global__ void __launch_bounds__(256) k_slice(const MatDesc *__restrict__ desc,
   }
   const int k = k0 + 8 * t;
   T x[8];
-  if (valid && k + 8 <= r.ke) {  // k a multiple of 8 from an even start, rows 32-byte aligned
+  if (valid && k + 8 <= r.ke && (reinterpret_cast<uintptr_t>(src + k) & 15) == 0) {
     constexpr int VN = 16 / (int)sizeof(T);
 #pragma unroll
     for (int q = 0; q < 8; q += VN) *reinterpret_cast<int4 *>(&x[q]) = *reinterpret_cast<const int4 *>(src + k + q);
@@ -199,14 +204,14 @@ struct Tile {
 };
 
 // Tile (ti, tj) of matrix b; false when it holds no entry of the update.
-__device__ inline bool make_tile(const MatDesc *__restrict__ desc, const Upd64 &u, int b, int ti, int tj, int n,
-                                 Tile &t) {
+__device__ inline bool make_tile(const MatDesc *__restrict__ desc, const MatDesc *__restrict__ out, const Upd64 &u,
+                                 int b, int ti, int tj, int n, Tile &t) {
   const MatDesc d = desc[b];
   Range r;
   if (!upd_range(d, u, r)) return false;
   t.v0 = ti * kUM;
   t.c0 = tj * n;
-  if (u.mode != 3 && t.c0 > t.v0 + kUM - 1) return false;
+  if (u.mode < 3 && t.c0 > t.v0 + kUM - 1) return false;
   t.br = band_rows(d, r.row0, r.ke);
   t.ncv = virt_cols(d, u, r, t.br);
   if (t.v0 >= t.br.nv || t.c0 >= t.ncv) return false;
@@ -225,13 +230,20 @@ __device__ inline bool make_tile(const MatDesc *__restrict__ desc, const Upd64 &
     }
   }
   if (ks >= r.ke) return false;
-  t.off = d.off;
-  t.ld = d.ld;
+  t.off = out[b].off;
+  t.ld = out[b].ld;
   t.b = b;
   t.ch0 = (ks - r.kb) / kUK;
   t.ch1 = (r.ke - r.kb + kUK - 1) / kUK;
   return true;
 }
+
+// Digit planes and row exponents of one operand: blocks of 64 rows, chunks and groups of columns.
+struct Planes {
+  const unsigned char *sl;
+  const int *ex;
+  int nrb, nkc, ng;
+};
 
 // Reads one group's accumulators (CPW columns from taddr) and adds sum_w B^(2D-w) P_w 2^(er + ec) to
 // acc; the accumulator of weight w is released on bfree + 8 w once read.
@@ -319,11 +331,9 @@ __device__ __forceinline__ void drain(uint32_t taddr, uint32_t bfree, int lane, 
 // shared memory (an MMA takes 65 clocks, measured, where the tensor pipe needs 32, since A is read
 // again by every MMA) and, for short K, by reading and writing C between groups.
 template <typename T>
-__global__ void __launch_bounds__(kUThreads, 1) k_update(const MatDesc *__restrict__ desc, T *__restrict__ base,
-                                                         Upd64 u, const unsigned char *__restrict__ sl,
-                                                         const int *__restrict__ ex, int nrb, int nkc, int ng,
-                                                         const unsigned char *__restrict__ slb,
-                                                         const int *__restrict__ exb, int nct, int per, int total,
+__global__ void __launch_bounds__(kUThreads, 1) k_update(const MatDesc *__restrict__ desc,
+                                                         const MatDesc *__restrict__ out, T *__restrict__ base, Upd64 u,
+                                                         Planes pa, Planes pb, int nct, int per, int total,
                                                          int *__restrict__ err) {
   using C = Dig<T>;
   constexpr int N = C::N, S = C::Stages, CPG = C::Grp / kUK;
@@ -369,7 +379,7 @@ __global__ void __launch_bounds__(kUThreads, 1) k_update(const MatDesc *__restri
       if (k >= 2) ok = tcp::mbar_wait(bused + 8 * slot, ((k >> 1) - 1) & 1);
       const long long idx = blockIdx.x + (32LL * k + lane) * gridDim.x;
       Tile t;
-      const bool valid = idx < total && make_tile(desc, u, (int)(idx / per), (int)(idx % per) / nct,
+      const bool valid = idx < total && make_tile(desc, out, u, (int)(idx / per), (int)(idx % per) / nct,
                                                   (int)(idx % per) % nct, N, t);
       const unsigned m = __ballot_sync(0xffffffffu, valid);
       if (valid) ring[slot][__popc(m & ((1u << lane) - 1u))] = t;
@@ -383,7 +393,6 @@ __global__ void __launch_bounds__(kUThreads, 1) k_update(const MatDesc *__restri
   } else if (warp == kDrain) {
     if (lane == 0) {
       bool ok = true;
-      const bool inv = u.mode == 3;
       int n = 0;
       for (int k = 0; ok; ++k) {
         const int slot = k & 1;
@@ -391,11 +400,9 @@ __global__ void __launch_bounds__(kUThreads, 1) k_update(const MatDesc *__restri
         const int cnt = ring_n[slot];
         for (int q = 0; q < (cnt & 255) && ok; ++q) {
           const Tile &t = ring[slot][q];
-          const int nrbB = inv ? N / 64 : nrb, b = t.b, ch1 = t.ch1;
-          const unsigned char *pa = sl + (((long long)b * nkc + t.ch0) * C::D * nrb + (t.v0 >> 6)) * kBlkBytes;
-          const unsigned char *pb = (inv ? slb + (long long)b * (u.pw / kUK) * C::D * nrbB * kBlkBytes
-                                         : sl + (long long)b * nkc * C::D * nrb * kBlkBytes) +
-                                    ((long long)t.ch0 * C::D * nrbB + (t.c0 >> 6)) * kBlkBytes;
+          const int ch1 = t.ch1;
+          const unsigned char *qa = pa.sl + (((long long)t.b * pa.nkc + t.ch0) * C::D * pa.nrb + (t.v0 >> 6)) * kBlkBytes;
+          const unsigned char *qb = pb.sl + (((long long)t.b * pb.nkc + t.ch0) * C::D * pb.nrb + (t.c0 >> 6)) * kBlkBytes;
           for (int c = t.ch0; c < ch1; ++c, ++n) {
             const int s = n % S;
             if (n >= S && !tcp::mbar_wait(bempty + 8 * s, ((n / S) - 1) & 1)) { ok = false; break; }
@@ -403,12 +410,12 @@ __global__ void __launch_bounds__(kUThreads, 1) k_update(const MatDesc *__restri
             tcp::mbar_expect(bar, stage_bytes<T>());
 #pragma unroll
             for (int i = 0; i < C::D; ++i) {
-              tcp::bulk_load(dst + i * 2 * kBlkBytes, pa + (long long)i * nrb * kBlkBytes, 2 * kBlkBytes, bar);
-              tcp::bulk_load(dst + a_bytes<T>() + i * (N / 64) * kBlkBytes, pb + (long long)i * nrbB * kBlkBytes,
+              tcp::bulk_load(dst + i * 2 * kBlkBytes, qa + (long long)i * pa.nrb * kBlkBytes, 2 * kBlkBytes, bar);
+              tcp::bulk_load(dst + a_bytes<T>() + i * (N / 64) * kBlkBytes, qb + (long long)i * pb.nrb * kBlkBytes,
                              (N / 64) * kBlkBytes, bar);
             }
-            pa += (long long)C::D * nrb * kBlkBytes;
-            pb += (long long)C::D * nrbB * kBlkBytes;
+            qa += (long long)C::D * pa.nrb * kBlkBytes;
+            qb += (long long)C::D * pb.nrb * kBlkBytes;
           }
         }
         tcp::mbar_arrive(bused + 8 * slot);
@@ -485,23 +492,23 @@ __global__ void __launch_bounds__(kUThreads, 1) k_update(const MatDesc *__restri
         const int g0 = t.ch0 / CPG, g1 = (t.ch1 + CPG - 1) / CPG;
         // the matrix row of this lane's tile row
         const int vrow = t.v0 + rq + lane, myrow = t.br.row(min(vrow, t.br.nv - 1)), nrow = min(32, t.br.nv - t.v0 - rq);
-        if (u.mode != 3 && lane < nrow && t.c0 + cq < t.ncv)  // C towards L2 while the products form
+        if (u.mode < 3 && lane < nrow && t.c0 + cq < t.ncv)  // C towards L2 while the products form
           asm volatile("prefetch.global.L2 [%0];" ::"l"(base + t.off + (long long)myrow * t.ld + t.br.row(t.c0 + cq)));
         T acc[CPW];
 #pragma unroll
         for (int c = 0; c < CPW; ++c) acc[c] = T(0);
         // the exponents of a group are fetched while the group before it is drained
-        const int *exr = ex + (long long)t.b * ng * (nrb * 64) + t.v0 + rq + lane;
-        const int *exc = (u.mode == 3 ? exb + (long long)t.b * N : ex + (long long)t.b * ng * (nrb * 64)) + t.c0 + cq + lane % CPW;
-        const int estep = u.mode == 3 ? 0 : nrb * 64;
-        int er1 = exr[(long long)g0 * (nrb * 64)], ec1 = exc[(long long)g0 * estep];
+        const int *exr = pa.ex + (long long)t.b * pa.ng * (pa.nrb * 64) + t.v0 + rq + lane;
+        const int *exc = pb.ex + (long long)t.b * pb.ng * (pb.nrb * 64) + t.c0 + cq + lane % CPW;
+        const int rstep = pa.nrb * 64, cstep = pb.nrb * 64;
+        int er1 = exr[(long long)g0 * rstep], ec1 = exc[(long long)g0 * cstep];
         for (int g = g0; g < g1; ++g, ++G) {
           const int er = er1;
           ecol[lane % CPW] = sizeof(T) == 8 ? ec1 : __float_as_int(half_scale(ec1));
           __syncwarp();
           if (g + 1 < g1) {
-            er1 = exr[(long long)(g + 1) * (nrb * 64)];
-            ec1 = exc[(long long)(g + 1) * estep];
+            er1 = exr[(long long)(g + 1) * rstep];
+            ec1 = exc[(long long)(g + 1) * cstep];
           }
           ok = ok && tcp::mbar_wait(bacc, G & 1);
           tcp::fence_after();
@@ -520,9 +527,9 @@ __global__ void __launch_bounds__(kUThreads, 1) k_update(const MatDesc *__restri
           const int vc = t.c0 + cq + c1 + lc;
           T *Cc = base + t.off + (u.mode == 3 ? u.K0 + vc : t.br.row(vc < t.ncv ? vc : 0));
           // rows of this lane: r0 + RPI i below nrow, on or below the diagonal
-          const int rmin = u.mode == 3 ? 0 : vc - t.v0 - rq, rend = vc < t.ncv ? nrow : 0;
+          const int rmin = u.mode >= 3 ? 0 : vc - t.v0 - rq, rend = vc < t.ncv ? nrow : 0;
           T cv[NI];
-          if (u.mode != 3) {
+          if (u.mode < 3) {
 #pragma unroll
             for (int i = 0; i < NI; ++i) {
               const int r = r0 + RPI * i, row = __shfl_sync(0xffffffffu, myrow, r);
@@ -533,7 +540,7 @@ __global__ void __launch_bounds__(kUThreads, 1) k_update(const MatDesc *__restri
           for (int i = 0; i < NI; ++i) {
             const int r = r0 + RPI * i, row = __shfl_sync(0xffffffffu, myrow, r);
             const T a = stage[r * (EC + 1) + lc];
-            if (r >= rmin && r < rend) Cc[(long long)row * t.ld] = u.mode == 3 ? a : cv[i] - a;
+            if (r >= rmin && r < rend) Cc[(long long)row * t.ld] = u.mode >= 3 ? a : cv[i] - a;
           }
           __syncwarp();
         }
@@ -560,8 +567,8 @@ __global__ void __launch_bounds__(kUThreads, 1) k_update(const MatDesc *__restri
 // A warp issues one FP64 instruction in 64 clocks (measured, dependent or not) and the SM four of
 // them at a time, so the work is spread over the four schedulers: in ldl_inv32 warps 0-3 hold
 // every fourth column of the block and of its inverse (lane = row) and eliminate one column a step,
-// root-free: the step's chain is one reciprocal, one scaling, one update (about 560 clocks), and the
-// other updates fit beside it; the square roots of the 32 pivots are taken together at the end.
+// root-free: the step's chain is one update, one reciprocal, one scaling, and the other updates run
+// beside it; the square roots of the 32 pivots are taken together at the end.
 // Between the halves 32 x 32 x 32 products over all warps (L_21 = A_21 Y_11^T,
 // A_22 -= L_21 L_21^T, Y_21 = -Y_22 (L_21 Y_11)), column groups paired so that the schedulers get
 // equal triangles.  Panels of 64 columns and not 128: the count of FP64 instructions grows with the
@@ -572,8 +579,20 @@ constexpr size_t diag_smem() {
   return sizeof(T) * (2 * (size_t)kDP * kDLD + 32 * 33);
 }
 
+// 1 / p: one step of Householder's third-order iteration y (1 + e + e^2), e = 1 - p y, from the FP32
+// reciprocal (relative error 2^-23, so 2^-66 after the step); far outside the FP32 range, the division.
+__device__ __forceinline__ double recip(double p) {
+  if (!(p > 1e-30 && p < 1e30)) return 1.0 / p;
+  const double y = (double)__fdividef(1.f, (float)p), e = fma(-p, y, 1.0);
+  return fma(y, fma(e, e, e), y);
+}
+__device__ __forceinline__ float recip(float p) { return 1.f / p; }
+
 // Lower Cholesky factor of the 32 x 32 block of P at (o, o) and its inverse into Y; warps 0-3.
-// Columns at and after the block's width hold the identity.
+// Columns at and after the block's width hold the identity.  The owner of column c + 1 updates it
+// first, publishes it and arrives at the column's barrier before it makes the rest of step c's
+// updates, so that the others never wait for those; four column buffers and two barriers in turn keep
+// the steps apart.
 template <typename T>
 __device__ __forceinline__ void ldl_inv32(T *P, T *Y, int o, int s, int lane, T (*Lc)[2][32], T *piv, bool &bad) {
   T a[8], y[8];
@@ -583,29 +602,35 @@ __device__ __forceinline__ void ldl_inv32(T *P, T *Y, int o, int s, int lane, T 
     a[q] = t <= lane ? P[(o + lane) * kDLD + o + t] : T(0);
     y[q] = t == lane ? T(1) : T(0);
   }
+  auto publish = [&](int c, T col) {  // column c, held by this warp
+    T p = __shfl_sync(0xffffffffu, col, c);
+    if (!(p > T(0))) { bad = true; p = T(1); }
+    const T inv = recip(p);
+    Lc[c & 3][0][lane] = col;                            // the column before scaling
+    Lc[c & 3][1][lane] = lane > c ? col * inv : T(0);   // unit-lower column
+    if (lane == c) piv[c] = p;
+    __threadfence_block();
+  };
+  if (s == 0) publish(0, a[0]);
 #pragma unroll
   for (int c = 0; c < 32; ++c) {
-    const int q0 = c >> 2, buf = c & 1;
-    if (s == (c & 3)) {
-      T p = __shfl_sync(0xffffffffu, a[q0], c);
-      if (!(p > T(0))) { bad = true; p = T(1); }
-      const T inv = T(1) / p;
-      Lc[buf][0][lane] = a[q0];                           // the column before scaling
-      Lc[buf][1][lane] = lane > c ? a[q0] * inv : T(0);   // unit-lower column
-      if (lane == c) piv[c] = p;
-    }
-    asm volatile("bar.sync 1, 128;" ::: "memory");
+    const int q0 = c >> 2, buf = c & 3;
+    // column c is published: its owner has arrived already (at c = 0 everyone waits)
+    if (c > 0 && s == (c & 3)) __syncwarp();
+    else if (c & 1) asm volatile("bar.sync 2, 128;" ::: "memory");
+    else asm volatile("bar.sync 1, 128;" ::: "memory");
     const T l = Lc[buf][1][lane];
-#pragma unroll
-    for (int d = 0; d < 4; ++d) {  // the next column's owner updates it first
-      const int q = q0 + (d == 3 ? 1 : 0);
-      if (d == 0 || d == 3) {
-        if (q < 8 && 4 * q + s > c) a[q] -= l * Lc[buf][0][4 * q + s];
-      }
+    const int qn = (c + 1) >> 2;  // the next column's index in its owner
+    const bool next = c < 31 && s == ((c + 1) & 3);
+    if (next) {
+      a[qn < 8 ? qn : 0] -= l * Lc[buf][0][c + 1 < 32 ? c + 1 : 0];
+      publish(c + 1, a[qn < 8 ? qn : 0]);
+      if ((c + 1) & 1) asm volatile("bar.arrive 2, 128;" ::: "memory");
+      else asm volatile("bar.arrive 1, 128;" ::: "memory");
     }
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
-      if (q > q0 + 1 && 4 * q + s > c) a[q] -= l * Lc[buf][0][4 * q + s];
+      if (q >= q0 && 4 * q + s > c && !(next && q == qn)) a[q] -= l * Lc[buf][0][4 * q + s];
       if (q <= q0 && 4 * q + s <= c) {
         const T yc = __shfl_sync(0xffffffffu, y[q], c);
         y[q] -= l * yc;
@@ -633,7 +658,7 @@ __global__ void __launch_bounds__(256) k_diag(const MatDesc *__restrict__ desc, 
   T *P = reinterpret_cast<T *>(smem_raw);  // [64][65] the block, lower, identity past w
   T *Y = P + kDP * kDLD;                        // [64][65] its inverse
   T *Tm = Y + kDP * kDLD;                       // [32][33]
-  __shared__ T Lc[2][2][32], piv[32];
+  __shared__ T Lc[4][2][32], piv[32];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   T *A = base + d.off + (long long)K0 * d.ld + K0;
   {
@@ -776,6 +801,7 @@ void launch_update(const MatDesc *d_desc, T *base, Upd64 u, int max_rows, int ma
       q.ka = ka;
       q.kz = std::min(zz, ka + kSliceK);
       const int kw = q.kz - ka, nkc = ceil_div(kw, kUK), ng = ceil_div(kw, C::Grp);
+      const Planes pa{sl, ex, nrb, nkc, ng}, pi{slb, exb, C::N / 64, kPanel64 / kUK, 1};
       k_slice<T><<<dim3(nrb * 64 / rpc, ng, nb), 256, 0, s>>>(d_desc + b0, base, q, nullptr, sl, ex, nrb, nkc, ng);
       count_launch();
       if (u.mode == 3) {
@@ -785,10 +811,41 @@ void launch_update(const MatDesc *d_desc, T *base, Upd64 u, int max_rows, int ma
         count_launch();
       }
       const int per = nrt * nct, total = per * nb;
-      k_update<T><<<std::min(total, kSms), kUThreads, update_smem<T>(), s>>>(d_desc + b0, base, q, sl, ex, nrb, nkc, ng,
-                                                                            slb, exb, nct, per, total, err);
+      k_update<T><<<std::min(total, kSms), kUThreads, update_smem<T>(), s>>>(d_desc + b0, d_desc + b0, base, q, pa,
+                                                                            u.mode == 3 ? pi : pa, nct, per, total, err);
       count_launch();
     }
+  }
+}
+
+template <typename T>
+size_t product_bytes(int count, int max_n) {
+  return 2 * (size_t)std::max(1, count) * rows_bytes<T>(max_n, std::max(max_n, 1));
+}
+
+// C = A B^T for `count` pairs of n x n matrices (n = desc.m = desc.e; the same n in all three
+// descriptors of a pair), in runs of pairs whose planes fit the workspace.
+template <typename T>
+void launch_product(const MatDesc *d_a, const T *A, const MatDesc *d_b, const T *B, const MatDesc *d_c, T *Cm, int count,
+                    int max_n, const SliceWs &ws, int *err, cudaStream_t s) {
+  if (count <= 0 || max_n <= 0) return;
+  using C = Dig<T>;
+  const int nrb = pad_rows(max_n) / 64, nkc = ceil_div(max_n, kUK), ng = ceil_div(max_n, C::Grp);
+  const int run = (int)std::max<size_t>(1, std::min<size_t>((size_t)count, ws.bytes / product_bytes<T>(1, max_n)));
+  const int nrt = ceil_div(max_n, kUM), nct = ceil_div(max_n, C::N), rpc = 256 / (C::Grp / 8);
+  const size_t planes = (size_t)run * planes_bytes<T>(nrb * 64, max_n);
+  unsigned char *sl[2] = {ws.mem, ws.mem + planes};
+  int *ex[2] = {reinterpret_cast<int *>(ws.mem + 2 * planes), nullptr};
+  ex[1] = ex[0] + (size_t)run * ng * nrb * 64;
+  const Upd64 u{4, 0, 0, 0, 0, max_n};
+  for (int b0 = 0; b0 < count; b0 += run) {
+    const int nb = std::min(run, count - b0), per = nrt * nct, total = per * nb;
+    k_slice<T><<<dim3(nrb * 64 / rpc, ng, nb), 256, 0, s>>>(d_a + b0, A, u, nullptr, sl[0], ex[0], nrb, nkc, ng);
+    k_slice<T><<<dim3(nrb * 64 / rpc, ng, nb), 256, 0, s>>>(d_b + b0, B, u, nullptr, sl[1], ex[1], nrb, nkc, ng);
+    k_update<T><<<std::min(total, kSms), kUThreads, update_smem<T>(), s>>>(
+        d_a + b0, d_c + b0, Cm, u, Planes{sl[0], ex[0], nrb, nkc, ng}, Planes{sl[1], ex[1], nrb, nkc, ng}, nct, per, total,
+        err);
+    count_launch(3);
   }
 }
 
@@ -796,7 +853,10 @@ void launch_update(const MatDesc *d_desc, T *base, Upd64 u, int max_rows, int ma
   template void launch_diag<T>(const MatDesc *, T *, int, int, int *, T *, T *, cudaStream_t);               \
   template size_t slice_bytes<T>(int, int, int);                                                             \
   template void launch_update<T>(const MatDesc *, T *, Upd64, int, int, int, const SliceWs &, int *,       \
-                                 cudaStream_t, const T *);
+                                 cudaStream_t, const T *);                                                  \
+  template size_t product_bytes<T>(int, int);                                                                \
+  template void launch_product<T>(const MatDesc *, const T *, const MatDesc *, const T *, const MatDesc *, T *, int, \
+                                  int, const SliceWs &, int *, cudaStream_t);
 BD_DIG_INST(float)
 BD_DIG_INST(double)
 

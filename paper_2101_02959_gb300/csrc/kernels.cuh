@@ -122,6 +122,11 @@ template <typename T>
 void launch_update(const MatDesc *d_desc, T *base, Upd64 u, int max_rows, int max_cols, int count, const SliceWs &ws,
                    int *err, cudaStream_t s, const T *pinv = nullptr);
 template <typename T>
+size_t product_bytes(int count, int max_n);
+template <typename T>
+void launch_product(const MatDesc *d_a, const T *A, const MatDesc *d_b, const T *B, const MatDesc *d_c, T *C, int count,
+                    int max_n, const SliceWs &ws, int *err, cudaStream_t s);
+template <typename T>
 void launch_diag(const MatDesc *d_desc, T *base, int K0, int count, int *err, T *store, T *pinv, cudaStream_t s);
 
 // The same products for many small matrices: one CTA per task over all its rows (columns)
