@@ -12,6 +12,33 @@ enum : int { DEV_ERR_NOT_SPD = 1, DEV_ERR_NAN = 2, DEV_ERR_TIMEOUT = 4 };
 
 constexpr int kWarp = 32;
 
+// Programmatic dependent launch: a kernel launched with launch_pdl may start while its predecessor on
+// the stream drains; it calls pdl_wait() first (which returns when the predecessor has completed and
+// its writes are visible) and then lets its own successor start the same way.  Every such kernel must call
+// it, in every thread and before any return, or its successor could run past work before it.
+__device__ __forceinline__ void pdl_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+template <class... P, class... A>
+void launch_maybe_pdl(bool pdl, void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args) {
+  cudaLaunchConfig_t c{};
+  c.gridDim = grid;
+  c.blockDim = block;
+  c.dynamicSmemBytes = smem;
+  c.stream = s;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  c.attrs = &at;
+  c.numAttrs = pdl ? 1 : 0;
+  cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
+}
+template <class... P, class... A>
+void launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args) {
+  launch_maybe_pdl(true, kernel, grid, block, smem, s, args...);
+}
+
 template <typename T>
 __device__ __forceinline__ T warp_sum(T v) {
 #pragma unroll

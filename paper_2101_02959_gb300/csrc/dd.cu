@@ -202,6 +202,7 @@ __global__ void k_coarse_rhs(int np, int gauge, const int *__restrict__ pl_ptr, 
 __global__ void k_coarse_resid(int np, const int *__restrict__ ptr, const int *__restrict__ col,
                                const double *__restrict__ val, const double *__restrict__ c,
                                const double *__restrict__ z, double *__restrict__ rho, const int *__restrict__ done) {
+  pdl_wait();
   if (done && *done) return;
   const int q = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (q >= np) return;
@@ -364,6 +365,7 @@ void launch_rho_blocks(int ncls, const ClassTask *cls, const PairTask *pairs, do
 // ---- sparse (CSR) matrix-vector product y = A x, y[zero] = 0 --------------------
 __global__ void k_spmv(int n, const int *__restrict__ ptr, const int *__restrict__ col, const double *__restrict__ val,
                        const double *__restrict__ x, double *__restrict__ y, int zero, const int *__restrict__ done) {
+  pdl_wait();
   if (done && *done) return;
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= n) return;
@@ -377,6 +379,7 @@ __global__ void k_spmv(int n, const int *__restrict__ ptr, const int *__restrict
 __global__ void k_gather_sum(int n, const int *__restrict__ ptr, const int *__restrict__ idx,
                              const double *__restrict__ src, double *__restrict__ y, int zero, double alpha,
                              const double *__restrict__ addend, const int *__restrict__ done, const CsrIn add_csr) {
+  pdl_wait();
   if (done && *done) return;
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= n) return;
@@ -441,6 +444,7 @@ __device__ inline void smem_gemv(const T *__restrict__ A, int n, const T *__rest
 // B w: lambda_ab = w_a - w_b on the class block.
 __global__ void k_jump(const LamTask *__restrict__ lt, const PairTask *__restrict__ pairs, const double *__restrict__ w,
                        double *__restrict__ lam, const int *__restrict__ done) {
+  pdl_wait();
   if (done && *done) return;
   const LamTask t = lt[blockIdx.y];
   const int u = blockIdx.x * blockDim.x + threadIdx.x;
@@ -451,6 +455,7 @@ __global__ void k_jump(const LamTask *__restrict__ lt, const PairTask *__restric
 // B^T lambda: w_(j,C) = sum of +-lambda over the multipliers touching (j, C).
 __global__ void k_jump_t(const WTask *__restrict__ wt, const WEnt *__restrict__ ent, const double *__restrict__ lam,
                          double *__restrict__ w, const int *__restrict__ done) {
+  pdl_wait();
   if (done && *done) return;
   const WTask t = wt[blockIdx.y];
   const int u = blockIdx.x * blockDim.x + threadIdx.x;
@@ -465,6 +470,7 @@ template <typename T>
 __global__ void k_jump_dt(const WTask *__restrict__ wt, const WEnt *__restrict__ ent, const T *__restrict__ blk,
                           const T *__restrict__ sinv, const double *__restrict__ mu, double *__restrict__ w,
                           const int *__restrict__ done) {
+  pdl_wait();
   if (done && *done) return;
   const WTask t = wt[blockIdx.x];
   extern __shared__ unsigned char smem_raw[];
@@ -492,6 +498,7 @@ template <typename T>
 __global__ void k_jump_d(const LamTask *__restrict__ lt, const PairTask *__restrict__ pairs, const T *__restrict__ blk,
                          const T *__restrict__ sinv, const double *__restrict__ y, double *__restrict__ mu,
                          const int *__restrict__ done) {
+  pdl_wait();
   if (done && *done) return;
   const LamTask t = lt[blockIdx.x];
   extern __shared__ unsigned char smem_raw[];
@@ -615,6 +622,7 @@ __global__ void k_pcg_alpha(KrylovState *__restrict__ ks, const double *__restri
 
 __global__ void k_pcg_xr(int n, const KrylovState *__restrict__ ks, const double *__restrict__ p,
                          const double *__restrict__ q, double *__restrict__ x, double *__restrict__ r) {
+  pdl_wait();
   if (ks->done) return;
   const double a = ks->alpha;
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) {
@@ -638,6 +646,7 @@ __global__ void k_pcg_beta(KrylovState *__restrict__ ks, const double *__restric
 }
 
 __global__ void k_pcg_p(int n, const KrylovState *__restrict__ ks, const double *__restrict__ z, double *__restrict__ p) {
+  pdl_wait();
   if (ks->done) return;
   const double b = ks->beta;
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n; t += gridDim.x * blockDim.x) p[t] = z[t] + b * p[t];
@@ -693,6 +702,7 @@ __global__ void k_pcg_dot_step(int n, int which, const double *__restrict__ a0, 
                                const double *__restrict__ a1, const double *__restrict__ b1,
                                double *__restrict__ partial, unsigned int *__restrict__ counter,
                                KrylovState *__restrict__ ks, double *__restrict__ hist) {
+  pdl_wait();
   if (ks->done) return;
   double s0 = 0.0, s1 = 0.0;
   for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < n; x += gridDim.x * blockDim.x) {
@@ -706,6 +716,7 @@ __global__ void k_pcg_dot_step(int n, int which, const double *__restrict__ a0, 
 // reduction of the operator output: s0 = a.y (and s1 = y.y when which = 1).
 __global__ void k_gather_sum_dot(int n, const int *__restrict__ ptr, const int *__restrict__ idx,
                                  const double *__restrict__ src, double *__restrict__ y, int zero, DotFuse f) {
+  pdl_wait();
   if (f.ks->done) return;
   double s0 = 0.0, s1 = 0.0;
   for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < n; r += gridDim.x * blockDim.x) {
@@ -723,6 +734,7 @@ __global__ void k_gather_sum_dot(int n, const int *__restrict__ ptr, const int *
 __global__ void k_spmv_dot(int n, const int *__restrict__ ptr, const int *__restrict__ col,
                            const double *__restrict__ val, const double *__restrict__ x, double *__restrict__ y,
                            int zero, DotFuse f) {
+  pdl_wait();
   if (f.ks->done) return;
   double s0 = 0.0, s1 = 0.0;
   for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < n; r += gridDim.x * blockDim.x) {
@@ -832,7 +844,7 @@ void launch_coarse_solve(const CoarseSolve &cs, const T *X, const double *yprim,
   count_launch();
   launch_symv_rows<T>(cs.np, X, cs.ld_x, c, z, 0, done, s);
   for (int it = 0; it < cs.nref; ++it) {
-    k_coarse_resid<<<ceil_div(cs.np, 8), 256, 0, s>>>(cs.np, cs.sptr, cs.scol, cs.sval, c, z, rho, done);
+    launch_pdl(k_coarse_resid, ceil_div(cs.np, 8), 256, 0, s, cs.np, cs.sptr, cs.scol, cs.sval, c, z, rho, done);
     count_launch();
     launch_symv_rows<T>(cs.np, X, cs.ld_x, rho, z, 1, done, s);
   }
@@ -849,40 +861,40 @@ void launch_small_gemm(int ntasks, int max_n, const GemmTask *tasks, const T *A,
 void launch_gather_sum_dot(int n, const int *ptr, const int *idx, const double *src, double *y, int zero,
                            const DotFuse &f, cudaStream_t s) {
   if (n == 0) return;
-  k_gather_sum_dot<<<std::min(ceil_div(n, 256), kRedBlocks), 256, 0, s>>>(n, ptr, idx, src, y, zero, f);
+  launch_pdl(k_gather_sum_dot, std::min(ceil_div(n, 256), kRedBlocks), 256, 0, s, n, ptr, idx, src, y, zero, f);
   count_launch();
 }
 void launch_spmv_dot(int n, const int *ptr, const int *col, const double *val, const double *x, double *y, int zero,
                      const DotFuse &f, cudaStream_t s) {
   if (n == 0) return;
-  k_spmv_dot<<<std::min(ceil_div(n, 256), kRedBlocks), 256, 0, s>>>(n, ptr, col, val, x, y, zero, f);
+  launch_pdl(k_spmv_dot, std::min(ceil_div(n, 256), kRedBlocks), 256, 0, s, n, ptr, col, val, x, y, zero, f);
   count_launch();
 }
 void launch_spmv(int n, const int *ptr, const int *col, const double *val, const double *x, double *y, int zero,
                  const int *done, cudaStream_t s) {
   if (n == 0) return;
-  k_spmv<<<GRID1(n)>>>(n, ptr, col, val, x, y, zero, done);
+  launch_pdl(k_spmv, ceil_div(n, 256), 256, 0, s, n, ptr, col, val, x, y, zero, done);
   count_launch();
 }
 
 void launch_gather_sum(int n, const int *ptr, const int *idx, const double *src, double *y, int zero, double alpha,
                        const double *addend, const int *done, cudaStream_t s, const CsrIn *add_csr) {
   if (n == 0) return;
-  k_gather_sum<<<GRID1(n)>>>(n, ptr, idx, src, y, zero, alpha, addend, done, add_csr ? *add_csr : CsrIn{});
+  launch_pdl(k_gather_sum, ceil_div(n, 256), 256, 0, s, n, ptr, idx, src, y, zero, alpha, addend, done, add_csr ? *add_csr : CsrIn{});
   count_launch();
 }
 
 void launch_jump(int nlt, int max_n, const LamTask *lt, const PairTask *pairs, const double *w, double *lam,
                  const int *done, cudaStream_t s) {
   if (nlt == 0) return;
-  k_jump<<<dim3(ceil_div(max_n, 128), nlt), 128, 0, s>>>(lt, pairs, w, lam, done);
+  launch_pdl(k_jump, dim3(ceil_div(max_n, 128), nlt), 128, 0, s, lt, pairs, w, lam, done);
   count_launch();
 }
 
 void launch_jump_t(int nwt, int max_n, const WTask *wt, const WEnt *ent, const double *lam, double *w,
                    const int *done, cudaStream_t s) {
   if (nwt == 0) return;
-  k_jump_t<<<dim3(ceil_div(max_n, 128), nwt), 128, 0, s>>>(wt, ent, lam, w, done);
+  launch_pdl(k_jump_t, dim3(ceil_div(max_n, 128), nwt), 128, 0, s, wt, ent, lam, w, done);
   count_launch();
 }
 
@@ -890,7 +902,7 @@ template <typename T>
 void launch_jump_dt(int nwt, int max_n, const WTask *wt, const WEnt *ent, const T *blk, const T *sinv,
                     const double *mu, double *w, const int *done, cudaStream_t s) {
   if (nwt == 0) return;
-  k_jump_dt<T><<<nwt, 256, 3 * sizeof(T) * max_n, s>>>(wt, ent, blk, sinv, mu, w, done);
+  launch_pdl(k_jump_dt<T>, nwt, 256, 3 * sizeof(T) * max_n, s, wt, ent, blk, sinv, mu, w, done);
   count_launch();
 }
 
@@ -898,7 +910,7 @@ template <typename T>
 void launch_jump_d(int nlt, int max_n, const LamTask *lt, const PairTask *pairs, const T *blk, const T *sinv,
                    const double *y, double *mu, const int *done, cudaStream_t s) {
   if (nlt == 0) return;
-  k_jump_d<T><<<nlt, 256, 6 * sizeof(T) * max_n, s>>>(lt, pairs, blk, sinv, y, mu, done);
+  launch_pdl(k_jump_d<T>, nlt, 256, 6 * sizeof(T) * max_n, s, lt, pairs, blk, sinv, y, mu, done);
   count_launch();
 }
 
@@ -968,16 +980,16 @@ void launch_pcg_beta(KrylovState *ks, const double *dots, double *hb, cudaStream
 }
 void launch_pcg_xr(int n, const KrylovState *ks, const double *p, const double *q, double *x, double *r,
                    cudaStream_t s) {
-  k_pcg_xr<<<std::max(1, std::min(ceil_div(n, 256), kRedBlocks)), 256, 0, s>>>(n, ks, p, q, x, r);
+  launch_pdl(k_pcg_xr, std::max(1, std::min(ceil_div(n, 256), kRedBlocks)), 256, 0, s, n, ks, p, q, x, r);
   count_launch();
 }
 void launch_pcg_p(int n, const KrylovState *ks, const double *z, double *p, cudaStream_t s) {
-  k_pcg_p<<<std::max(1, std::min(ceil_div(n, 256), kRedBlocks)), 256, 0, s>>>(n, ks, z, p);
+  launch_pdl(k_pcg_p, std::max(1, std::min(ceil_div(n, 256), kRedBlocks)), 256, 0, s, n, ks, z, p);
   count_launch();
 }
 void launch_pcg_dot_step(int n, int which, const double *a0, const double *b0, const double *a1, const double *b1,
                         double *partial, unsigned int *counter, KrylovState *ks, double *hist, cudaStream_t s) {
-  k_pcg_dot_step<<<kRedBlocks, 256, 0, s>>>(n, which, a0, b0, a1, b1, partial, counter, ks, hist);
+  launch_pdl(k_pcg_dot_step, kRedBlocks, 256, 0, s, n, which, a0, b0, a1, b1, partial, counter, ks, hist);
   count_launch();
 }
 
@@ -1023,6 +1035,7 @@ template void launch_copy<double, float>(int, long long, const CopyTask *, const
 // step return at once when `stop` is set (converged, diverged or at maxit).
 __global__ void k_multidot(int n, int k, const double *__restrict__ V, const double *__restrict__ z,
                            double *__restrict__ partial, const GmresState *__restrict__ gs) {
+  pdl_wait();
   if (gs->stop) return;
   __shared__ double sh[32];
   const int q = blockIdx.y;
@@ -1036,6 +1049,7 @@ __global__ void k_multidot(int n, int k, const double *__restrict__ V, const dou
 // h[q] (+)= sum of the partials of dot q, q < k (fixed order)
 __global__ void k_multidot_fin(int k, int nblk, const double *__restrict__ partial, double *__restrict__ h, int add,
                                const GmresState *__restrict__ gs) {
+  pdl_wait();
   if (gs->stop) return;
   const int q = threadIdx.x;
   if (q >= k) return;
@@ -1047,6 +1061,7 @@ __global__ void k_multidot_fin(int k, int nblk, const double *__restrict__ parti
 // z -= sum_q c[q] V_q  (c = the projections just computed)
 __global__ void k_orth_sub(int n, int k, const double *__restrict__ V, const double *__restrict__ c,
                            double *__restrict__ z, const GmresState *__restrict__ gs) {
+  pdl_wait();
   if (gs->stop) return;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     double acc = z[i];
@@ -1058,6 +1073,7 @@ __global__ void k_orth_sub(int n, int k, const double *__restrict__ V, const dou
 // column j of H from (h1 + h2, ||z||), Givens rotations, residual estimate, stop test
 __global__ void k_gmres_rot(GmresState *__restrict__ gs, const double *__restrict__ h1, const double *__restrict__ h2,
                             const double *__restrict__ zz, int j) {
+  pdl_wait();
   if (gs->stop) return;
   const int m = gs->restart;
   double *H = gs->H;
@@ -1093,6 +1109,7 @@ __global__ void k_gmres_rot(GmresState *__restrict__ gs, const double *__restric
 // stop are never read: the update uses only the first gs->j basis vectors.
 __global__ void k_gmres_scale(int n, const double *__restrict__ z, double *__restrict__ vout,
                               const GmresState *__restrict__ gs) {
+  pdl_wait();
   const double inv = gs->hn > 0.0 ? 1.0 / gs->hn : 0.0;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) vout[i] = z[i] * inv;
 }
@@ -1140,16 +1157,16 @@ __global__ void k_gmres_begin(GmresState *__restrict__ gs, const double *__restr
 void launch_gmres_step(int n, int j, double *V, double *z, double *partial, double *h1, double *h2, double *zz,
                        GmresState *gs, cudaStream_t s) {
   const int nblk = 32;
-  k_multidot<<<dim3(nblk, j + 1), 256, 0, s>>>(n, j + 1, V, z, partial, gs);
-  k_multidot_fin<<<1, 64, 0, s>>>(j + 1, nblk, partial, h1, 0, gs);
-  k_orth_sub<<<std::max(1, std::min(ceil_div(n, 256), kRedBlocks)), 256, 0, s>>>(n, j + 1, V, h1, z, gs);
-  k_multidot<<<dim3(nblk, j + 1), 256, 0, s>>>(n, j + 1, V, z, partial, gs);
-  k_multidot_fin<<<1, 64, 0, s>>>(j + 1, nblk, partial, h2, 0, gs);
-  k_orth_sub<<<std::max(1, std::min(ceil_div(n, 256), kRedBlocks)), 256, 0, s>>>(n, j + 1, V, h2, z, gs);
-  k_multidot<<<dim3(nblk, 1), 256, 0, s>>>(n, 1, z, z, partial, gs);
-  k_multidot_fin<<<1, 64, 0, s>>>(1, nblk, partial, zz, 0, gs);
-  k_gmres_rot<<<1, 1, 0, s>>>(gs, h1, h2, zz, j);
-  k_gmres_scale<<<std::max(1, std::min(ceil_div(n, 256), kRedBlocks)), 256, 0, s>>>(n, z, V + (long long)(j + 1) * n,
+  launch_pdl(k_multidot, dim3(nblk, j + 1), 256, 0, s, n, j + 1, V, z, partial, gs);
+  launch_pdl(k_multidot_fin, 1, 64, 0, s, j + 1, nblk, partial, h1, 0, gs);
+  launch_pdl(k_orth_sub, std::max(1, std::min(ceil_div(n, 256), kRedBlocks)), 256, 0, s, n, j + 1, V, h1, z, gs);
+  launch_pdl(k_multidot, dim3(nblk, j + 1), 256, 0, s, n, j + 1, V, z, partial, gs);
+  launch_pdl(k_multidot_fin, 1, 64, 0, s, j + 1, nblk, partial, h2, 0, gs);
+  launch_pdl(k_orth_sub, std::max(1, std::min(ceil_div(n, 256), kRedBlocks)), 256, 0, s, n, j + 1, V, h2, z, gs);
+  launch_pdl(k_multidot, dim3(nblk, 1), 256, 0, s, n, 1, z, z, partial, gs);
+  launch_pdl(k_multidot_fin, 1, 64, 0, s, 1, nblk, partial, zz, 0, gs);
+  launch_pdl(k_gmres_rot, 1, 1, 0, s, gs, h1, h2, zz, j);
+  launch_pdl(k_gmres_scale, std::max(1, std::min(ceil_div(n, 256), kRedBlocks)), 256, 0, s, n, z, V + (long long)(j + 1) * n,
                                                                                    gs);
   count_launch(10);
 }
@@ -1157,7 +1174,7 @@ void launch_gmres_step(int n, int j, double *V, double *z, double *partial, doub
 void launch_gmres_begin(int n, const double *r, double *v0, GmresState *gs, const double *rr, int first,
                         cudaStream_t s) {
   k_gmres_begin<<<1, 1, 0, s>>>(gs, rr, first);
-  k_gmres_scale<<<std::max(1, std::min(ceil_div(n, 256), kRedBlocks)), 256, 0, s>>>(n, r, v0, gs);
+  launch_pdl(k_gmres_scale, std::max(1, std::min(ceil_div(n, 256), kRedBlocks)), 256, 0, s, n, r, v0, gs);
   count_launch(2);
 }
 

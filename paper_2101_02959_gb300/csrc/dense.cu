@@ -556,6 +556,7 @@ template <typename T>
 __global__ void __launch_bounds__(256) k_gemv(const GemvDesc *__restrict__ tasks, const T *__restrict__ A,
                                               const double *__restrict__ x, const int *__restrict__ xidx,
                                               double *__restrict__ y, double alpha, const int *__restrict__ done) {
+  pdl_wait();
   if (done && *done) return;
   const GemvDesc t = tasks[blockIdx.y];
   const int rbeg = blockIdx.x * kGemvRows;
@@ -613,6 +614,7 @@ __global__ void __launch_bounds__(256) k_symv_batched(const SymvTask *__restrict
                                                       const double *__restrict__ x, const int *__restrict__ xidx,
                                                       double *__restrict__ y, double alpha, const int *__restrict__ done,
                                                       T *__restrict__ scratch, int *__restrict__ counter, int ld_scr) {
+  pdl_wait();
   if (done && *done) return;
   using VT = typename Vec16<T>::V;
   constexpr int VN = Vec16<T>::N;
@@ -798,7 +800,7 @@ void launch_symv_batched(int ntasks, int max_n, const SymvTask *d_tasks, const f
                          const int *xidx, double *y, double alpha, const int *done, float *scratch, int *counter,
                          int ld_scr, cudaStream_t s) {
   if (ntasks == 0 || max_n == 0) return;
-  k_symv_batched<float><<<ntasks, 256, symv_smem<float>(max_n), s>>>(d_tasks, A, x, xidx, y, alpha, done, scratch,
+  launch_pdl(k_symv_batched<float>, ntasks, 256, symv_smem<float>(max_n), s, d_tasks, A, x, xidx, y, alpha, done, scratch,
                                                                     counter, ld_scr);
   count_launch();
 }
@@ -869,6 +871,7 @@ __global__ void __launch_bounds__(256) k_symv_fix(const SymvTask *__restrict__ t
                                                   const int *__restrict__ xidx, double *__restrict__ y, double alpha,
                                                   const int *__restrict__ done, double *__restrict__ scratch,
                                                   int *__restrict__ counter, int ld_scr) {
+  pdl_wait();
   if (done && *done) return;
   const SymvTask t = tasks[blockIdx.x];
   const int S = t.nparts, sidx = t.part;
@@ -1006,7 +1009,7 @@ void launch_symv_fix(int ntasks, int max_n, const SymvTask *d_tasks, const int2 
                      const int *xidx, double *y, double alpha, const int *done, double *scratch, int *counter,
                      int ld_scr, cudaStream_t s) {
   if (ntasks == 0 || max_n == 0) return;
-  k_symv_fix<<<ntasks, 256, symv_fix_smem(max_n), s>>>(d_tasks, tiles, ex, x, xidx, y, alpha, done, scratch, counter,
+  launch_pdl(k_symv_fix, ntasks, 256, symv_fix_smem(max_n), s, d_tasks, tiles, ex, x, xidx, y, alpha, done, scratch, counter,
                                                        ld_scr);
   count_launch();
 }
@@ -1064,6 +1067,7 @@ __global__ void __launch_bounds__(256) k_gemv_task(const GemvDesc *__restrict__ 
                                                    const double *__restrict__ x, const int *__restrict__ xidx,
                                                    double *__restrict__ y, double alpha,
                                                    const int *__restrict__ done) {
+  pdl_wait();
   if (done && *done) return;
   const GemvDesc t = tasks[blockIdx.x];
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1102,6 +1106,7 @@ __global__ void __launch_bounds__(256) k_gemv_t_task(const GemvDesc *__restrict_
                                                      const double *__restrict__ x, const int *__restrict__ xidx,
                                                      double *__restrict__ y, double alpha,
                                                      const int *__restrict__ done, const CsrIn csr) {
+  pdl_wait();
   if (done && *done) return;
   const GemvDesc t = tasks[blockIdx.x];
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1128,7 +1133,7 @@ template <typename T>
 void launch_gemv_task(int ntasks, int max_rows, int max_cols, const GemvDesc *d_tasks, const T *A, const double *x,
                       const int *xidx, double *y, double alpha, const int *done, cudaStream_t s) {
   if (ntasks == 0 || max_rows == 0) return;
-  k_gemv_task<T><<<ntasks, 256, sizeof(T) * (size_t)std::max(1, max_cols), s>>>(d_tasks, A, x, xidx, y, alpha, done);
+  launch_pdl(k_gemv_task<T>, ntasks, 256, sizeof(T) * (size_t)std::max(1, max_cols), s, d_tasks, A, x, xidx, y, alpha, done);
   count_launch();
 }
 
@@ -1138,8 +1143,10 @@ void launch_gemv_t_task(int ntasks, int max_rows, int max_cols, const GemvDesc *
                         const CsrIn *csr) {
   if (ntasks == 0 || max_cols == 0) return;
   const int threads = max_cols <= 128 ? 128 : 256;
-  k_gemv_t_task<T><<<ntasks, threads, sizeof(T) * (size_t)std::max(1, max_rows), s>>>(
-      d_tasks, A, x, xidx, y, alpha, done, csr ? *csr : CsrIn{});
+  const size_t sm = sizeof(T) * (size_t)std::max(1, max_rows);
+  const CsrIn c = csr ? *csr : CsrIn{};
+  // without csr this follows the join with the coarse solve's stream: an ordinary launch
+  launch_maybe_pdl(csr != nullptr, k_gemv_t_task<T>, ntasks, threads, sm, s, d_tasks, A, x, xidx, y, alpha, done, c);
   count_launch();
 }
 
@@ -1159,6 +1166,7 @@ template <typename T>
 __global__ void __launch_bounds__(256) k_symv_rows(int n, const T *__restrict__ A, int ld,
                                                    const double *__restrict__ x, double *__restrict__ y,
                                                    int accumulate, const int *__restrict__ done) {
+  pdl_wait();
   if (done && *done) return;
   using VT = typename Vec16<T>::V;
   constexpr int VN = Vec16<T>::N;
@@ -1232,7 +1240,7 @@ template <typename T>
 void launch_symv_rows(int n, const T *A, int ld, const double *x, double *y, int accumulate, const int *done,
                       cudaStream_t s) {
   if (n == 0) return;
-  k_symv_rows<T><<<ceil_div(n, 8), 256, sizeof(T) * (size_t)((n + 7) & ~7), s>>>(n, A, ld, x, y, accumulate, done);
+  launch_pdl(k_symv_rows<T>, ceil_div(n, 8), 256, sizeof(T) * (size_t)((n + 7) & ~7), s, n, A, ld, x, y, accumulate, done);
   count_launch();
 }
 
@@ -1242,7 +1250,7 @@ void launch_gemv(int ntasks, int max_rows, int max_cols, const GemvDesc *d_tasks
   if (ntasks == 0 || max_rows == 0) return;
   dim3 g(ceil_div(max_rows, kGemvRows), ntasks);
   const size_t sm = sizeof(T) * (size_t)std::max(1, max_cols);
-  k_gemv<T><<<g, 256, sm, s>>>(d_tasks, A, x, xidx, y, alpha, done);
+  launch_pdl(k_gemv<T>, g, 256, sm, s, d_tasks, A, x, xidx, y, alpha, done);
   count_launch();
 }
 
