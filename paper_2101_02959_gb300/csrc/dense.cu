@@ -43,221 +43,128 @@ template <> struct Vec16<double> {
   __device__ static void axpy(double *acc, const double2 a, double s) { acc[0] += a.x * s; acc[1] += a.y * s; }
 };
 
-// ---- 32 x 32 Cholesky in one warp: lane r holds row r in registers ------------
-// Columns c < wb are eliminated (pivot broadcast by shuffle, scaled column, rank-1
-// update of the rows below); rows and columns from wb on must hold the identity.
-template <typename T>
-__device__ __forceinline__ void warp_chol32(T (&a)[32], int lane, int wb, bool &bad) {
-#pragma unroll
-  for (int c = 0; c < 32; ++c) {
-    if (c < wb) {  // uniform across the warp
-      T piv = __shfl_sync(0xffffffffu, a[c], c);
-      if (!(piv > T(0))) { bad = true; piv = T(1); }
-      // the hardware estimate: relative error a few units in the last place, the level of
-      // FP32 rounding in the factors
-      const T inv = rsqrtf(piv), sd = piv * inv;
-      a[c] = (lane == c) ? sd : a[c] * inv;  // rows above c hold 0 here
-#pragma unroll
-      for (int t = c + 1; t < 32; ++t) {
-        const T lt = __shfl_sync(0xffffffffu, a[c], t);
-        if (lane >= t) a[t] -= a[c] * lt;
-      }
-    }
-  }
-}
-
-// ---- outer panel: partial Cholesky of the columns [K0, K0 + w), w <= kPW ---------
-// Two launches per outer panel.  The diagonal launch (ROWS = false, one CTA per
-// matrix) stages the w x w diagonal block (lower triangle, identity outside w) in
-// shared memory and factors it 32 columns at a time: warp 0 factors the 32 x 32
-// diagonal sub-block in registers, one thread per remaining row solves
-// x L_bb^T = a, and all threads apply the rank-32 update to the remaining columns
-// (4 x 4 register tiles over a transposed copy of the solved columns).  It writes
-// L_11 in place and the factored 32 x 32 diagonal sub-blocks to the block store
-// (slots dblk + K0 / 32 + q).  The rows launch (ROWS = true) then solves the rows
-// below, RB per CTA, the same way, reading the finished L_11 one 32-column slice at
-// a time instead of factoring it.
-constexpr int kPW = kEnginePanel;  // outer panel width
+// ---- rows below a 128-column panel: L_21 = A_21 L_11^-T (FP32) ----------------------
+// The diagonal block is factored already (k_diag128).  RB rows per CTA, staged in shared memory; 32
+// columns at a time: one thread per row solves x L_bb^T = a, then all threads apply the rank-32 update
+// to the remaining columns (4 x 4 register tiles over a transposed copy of the solved columns), reading
+// the finished L_11 one 32-column slice at a time.  Rows: those the band lets the panel reach.
+constexpr int kPW = kEnginePanel;  // panel width
 constexpr int kLDP = kPW + 4;      // row stride of the staged panel (16-byte aligned rows)
-template <typename T> struct PanelRows;
-template <> struct PanelRows<float> { static constexpr int RB = 128; };
+constexpr int kPanelRB = 128, kPanelNR = kPW + kPanelRB;
+constexpr size_t kPanelSmem = sizeof(float) * ((size_t)kPanelRB * kLDP + 32 * kPanelNR + 32 * 32 + 32);
 
-template <typename T, bool ROWS>
-constexpr size_t bigpanel_smem() {
-  constexpr int RB = PanelRows<T>::RB, NR = kPW + RB, NS = ROWS ? RB : kPW;
-  return sizeof(T) * ((size_t)NS * kLDP + 32 * NR + 32 * 32 + 32);
-}
-
-template <typename T, bool ROWS>
-__global__ void __launch_bounds__(256, 2) k_bigpanel(const MatDesc *__restrict__ desc, T *__restrict__ base, int K0,
-                                                     int *__restrict__ err, T *__restrict__ store) {
-  constexpr int RB = PanelRows<T>::RB, NR = kPW + RB;
-  constexpr int NS = ROWS ? RB : kPW;         // staged rows
-  constexpr int OWN0 = ROWS ? 0 : kPW;        // staged index of the first own row (rows launch only)
-  using VT = typename Vec16<T>::V;
-  constexpr int VN = Vec16<T>::N, VPP = kPW / VN;  // vectors per staged row
+__global__ void __launch_bounds__(256, 2) k_panel_rows(const MatDesc *__restrict__ desc, float *__restrict__ base,
+                                                       int K0) {
+  constexpr int RB = kPanelRB, NR = kPanelNR, VPP = kPW / 4;  // VPP: vectors per staged row
   const MatDesc d = desc[blockIdx.y];
   if (K0 >= d.e) return;
   const int w = min(kPW, d.e - K0);
-  // rows launch: the rows below the panel that it reaches (interior rows up to the band)
   const BandRows br = band_rows(d, K0 + w, K0 + w);
   const int v0 = blockIdx.x * RB;
-  if (ROWS && v0 >= br.nv) return;
-  const int nrows = ROWS ? min(RB, br.nv - v0) : 0;
-  T *A = base + d.off;
+  if (v0 >= br.nv) return;
+  const int nrows = min(RB, br.nv - v0);
+  float *A = base + d.off;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  T *P = reinterpret_cast<T *>(smem_raw);  // [NS][kLDP]: (diagonal rows,) own rows
-  T *PT = P + NS * kLDP;                   // [32][NR]: the current 32 columns, transposed (row p of the panel)
-  T *Lt = PT + 32 * NR;                    // [32][32]: Lt[c][t] = L_bb[t][c]
-  T *rd = Lt + 32 * 32;                    // [32]: 1 / L_bb[c][c]
+  float *P = reinterpret_cast<float *>(smem_raw);  // [RB][kLDP] own rows
+  float *PT = P + RB * kLDP;                       // [32][NR]: 32 columns, transposed (L_11 rows, then own)
+  float *Lt = PT + 32 * NR;                        // [32][32]: Lt[c][t] = L_bb[t][c]
+  float *rd = Lt + 32 * 32;                        // [32]: 1 / L_bb[c][c]
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  // panel row p (diagonal rows p < kPW, own rows kPW + q) -> staged row
-  auto prow = [&](int p) { return P + (p - kPW + OWN0) * kLDP; };
-  // ---- stage: kBatch vector loads in flight per thread and batch
-  constexpr int kVec = NS * VPP, kBatch = 8;
+  // stage: kBatch vector loads in flight per thread and batch
+  constexpr int kVec = RB * VPP, kBatch = 8;
   for (int base_i = 0; base_i < kVec; base_i += 256 * kBatch) {
-    VT buf[kBatch];
+    float4 buf[kBatch];
 #pragma unroll
     for (int u = 0; u < kBatch; ++u) {
-      const int idx = base_i + tid + 256 * u;
-      const int sr = idx / VPP, cv = idx % VPP;
-      const bool diag = !ROWS && sr < kPW;
-      const bool ok = idx < kVec && cv * VN < w && (diag ? sr < w : sr - OWN0 < nrows);
-      const long long grow = diag ? K0 + sr : (ok ? br.row(v0 + sr - OWN0) : 0);
-      buf[u] = ok ? *reinterpret_cast<const VT *>(A + grow * d.ld + K0 + cv * VN) : VT{};
+      const int idx = base_i + tid + 256 * u, sr = idx / VPP, cv = idx % VPP;
+      const bool ok = idx < kVec && cv * 4 < w && sr < nrows;
+      buf[u] = ok ? *reinterpret_cast<const float4 *>(A + (long long)br.row(v0 + sr) * d.ld + K0 + cv * 4) : float4{};
     }
 #pragma unroll
     for (int u = 0; u < kBatch; ++u) {
-      const int idx = base_i + tid + 256 * u;
-      const int sr = idx / VPP, cv = idx % VPP;
+      const int idx = base_i + tid + 256 * u, sr = idx / VPP, cv = idx % VPP;
       if (idx < kVec) {
-        const bool diag = !ROWS && sr < kPW;
-        VT o;
-#pragma unroll
-        for (int q = 0; q < VN; ++q) {
-          const int j = cv * VN + q;
-          const T e = Vec16<T>::get(buf[u], q);
-          if (diag) Vec16<T>::set(o, q, (sr < w && j < w && j <= sr) ? e : (j == sr ? T(1) : T(0)));
-          else Vec16<T>::set(o, q, (sr - OWN0 < nrows && j < w) ? e : T(0));
-        }
-        *reinterpret_cast<VT *>(P + sr * kLDP + cv * VN) = o;
+        float4 o = buf[u];
+        if (cv * 4 + 1 >= w) o.y = 0.f;
+        if (cv * 4 + 2 >= w) o.z = 0.f;
+        if (cv * 4 + 3 >= w) o.w = 0.f;
+        *reinterpret_cast<float4 *>(P + sr * kLDP + cv * 4) = o;
       }
     }
   }
-  bool bad = false;
   const int nbk = ceil_div(w, 32);
   for (int bq = 0; bq < nbk; ++bq) {
     const int c0 = 32 * bq, wb = min(32, w - c0);
-    const int nbelow = max(0, w - c0 - 32);  // diagonal-block rows below the sub-block
+    const int nbelow = max(0, w - c0 - 32);  // L_11 rows below the sub-block
     __syncthreads();
     if (wid == 0) {
-      T a[32];
-      {
-        const T *src = ROWS ? A + (long long)(K0 + c0 + (lane < wb ? lane : 0)) * d.ld + K0 + c0
-                            : P + (c0 + lane) * kLDP + c0;
+      const float *src = A + (long long)(K0 + c0 + (lane < wb ? lane : 0)) * d.ld + K0 + c0;
+      float dg = 1.f;
 #pragma unroll
-        for (int i = 0; i < 32 / VN; ++i) {
-          const bool rd_ok = !ROWS || (lane < wb && i * VN <= lane);
-          const VT v = rd_ok ? *reinterpret_cast<const VT *>(src + i * VN) : VT{};
+      for (int i = 0; i < 8; ++i) {
+        const float4 v = lane < wb && i * 4 <= lane ? *reinterpret_cast<const float4 *>(src + i * 4) : float4{};
 #pragma unroll
-          for (int q = 0; q < VN; ++q) {
-            const int t = i * VN + q;
-            a[t] = (lane < wb && t <= lane) ? Vec16<T>::get(v, q) : (t == lane ? T(1) : T(0));
-          }
+        for (int q = 0; q < 4; ++q) {
+          const int t = i * 4 + q;
+          const float e = (lane < wb && t <= lane) ? Vec16<float>::get(v, q) : (t == lane ? 1.f : 0.f);
+          if (t == lane) dg = e;
+          Lt[t * 32 + lane] = e;
         }
       }
-      if (!ROWS) warp_chol32(a, lane, wb, bad);
-      T dg = T(1);
-#pragma unroll
-      for (int t = 0; t < 32; ++t) {
-        const T v = (t <= lane) ? a[t] : T(0);
-        if (t == lane) dg = v;
-        if (!ROWS) P[(c0 + lane) * kLDP + c0 + t] = v;
-        Lt[t * 32 + lane] = v;
-      }
-      rd[lane] = T(1) / dg;
-      if (!ROWS) {
-        T *sb = store + ((long long)d.dblk + K0 / kNB + bq) * kNB * kNB + lane * kNB;
-#pragma unroll
-        for (int i = 0; i < 32 / VN; ++i) {
-          VT o;
-#pragma unroll
-          for (int q = 0; q < VN; ++q) Vec16<T>::set(o, q, (i * VN + q <= lane) ? a[i * VN + q] : T(0));
-          *reinterpret_cast<VT *>(sb + i * VN) = o;
-        }
-      }
-    } else if (ROWS) {
+      rd[lane] = 1.f / dg;
+    } else {
       // the finished L_11 rows below the sub-block, columns [c0, c0 + 32), transposed
-      for (int idx = tid - 32; idx < nbelow * (32 / VN); idx += 256 - 32) {
-        const int r = idx / (32 / VN), cv = idx % (32 / VN), p = c0 + 32 + r;
-        const VT v = *reinterpret_cast<const VT *>(A + (long long)(K0 + p) * d.ld + K0 + c0 + cv * VN);
+      for (int idx = tid - 32; idx < nbelow * 8; idx += 256 - 32) {
+        const int r = idx / 8, cv = idx % 8, p = c0 + 32 + r;
+        const float4 v = *reinterpret_cast<const float4 *>(A + (long long)(K0 + p) * d.ld + K0 + c0 + cv * 4);
 #pragma unroll
-        for (int q = 0; q < VN; ++q) PT[(cv * VN + q) * NR + p] = Vec16<T>::get(v, q);
+        for (int q = 0; q < 4; ++q) PT[(cv * 4 + q) * NR + p] = Vec16<float>::get(v, q);
       }
     }
     __syncthreads();
-    // rows below the sub-block: (diagonal rows [c0 + 32, w),) then the own rows
-    const int ndiag = ROWS ? 0 : nbelow;
-    const int nsolve = ndiag + nrows;
-    for (int qr = tid; qr < nsolve; qr += 256) {
-      const int p = qr < ndiag ? c0 + 32 + qr : kPW + (qr - ndiag);
-      T x[32];
-      T *src = prow(p) + c0;
+    if (tid < nrows) {
+      float x[32];
+      float *src = P + tid * kLDP + c0;
 #pragma unroll
-      for (int i = 0; i < 32 / VN; ++i) {
-        const VT v = *reinterpret_cast<const VT *>(src + i * VN);
+      for (int i = 0; i < 8; ++i) {
+        const float4 v = *reinterpret_cast<const float4 *>(src + i * 4);
 #pragma unroll
-        for (int q = 0; q < VN; ++q) x[i * VN + q] = Vec16<T>::get(v, q);
+        for (int q = 0; q < 4; ++q) x[i * 4 + q] = Vec16<float>::get(v, q);
       }
 #pragma unroll
       for (int c = 0; c < 32; ++c) {
         x[c] *= rd[c];
 #pragma unroll
-        for (int i = (c + 1) / VN; i < 32 / VN; ++i) {
-          const VT lv = *reinterpret_cast<const VT *>(&Lt[c * 32 + i * VN]);
+        for (int i = (c + 1) / 4; i < 8; ++i) {
+          const float4 lv = *reinterpret_cast<const float4 *>(&Lt[c * 32 + i * 4]);
 #pragma unroll
-          for (int q = 0; q < VN; ++q)
-            if (i * VN + q > c) x[i * VN + q] -= Vec16<T>::get(lv, q) * x[c];
+          for (int q = 0; q < 4; ++q)
+            if (i * 4 + q > c) x[i * 4 + q] -= Vec16<float>::get(lv, q) * x[c];
         }
       }
 #pragma unroll
-      for (int i = 0; i < 32 / VN; ++i) {
-        VT o;
+      for (int i = 0; i < 8; ++i)
+        *reinterpret_cast<float4 *>(src + i * 4) = make_float4(x[4 * i], x[4 * i + 1], x[4 * i + 2], x[4 * i + 3]);
 #pragma unroll
-        for (int q = 0; q < VN; ++q) Vec16<T>::set(o, q, x[i * VN + q]);
-        *reinterpret_cast<VT *>(src + i * VN) = o;
-      }
-#pragma unroll
-      for (int t = 0; t < 32; ++t) PT[t * NR + p] = x[t];
+      for (int t = 0; t < 32; ++t) PT[t * NR + kPW + tid] = x[t];
     }
     __syncthreads();
-    // rank-32 update of the panel columns [c0 + 32, w): rows as above (lower part for
-    // the diagonal rows), 4 x 4 tiles; tiles straddle no part (both parts 4-aligned)
+    // rank-32 update of the panel columns [c0 + 32, w), 4 x 4 tiles
     const int jb = c0 + 32, ncol = w - jb;
     if (ncol > 0) {
-      const int nd4 = (ndiag + 3) / 4, nr4 = (nrows + 3) / 4, nc4 = (ncol + 3) / 4;
-      const int ntiles = (nd4 + nr4) * nc4;
-      for (int mt = tid; mt < ntiles; mt += 256) {
-        const int rq = mt / nc4, cq = mt % nc4;
-        const bool own = rq >= nd4;
-        const int p0 = own ? kPW + 4 * (rq - nd4) : jb + 4 * rq;
-        const int j0 = jb + 4 * cq;
-        if (!own && p0 + 3 < j0) continue;  // strictly above the diagonal
-        T acc[4][4];
+      const int nr4 = (nrows + 3) / 4, nc4 = (ncol + 3) / 4;
+      for (int mt = tid; mt < nr4 * nc4; mt += 256) {
+        const int r0 = 4 * (mt / nc4), j0 = jb + 4 * (mt % nc4);
+        float acc[4][4];
 #pragma unroll
         for (int i = 0; i < 4; ++i)
 #pragma unroll
-          for (int j = 0; j < 4; ++j) acc[i][j] = T(0);
+          for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
 #pragma unroll 8
         for (int k = 0; k < 32; ++k) {
-          T av[4], bv[4];
-#pragma unroll
-          for (int i = 0; i < 4; i += VN) {
-            const VT x = *reinterpret_cast<const VT *>(&PT[k * NR + p0 + i]);
-            const VT y = *reinterpret_cast<const VT *>(&PT[k * NR + j0 + i]);
-#pragma unroll
-            for (int q = 0; q < VN; ++q) { av[i + q] = Vec16<T>::get(x, q); bv[i + q] = Vec16<T>::get(y, q); }
-          }
+          const float4 x = *reinterpret_cast<const float4 *>(&PT[k * NR + kPW + r0]);
+          const float4 y = *reinterpret_cast<const float4 *>(&PT[k * NR + j0]);
+          const float av[4] = {x.x, x.y, x.z, x.w}, bv[4] = {y.x, y.y, y.z, y.w};
 #pragma unroll
           for (int i = 0; i < 4; ++i)
 #pragma unroll
@@ -265,9 +172,8 @@ __global__ void __launch_bounds__(256, 2) k_bigpanel(const MatDesc *__restrict__
         }
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-          const int p = p0 + i;
-          if (own ? (p - kPW >= nrows) : (p >= w)) continue;
-          T *row = prow(p);
+          if (r0 + i >= nrows) continue;
+          float *row = P + (r0 + i) * kLDP;
 #pragma unroll
           for (int j = 0; j < 4; ++j)
             if (j0 + j < w) row[j0 + j] -= acc[i][j];
@@ -275,24 +181,16 @@ __global__ void __launch_bounds__(256, 2) k_bigpanel(const MatDesc *__restrict__
       }
     }
   }
-  if (bad && tid == 0) atomicOr(err, DEV_ERR_NOT_SPD);
   __syncthreads();
-  // own rows back to the matrix; the diagonal launch also writes L_11 (lower part)
   for (int idx = tid; idx < nrows * VPP; idx += 256) {
     const int q = idx / VPP, cv = idx % VPP;
-    if (cv * VN >= w) continue;
-    const T *src = P + (OWN0 + q) * kLDP + cv * VN;
-    T *dst = A + (long long)br.row(v0 + q) * d.ld + K0 + cv * VN;
-    if (cv * VN + VN <= w) {
-      *reinterpret_cast<VT *>(dst) = *reinterpret_cast<const VT *>(src);
+    if (cv * 4 >= w) continue;
+    const float *src = P + q * kLDP + cv * 4;
+    float *dst = A + (long long)br.row(v0 + q) * d.ld + K0 + cv * 4;
+    if (cv * 4 + 4 <= w) {
+      *reinterpret_cast<float4 *>(dst) = *reinterpret_cast<const float4 *>(src);
     } else {
-      for (int u = 0; cv * VN + u < w; ++u) dst[u] = src[u];
-    }
-  }
-  if (!ROWS) {
-    for (int idx = tid; idx < w * w; idx += 256) {
-      const int i = idx / w, j = idx % w;
-      if (j <= i) A[(long long)(K0 + i) * d.ld + K0 + j] = P[i * kLDP + j];
+      for (int u = 0; cv * 4 + u < w; ++u) dst[u] = src[u];
     }
   }
 }
@@ -472,11 +370,9 @@ void engine_partial_cholesky(const EngineShape &sh, const MatDesc *d_desc, T *ba
         launch_diag<T>(d_desc, base, k0, sh.count, d_err, store, pinv, s);
         launch_update<T>(d_desc, base, Upd64{3, k0, 0, PW, 0, 0}, max_below, PW, sh.count, ws, d_err, s, pinv);
       } else if constexpr (!f64) {
-        k_bigpanel<T, false><<<dim3(1, sh.count), 256, bigpanel_smem<T, false>(), s>>>(d_desc, base, k0, d_err, store);
-        count_launch();
+        launch_diag128(d_desc, base, k0, sh.count, d_err, store, s);
         if (max_below > 0) {
-          k_bigpanel<T, true><<<dim3(ceil_div(max_below, PanelRows<T>::RB), sh.count), 256, bigpanel_smem<T, true>(),
-                                s>>>(d_desc, base, k0, d_err, store);
+          k_panel_rows<<<dim3(ceil_div(max_below, kPanelRB), sh.count), 256, kPanelSmem, s>>>(d_desc, base, k0);
           count_launch();
         }
       }
@@ -1423,10 +1319,7 @@ size_t dense_smem_limit() { return 200 * 1024; }
 bool dense_configure() {
   const int lim = (int)dense_smem_limit();
   bool ok = true;
-  ok &= cudaFuncSetAttribute(k_bigpanel<float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)bigpanel_smem<float, false>()) == cudaSuccess;
-  ok &= cudaFuncSetAttribute(k_bigpanel<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)bigpanel_smem<float, true>()) == cudaSuccess;
+  ok &= cudaFuncSetAttribute(k_panel_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPanelSmem) == cudaSuccess;
   ok &= cudaFuncSetAttribute(k_trsv<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim) == cudaSuccess;
   ok &= cudaFuncSetAttribute(k_trsv<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim) == cudaSuccess;
   ok &= cudaFuncSetAttribute(k_gemv<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim) == cudaSuccess;

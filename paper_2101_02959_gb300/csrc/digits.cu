@@ -586,20 +586,21 @@ __device__ __forceinline__ double recip(double p) {
   const double y = (double)__fdividef(1.f, (float)p), e = fma(-p, y, 1.0);
   return fma(y, fma(e, e, e), y);
 }
-__device__ __forceinline__ float recip(float p) { return 1.f / p; }
+// the hardware estimate: a few units in the last place, the level of FP32 rounding in the factors
+__device__ __forceinline__ float recip(float p) { return __fdividef(1.f, p); }
 
-// Lower Cholesky factor of the 32 x 32 block of P at (o, o) and its inverse into Y; warps 0-3.
+// Lower Cholesky factor of the 32 x 32 block P (row stride LP) and its inverse into Y (LY); warps 0-3.
 // Columns at and after the block's width hold the identity.  The owner of column c + 1 updates it
 // first, publishes it and arrives at the column's barrier before it makes the rest of step c's
 // updates, so that the others never wait for those; four column buffers and two barriers in turn keep
 // the steps apart.
-template <typename T>
-__device__ __forceinline__ void ldl_inv32(T *P, T *Y, int o, int s, int lane, T (*Lc)[2][32], T *piv, bool &bad) {
+template <int LP, int LY, typename T>
+__device__ __forceinline__ void ldl_inv32(T *P, T *Y, int s, int lane, T (*Lc)[2][32], T *piv, bool &bad) {
   T a[8], y[8];
 #pragma unroll
   for (int q = 0; q < 8; ++q) {
     const int t = 4 * q + s;
-    a[q] = t <= lane ? P[(o + lane) * kDLD + o + t] : T(0);
+    a[q] = t <= lane ? P[lane * LP + t] : T(0);
     y[q] = t == lane ? T(1) : T(0);
   }
   auto publish = [&](int c, T col) {  // column c, held by this warp
@@ -643,8 +644,8 @@ __device__ __forceinline__ void ldl_inv32(T *P, T *Y, int o, int s, int lane, T 
   for (int q = 0; q < 8; ++q) {
     const int t = 4 * q + s;
     const T rt = __shfl_sync(0xffffffffu, rs, t);
-    P[(o + lane) * kDLD + o + t] = lane < t ? T(0) : (lane == t ? pl * rs : a[q] * rt);
-    Y[(o + lane) * kDLD + o + t] = t <= lane ? y[q] * rs : T(0);
+    P[lane * LP + t] = lane < t ? T(0) : (lane == t ? pl * rs : a[q] * rt);
+    Y[lane * LY + t] = t <= lane ? y[q] * rs : T(0);
   }
 }
 
@@ -678,7 +679,7 @@ __global__ void __launch_bounds__(256) k_diag(const MatDesc *__restrict__ desc, 
   for (int h = 0; h < nbk; ++h) {
     const int o = 32 * h;
     __syncthreads();
-    if (warp < 4) ldl_inv32(P, Y, o, warp, lane, Lc, piv, bad);
+    if (warp < 4) ldl_inv32<kDLD, kDLD>(P + o * kDLD + o, Y + o * kDLD + o, warp, lane, Lc, piv, bad);
     __syncthreads();
     T *sb = store + ((long long)d.dblk + K0 / kNB + h) * kNB * kNB;
     for (int q = tid; q < 1024; q += 256) sb[q] = P[(o + (q >> 5)) * kDLD + o + (q & 31)];
@@ -744,6 +745,118 @@ __global__ void __launch_bounds__(256) k_diag(const MatDesc *__restrict__ desc, 
   }
 }
 
+// ---- FP32 diagonal block of a 128-column panel --------------------------------------
+// One CTA per matrix, 32 columns at a time: factor and inverse as above, the block's rows below by
+// that inverse (warp = four columns, lane = row), rank-32 update of the rest (4 x 4 tiles a thread).
+// A latency chain of 128 pivots: 44 us with one warp factoring and one thread per row substituting,
+// 33 us here; a coarse matrix of 2,600 unknowns runs 21 of these one after another.
+constexpr int kWP = kEnginePanel, kWLD = kWP + 1;
+constexpr size_t kDiag128Smem = sizeof(float) * (size_t)kWP * kWLD;
+
+__global__ void __launch_bounds__(256) k_diag128(const MatDesc *__restrict__ desc, float *__restrict__ base, int K0,
+                                                 int *__restrict__ err, float *__restrict__ store) {
+  const MatDesc d = desc[blockIdx.x];
+  if (K0 >= d.e) return;
+  const int w = min(kWP, d.e - K0);
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  float *P = reinterpret_cast<float *>(smem_raw);  // [128][129] the block, lower, identity past w
+  __shared__ float Y[32 * 33], Lc[4][2][32], piv[32];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  float *A = base + d.off + (long long)K0 * d.ld + K0;
+  for (int r0 = warp; r0 < kWP; r0 += 64) {  // eight rows in flight per warp
+    float v[8][4];
+#pragma unroll
+    for (int q = 0; q < 8; ++q)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const int r = r0 + 8 * q, j = 32 * c + lane;
+        v[q][c] = (r < w && j <= r) ? A[(long long)r * d.ld + j] : (r == j ? 1.f : 0.f);
+      }
+#pragma unroll
+    for (int q = 0; q < 8; ++q)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) P[(r0 + 8 * q) * kWLD + 32 * c + lane] = v[q][c];
+  }
+  bool bad = false;
+  const int nbk = ceil_div(w, 32), grp = 4 * (warp < 4 ? warp : 11 - warp);
+  for (int h = 0; h < nbk; ++h) {
+    const int o = 32 * h;
+    __syncthreads();
+    if (warp < 4) ldl_inv32<kWLD, 33>(P + o * kWLD + o, Y, warp, lane, Lc, piv, bad);
+    __syncthreads();
+    float *sb = store + ((long long)d.dblk + K0 / kNB + h) * kNB * kNB;
+    for (int q = tid; q < 1024; q += 256) sb[q] = P[(o + (q >> 5)) * kWLD + o + (q & 31)];
+    if (h + 1 == nbk) break;
+    const int nrb = nbk - h - 1;  // 32-row blocks below
+    float x[3][4];
+#pragma unroll
+    for (int b = 0; b < 3; ++b)
+#pragma unroll
+      for (int u = 0; u < 4; ++u) x[b][u] = 0.f;
+#pragma unroll 4
+    for (int k = 0; k < grp + 4; ++k) {  // Y lower: k <= column
+      float y[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) y[u] = Y[(grp + u) * 33 + k];
+#pragma unroll
+      for (int b = 0; b < 3; ++b) {
+        if (b < nrb) {
+          const float l = P[(o + 32 + 32 * b + lane) * kWLD + o + k];
+#pragma unroll
+          for (int u = 0; u < 4; ++u) x[b][u] += l * y[u];
+        }
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int b = 0; b < 3; ++b)
+      if (b < nrb)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) P[(o + 32 + 32 * b + lane) * kWLD + o + grp + u] = x[b][u];
+    __syncthreads();
+    // rows and columns from o + 32 on, lower 4 x 4 tiles
+    const int n4 = 8 * nrb, nt = n4 * (n4 + 1) / 2;
+    for (int t = tid; t < nt; t += 256) {
+      int ti = (int)((sqrtf(8.f * t + 1.f) - 1.f) * 0.5f);
+      while ((ti + 1) * (ti + 2) / 2 <= t) ++ti;
+      while (ti * (ti + 1) / 2 > t) --ti;
+      const int tj = t - ti * (ti + 1) / 2, r = o + 32 + 4 * ti, c = o + 32 + 4 * tj;
+      float a[4][4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) a[i][j] = 0.f;
+#pragma unroll 8
+      for (int k = 0; k < 32; ++k) {
+        float p[4], q[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          p[i] = P[(r + i) * kWLD + o + k];
+          q[i] = P[(c + i) * kWLD + o + k];
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) a[i][j] += p[i] * q[j];
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (r + i < w && c + j <= r + i) P[(r + i) * kWLD + c + j] -= a[i][j];
+    }
+  }
+  __syncthreads();
+  if (bad && lane == 0) atomicOr(err, DEV_ERR_NOT_SPD);
+  for (int r = warp; r < w; r += 8)
+    for (int j = lane; j <= r; j += 32) A[(long long)r * d.ld + j] = P[r * kWLD + j];
+}
+
+void launch_diag128(const MatDesc *d_desc, float *base, int K0, int count, int *err, float *store, cudaStream_t s) {
+  k_diag128<<<count, 256, kDiag128Smem, s>>>(d_desc, base, K0, err, store);
+  count_launch();
+}
+
 template <typename T>
 void launch_diag(const MatDesc *d_desc, T *base, int K0, int count, int *err, T *store, T *pinv, cudaStream_t s) {
   k_diag<T><<<count, 256, diag_smem<T>(), s>>>(d_desc, base, K0, err, store, pinv);
@@ -755,7 +868,10 @@ static bool configure() {
   return cudaFuncSetAttribute(k_update<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, update_smem<T>()) == cudaSuccess &&
          cudaFuncSetAttribute(k_diag<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)diag_smem<T>()) == cudaSuccess;
 }
-bool digits_configure() { return configure<float>() && configure<double>(); }
+bool digits_configure() {
+  return configure<float>() && configure<double>() &&
+         cudaFuncSetAttribute(k_diag128, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDiag128Smem) == cudaSuccess;
+}
 
 // Workspace of the digit planes of one matrix (rows x cols) and of a panel inverse.
 template <typename T>

@@ -99,7 +99,7 @@ struct EngineShape {
   std::vector<const int *> ifirst;  // host copies of MatDesc::ifirst (empty or nullptr: dense)
 };
 // The engine works through outer blocks of sh.ob columns: panels of kEnginePanel
-// columns (k_bigpanel), each followed by an update of the rest of its block, then
+// columns (k_diag128 and k_panel_rows, or k_diag and k_update), each followed by an update of the rest of its block, then
 // one long-K (K = ob) update of the trailing columns.  store: block store
 // receiving the factored kNB x kNB diagonal blocks L_kk; matrix b uses slots
 // [desc[b].dblk, desc[b].dblk + ceil(e_b / kNB)) (row-major, identity outside the last
@@ -128,6 +128,7 @@ void launch_product(const MatDesc *d_a, const T *A, const MatDesc *d_b, const T 
                     int max_n, const SliceWs &ws, int *err, cudaStream_t s);
 template <typename T>
 void launch_diag(const MatDesc *d_desc, T *base, int K0, int count, int *err, T *store, T *pinv, cudaStream_t s);
+void launch_diag128(const MatDesc *d_desc, float *base, int K0, int count, int *err, float *store, cudaStream_t s);
 
 // The same products for many small matrices: one CTA per task over all its rows (columns)
 template <typename T>
