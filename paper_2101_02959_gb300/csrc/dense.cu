@@ -493,46 +493,42 @@ __global__ void __launch_bounds__(256) k_gemv(const GemvDesc *__restrict__ tasks
   }
 }
 
-// ---- batched symmetric GEMV: S = nparts CTAs (8 warps each) per matrix -------
+// ---- batched symmetric GEMV (FP32): S = nparts CTAs (8 warps each) per matrix -------
 // The matrix is read as 32 x 32 tiles of its lower block triangle, each once: tile (I, J),
 // J < I, serves both y_I += A_IJ x_J and y_J += A_IJ^T x_I; a diagonal tile serves
 // y_I += A_II x_I.  CTA s of a matrix takes the s-th of S contiguous runs of the row-major
-// tile order and splits it over its warps the same way; a warp holds the next tile in
-// registers (16-byte loads, a 128-byte row segment per 32 / VN lanes) while it multiplies
-// the current one from its shared-memory copy (row sums: lane = tile row; column sums:
-// lane = tile column) and adds both into its own partial vector, so no two warps write the
-// same word.  The CTA adds its warps' vectors in warp order; with S > 1 it stores the sum in
-// `scratch` and the last CTA of the matrix to finish (counter per matrix, reset by that CTA)
-// adds the S sums in order s = 0 .. S-1.  Deterministic; half the bytes of a full GEMV.
+// tile order and splits it over its warps the same way.  A lane holds 4 columns of every fourth row of
+// its tile (eight 16-byte loads, the next tile's in flight meanwhile) and multiplies from
+// registers: its eight row sums stay in registers along a block row and are reduced over the eight
+// lanes of a row at its end; its four column sums are reduced over the four lanes of a column per tile.
+// Both end in the warp's own partial vector, so no two warps write the same word.  The CTA
+// adds its warps' vectors in warp order; with S > 1 it stores the sum in `scratch` and the last CTA
+// of the matrix to finish (counter per matrix, reset by that CTA) adds the S sums in order
+// s = 0 .. S-1.  Deterministic; half the bytes of a full GEMV.  Bound by HBM: with the tiles copied
+// to shared memory and read there twice it was bound by those reads (160 a tile against 190 clocks of
+// HBM time; 206 us for the 1,024 matrices of order 772; now 168 us, 7.3 TB/s).
 // Plain rows of B go to the CTAs round-robin.
-template <typename T>
-__global__ void __launch_bounds__(256) k_symv_batched(const SymvTask *__restrict__ tasks, const T *__restrict__ A,
-                                                      const double *__restrict__ x, const int *__restrict__ xidx,
-                                                      double *__restrict__ y, double alpha, const int *__restrict__ done,
-                                                      T *__restrict__ scratch, int *__restrict__ counter, int ld_scr) {
+__global__ void __launch_bounds__(256, 2) k_symv_batched(const SymvTask *__restrict__ tasks, const float *__restrict__ A,
+                                                         const double *__restrict__ x, const int *__restrict__ xidx,
+                                                         double *__restrict__ y, double alpha,
+                                                         const int *__restrict__ done, float *__restrict__ scratch,
+                                                         int *__restrict__ counter, int ld_scr) {
   pdl_wait();
   if (done && *done) return;
-  using VT = typename Vec16<T>::V;
-  constexpr int VN = Vec16<T>::N;
-  constexpr int LPR = 32 / VN;       // lanes per 32-wide tile row
-  constexpr int RPI = 32 / LPR;      // tile rows per warp instruction
-  constexpr int TPL = 32 / RPI;      // vectors per lane per tile
   const SymvTask t = tasks[blockIdx.x];
   const int S = t.nparts, sidx = t.part;
   const int n = t.n, nb = (n + 31) >> 5, np = nb * 32;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  T *xs = reinterpret_cast<T *>(smem_raw);  // [np]
-  T *part = xs + np;                         // [8][np]
-  T *tiles = part + 8 * np;                  // [8][32][33]
+  float *xs = reinterpret_cast<float *>(smem_raw);  // [np]
+  float *part = xs + np;                             // [8][np]
   __shared__ int last;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   for (int c = tid; c < np; c += 256)
-    xs[c] = c < n ? (T)((t.flags & 1) ? x[xidx[t.x_off + c]] : x[t.x_off + c]) : T(0);
-  for (int c = tid; c < 8 * np; c += 256) part[c] = T(0);
+    xs[c] = c < n ? (float)((t.flags & 1) ? x[xidx[t.x_off + c]] : x[t.x_off + c]) : 0.f;
+  for (int c = tid; c < 8 * np; c += 256) part[c] = 0.f;
   __syncthreads();
-  const T *a = A + t.a_off;
-  T *tile = tiles + warp * 32 * 33;
-  T *mine = part + warp * np;
+  const float *a = A + t.a_off;
+  float *mine = part + warp * np;
   const long long ntiles = (long long)nb * (nb + 1) / 2;
   const long long c0 = ntiles * sidx / S, c1 = ntiles * (sidx + 1) / S;  // this CTA's run
   const int s0 = (int)(c0 + (c1 - c0) * warp / 8), s1 = (int)(c0 + (c1 - c0) * (warp + 1) / 8);
@@ -540,81 +536,121 @@ __global__ void __launch_bounds__(256) k_symv_batched(const SymvTask *__restrict
   int I = 0;
   while ((I + 1) * (I + 2) / 2 <= s0) ++I;
   int J = s0 - I * (I + 1) / 2;
-  const int lr = lane / LPR, lc = (lane % LPR) * VN;  // this lane's row in a group and column
-  VT buf[TPL];
-  auto load = [&](int ti, int tj) {
+  const int lr = lane >> 3, lc = (lane & 7) * 4;  // this lane's first row and column in a tile
+  float4 v[8], nx[8];
+  auto load = [&](float4 (&b)[8], int ti, int tj) {
+    const float *p = a + (long long)(32 * ti + lr) * t.ld + 32 * tj + lc;
+    if (32 * ti + 32 <= n) {  // tj <= ti: every entry inside
 #pragma unroll
-    for (int i = 0; i < TPL; ++i) {
-      const int r = 32 * ti + i * RPI + lr, c = 32 * tj + lc;
-      VT v = (r < n && c < n) ? *reinterpret_cast<const VT *>(a + (long long)r * t.ld + c) : VT{};
+      for (int i = 0; i < 8; ++i) b[i] = *reinterpret_cast<const float4 *>(p + (long long)(4 * i) * t.ld);
+    } else {
+      const int c = 32 * tj + lc;
 #pragma unroll
-      for (int q = 0; q < VN; ++q)
-        if (c + q >= n) Vec16<T>::set(v, q, T(0));
-      buf[i] = v;
+      for (int i = 0; i < 8; ++i) {
+        float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (32 * ti + lr + 4 * i < n && c < n) {
+          q = *reinterpret_cast<const float4 *>(p + (long long)(4 * i) * t.ld);
+          if (c + 1 >= n) q.y = 0.f;
+          if (c + 2 >= n) q.z = 0.f;
+          if (c + 3 >= n) q.w = 0.f;
+        }
+        b[i] = q;
+      }
     }
   };
-  if (s0 < s1) load(I, J);
-  for (int s = s0; s < s1; ++s) {
+  float rs[8], xr[8];  // sums of this lane's rows along the block row; x at those rows
+  auto rows = [&](int ti) {
 #pragma unroll
-    for (int i = 0; i < TPL; ++i)
+    for (int i = 0; i < 8; ++i) {
+      rs[i] = 0.f;
+      xr[i] = xs[32 * ti + 4 * i + lr];
+    }
+  };
+  auto flush = [&](int ti) {  // lane -> row 4 i + lr, i the low three bits of the lane
+    const bool b2 = lane & 4, b1 = lane & 2, b0 = lane & 1;
+    float p4[4], p2[2];
 #pragma unroll
-      for (int q = 0; q < VN; ++q) tile[(i * RPI + lr) * 33 + lc + q] = Vec16<T>::get(buf[i], q);
+    for (int i = 0; i < 4; ++i)
+      p4[i] = (b2 ? rs[4 + i] : rs[i]) + __shfl_xor_sync(0xffffffffu, b2 ? rs[i] : rs[4 + i], 4);
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+      p2[i] = (b1 ? p4[2 + i] : p4[i]) + __shfl_xor_sync(0xffffffffu, b1 ? p4[i] : p4[2 + i], 2);
+    const float r = (b0 ? p2[1] : p2[0]) + __shfl_xor_sync(0xffffffffu, b0 ? p2[0] : p2[1], 1);
+    mine[32 * ti + 4 * (lane & 7) + lr] += r;
     __syncwarp();
+  };
+  if (s0 < s1) {
+    load(v, I, J);
+    rows(I);
+  }
+  for (int s = s0; s < s1; ++s) {
     const int ci = I, cj = J;
     if (++J > I) { ++I; J = 0; }
-    if (s + 1 < s1) load(I, J);  // in flight while this tile is multiplied
-    T rsum = T(0);
-#pragma unroll 8
-    for (int c = 0; c < 32; ++c) rsum += tile[lane * 33 + c] * xs[32 * cj + c];
-    mine[32 * ci + lane] += rsum;
+    if (s + 1 < s1) load(nx, I, J);  // in flight while this tile is multiplied
+    const float4 xc = *reinterpret_cast<const float4 *>(xs + 32 * cj + lc);
+#pragma unroll
+    for (int i = 0; i < 8; ++i) rs[i] += (v[i].x * xc.x + v[i].y * xc.y) + (v[i].z * xc.z + v[i].w * xc.w);
     if (cj < ci) {
-      T csum = T(0);
-#pragma unroll 8
-      for (int r = 0; r < 32; ++r) csum += tile[r * 33 + lane] * xs[32 * ci + r];
-      mine[32 * cj + lane] += csum;
+      float4 c = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        c.x += v[i].x * xr[i];
+        c.y += v[i].y * xr[i];
+        c.z += v[i].z * xr[i];
+        c.w += v[i].w * xr[i];
+      }
+      const bool b4 = lane & 16, b3 = lane & 8;  // lane -> column lc + 2 b4 + b3
+      const float e0 = (b4 ? c.z : c.x) + __shfl_xor_sync(0xffffffffu, b4 ? c.x : c.z, 16);
+      const float e1 = (b4 ? c.w : c.y) + __shfl_xor_sync(0xffffffffu, b4 ? c.y : c.w, 16);
+      const float e = (b3 ? e1 : e0) + __shfl_xor_sync(0xffffffffu, b3 ? e0 : e1, 8);
+      mine[32 * cj + lc + (b4 ? 2 : 0) + (b3 ? 1 : 0)] += e;
+      __syncwarp();
     }
-    __syncwarp();
+    if (I != ci || s + 1 == s1) {
+      flush(ci);
+      if (s + 1 < s1) rows(I);
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = nx[i];
   }
   // plain rows of B: one warp per row, rows dealt to the CTAs round-robin
   for (int r = sidx + S * warp; r < t.nb; r += 8 * S) {
-    const T *brow = A + t.b_off + (long long)r * t.ld;
-    T acc = T(0);
+    const float *brow = A + t.b_off + (long long)r * t.ld;
+    float acc = 0.f;
     for (int c = lane; c < n; c += 32) acc += brow[c] * xs[c];
     acc = warp_sum(acc);
     if (lane == 0) {
-      const double v = alpha * (double)acc;
-      y[t.yb_off + r] = (t.flags & 2) ? y[t.yb_off + r] + v : v;
+      const double o = alpha * (double)acc;
+      y[t.yb_off + r] = (t.flags & 2) ? y[t.yb_off + r] + o : o;
     }
   }
   __syncthreads();
+  auto column = [&](int r) {
+    float s = part[r];
+#pragma unroll
+    for (int w = 1; w < 8; ++w) s += part[w * np + r];
+    return s;
+  };
   if (S == 1) {
     for (int r = tid; r < n; r += 256) {
-      T v = part[r];
-#pragma unroll
-      for (int w = 1; w < 8; ++w) v += part[w * np + r];
-      const double o = alpha * (double)v;
+      const double o = alpha * (double)column(r);
       y[t.y_off + r] = (t.flags & 2) ? y[t.y_off + r] + o : o;
     }
     return;
   }
-  T *mysum = scratch + ((long long)t.scr + sidx) * ld_scr;
-  for (int r = tid; r < n; r += 256) {
-    T v = part[r];
-#pragma unroll
-    for (int w = 1; w < 8; ++w) v += part[w * np + r];
-    mysum[r] = v;
-  }
+  float *mysum = scratch + ((long long)t.scr + sidx) * ld_scr;
+  for (int r = tid; r < n; r += 256) mysum[r] = column(r);
   __threadfence();
   __syncthreads();
   if (tid == 0) last = (atomicAdd(&counter[t.ctr], 1) == S - 1);
   __syncthreads();
   if (!last) return;
   __threadfence();
-  const T *sums = scratch + (long long)t.scr * ld_scr;
+  const float *sums = scratch + (long long)t.scr * ld_scr;
   for (int r = tid; r < n; r += 256) {
-    T v = __ldcg(sums + r);
-    for (int q = 1; q < S; ++q) v += __ldcg(sums + (long long)q * ld_scr + r);
-    const double o = alpha * (double)v;
+    float s = __ldcg(sums + r);
+    for (int q = 1; q < S; ++q) s += __ldcg(sums + (long long)q * ld_scr + r);
+    const double o = alpha * (double)s;
     y[t.y_off + r] = (t.flags & 2) ? y[t.y_off + r] + o : o;
   }
   if (tid == 0) counter[t.ctr] = 0;  // ready for the next launch
@@ -627,7 +663,7 @@ static size_t symv_fix_smem(int max_n) {
 template <typename T>
 size_t symv_smem(int max_n) {
   const size_t np = (size_t)((max_n + 31) / 32) * 32;
-  return std::is_same<T, double>::value ? symv_fix_smem(max_n) : sizeof(T) * (9 * np + 8 * 32 * 33);
+  return std::is_same<T, double>::value ? symv_fix_smem(max_n) : sizeof(T) * 9 * np;
 }
 
 // The CTAs of a launch: whole matrices while they fill the resident slots (a split costs a
@@ -696,7 +732,7 @@ void launch_symv_batched(int ntasks, int max_n, const SymvTask *d_tasks, const f
                          const int *xidx, double *y, double alpha, const int *done, float *scratch, int *counter,
                          int ld_scr, cudaStream_t s) {
   if (ntasks == 0 || max_n == 0) return;
-  launch_pdl(k_symv_batched<float>, ntasks, 256, symv_smem<float>(max_n), s, d_tasks, A, x, xidx, y, alpha, done, scratch,
+  launch_pdl(k_symv_batched, ntasks, 256, symv_smem<float>(max_n), s, d_tasks, A, x, xidx, y, alpha, done, scratch,
                                                                     counter, ld_scr);
   count_launch();
 }
@@ -890,7 +926,7 @@ int symv_occupancy(int max_n) {
   const cudaError_t e =
       std::is_same<T, double>::value
           ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_symv_fix, 256, symv_smem<T>(max_n))
-          : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_symv_batched<float>, 256, symv_smem<T>(max_n));
+          : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_symv_batched, 256, symv_smem<T>(max_n));
   if (e != cudaSuccess) return 0;
   return occ;
 }
@@ -1327,7 +1363,7 @@ bool dense_configure() {
   ok &= cudaFuncSetAttribute(k_gemv_t<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim) == cudaSuccess;
   ok &= cudaFuncSetAttribute(k_gemv_t<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim) == cudaSuccess;
   ok &= cudaFuncSetAttribute(k_symv_rows<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim) == cudaSuccess;
-  ok &= cudaFuncSetAttribute(k_symv_batched<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim) == cudaSuccess;
+  ok &= cudaFuncSetAttribute(k_symv_batched, cudaFuncAttributeMaxDynamicSharedMemorySize, lim) == cudaSuccess;
   ok &= cudaFuncSetAttribute(k_symv_fix, cudaFuncAttributeMaxDynamicSharedMemorySize, lim) == cudaSuccess;
   ok &= cudaFuncSetAttribute(k_symv_rows<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim) == cudaSuccess;
   ok &= cudaFuncSetAttribute(k_gemv_task<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim) == cudaSuccess;
