@@ -394,23 +394,25 @@ class Solver:
         self._check(self._lib.bidomain_mlp_sizes(self._h, *[C.byref(x) for x in v]), "bidomain_mlp_sizes")
         return dict(zip(("n_in", "n_hidden", "n_out", "batch"), (x.value for x in v)))
 
+    def _n_mlp_params(self):
+        """Length of the packed parameters."""
+        sz = self.mlp_sizes()
+        return sz["n_hidden"] * (sz["n_in"] + 1) + sz["n_hidden"] * (sz["n_hidden"] + 1) + \
+            sz["n_out"] * (sz["n_hidden"] + 1)
+
     def mlp_params(self, w=None):
         """Packed float32 parameters: upload `w` when given, else download."""
         if w is not None:
             w = np.ascontiguousarray(w, dtype=np.float32)
             self._check(self._lib.bidomain_mlp_params(self._h, w.ctypes.data, 1), "bidomain_mlp_params")
             return w
-        sz = self.mlp_sizes()
-        n = sz["n_hidden"] * (sz["n_in"] + 1) + sz["n_hidden"] * (sz["n_hidden"] + 1) + \
-            sz["n_out"] * (sz["n_hidden"] + 1)
-        out = np.zeros(n, np.float32)
+        out = np.zeros(self._n_mlp_params(), np.float32)
         self._check(self._lib.bidomain_mlp_params(self._h, out.ctypes.data, 0), "bidomain_mlp_params")
         return out
 
     def mlp_loss_grad(self, X, T, mask):
         X, T, mask = (np.ascontiguousarray(a, dtype=np.float32) for a in (X, T, mask))
-        w = self.mlp_params()
-        g = np.zeros_like(w)
+        g = np.empty(self._n_mlp_params(), np.float32)
         loss = C.c_double()
         self._check(self._lib.bidomain_mlp_loss_grad(self._h, X.ctypes.data, T.ctypes.data, mask.ctypes.data,
                                                 C.byref(loss), g.ctypes.data), "bidomain_mlp_loss_grad")

@@ -2171,14 +2171,14 @@ int bidomain_mlp_loss_grad(bd_handle *h, const float *X, const float *T, const f
   return guard(h, [&] {
     MlpDev &M = h->mlp;
     const size_t nx = (size_t)M.batch * M.n_in, ny = (size_t)M.batch * M.n_out;
-    std::vector<float> mk(mask, mask + ny);
-    double cnt = 0.0;
-    for (float v : mk) cnt += v;
     ck(cudaMemcpyAsync(M.Xf, X, sizeof(float) * nx, cudaMemcpyHostToDevice, h->s), "mlp X");
     ck(cudaMemcpyAsync(M.T, T, sizeof(float) * ny, cudaMemcpyHostToDevice, h->s), "mlp T");
     ck(cudaMemcpyAsync(M.mask, mask, sizeof(float) * ny, cudaMemcpyHostToDevice, h->s), "mlp mask");
     mlp_inputs_from_f32(M, h->s);
     mlp_forward(M, h->d_err, h->s);
+    double part[8] = {};  // the mask's sum, while the device works; eight chains instead of one
+    for (size_t i = 0; i < ny; ++i) part[i & 7] += mask[i];
+    const double cnt = ((part[0] + part[1]) + (part[2] + part[3])) + ((part[4] + part[5]) + (part[6] + part[7]));
     mlp_backward(M, (float)(1.0 / std::max(cnt, 1.0)), h->d_partial, h->d_err, h->s);
     launch_sum_partials(kRedBlocks, h->d_partial, h->d_scal + 4, h->s);
     if (loss) *loss = read_scalar(*h, h->d_scal + 4);
