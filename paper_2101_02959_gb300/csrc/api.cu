@@ -239,6 +239,7 @@ struct bd_handle {
   // the local constrained solve (fork / join events; captured into the Krylov graphs too)
   cudaStream_t s2 = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
+  LookAhead ahead;  // stream and events of the panels worked ahead of a trailing update
   int device = -1;  // the device current at bidomain_setup: every buffer of the handle lives there
   long step_n = 0;
   DevMem mem;
@@ -1163,7 +1164,7 @@ void run_engine_groups(bd_handle &h, const EngineShape &all, const MatDesc *d_de
       g.max_m = std::max(g.max_m, all.m[q]);
       g.max_e = std::max(g.max_e, all.e[q]);
     }
-    engine_partial_cholesky<T>(g, d_desc + a, base, h.d_err, h.s, linv, &h.prof, h.tc(), h.ws);
+    engine_partial_cholesky<T>(g, d_desc + a, base, h.d_err, h.s, linv, &h.prof, h.tc(), h.ws, &h.ahead);
   }
 }
 
@@ -1219,7 +1220,7 @@ void linearize_t(bd_handle &h, Dense<T> &D, bool precond) {
   {  // one large matrix: its trailing updates go to the tensor cores like the local ones
     EngineShape co = h.shCo;
     co.ob = h.tune_ob;
-    engine_partial_cholesky<T>(co, h.d_Codesc, D.Co, h.d_err, s, D.LdCo, &h.prof, h.tc(), h.ws);
+    engine_partial_cholesky<T>(co, h.d_Codesc, D.Co, h.d_err, s, D.LdCo, &h.prof, h.tc(), h.ws, &h.ahead);
   }
   launch_copy<T, T>(h.cp_coinv.n, h.cp_coinv.max_elems, h.cp_coinv.d, D.Co, D.CoInv, s);
   if (h.d_CoInv64) coarse_refine64<T>(h.np, D.CoInv, pad8(h.np), h.d_Co64d, h.d_CoInv64, h.d_CoW, h.d_CoY, s);
@@ -1964,6 +1965,9 @@ int bidomain_setup(const bd_mesh *mesh, const bd_conductivity *cond, const bd_io
     if (stream) h->s = (cudaStream_t)stream;
     else { ck(cudaStreamCreateWithFlags(&h->s, cudaStreamNonBlocking), "stream"); h->own_stream = true; }
     ck(cudaStreamCreateWithFlags(&h->s2, cudaStreamNonBlocking), "stream");
+    ck(cudaStreamCreateWithFlags(&h->ahead.s, cudaStreamNonBlocking), "stream");
+    ck(cudaEventCreateWithFlags(&h->ahead.cols, cudaEventDisableTiming), "event");
+    ck(cudaEventCreateWithFlags(&h->ahead.panels, cudaEventDisableTiming), "event");
     ck(cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming), "event");
     ck(cudaEventCreateWithFlags(&h->ev_join, cudaEventDisableTiming), "event");
     if (h->opt.precision != BD_MIXED) h->opt.use_tensor_cores = 0;
@@ -2339,7 +2343,9 @@ int bidomain_destroy(bd_handle *h) {
   cudaStreamSynchronize(h->s);
   if (h->s2) cudaStreamSynchronize(h->s2);
   cudaStream_t s = h->s, s2 = h->s2;
+  if (h->ahead.s) cudaStreamSynchronize(h->ahead.s);
   cudaEvent_t e1 = h->ev_fork, e2 = h->ev_join;
+  const LookAhead la = h->ahead;
   const bool own = h->own_stream;
   for (auto &g : h->pcg_exec)
     if (g) cudaGraphExecDestroy(g);
@@ -2347,6 +2353,9 @@ int bidomain_destroy(bd_handle *h) {
   if (e1) cudaEventDestroy(e1);
   if (e2) cudaEventDestroy(e2);
   if (s2) cudaStreamDestroy(s2);
+  if (la.cols) cudaEventDestroy(la.cols);
+  if (la.panels) cudaEventDestroy(la.panels);
+  if (la.s) cudaStreamDestroy(la.s);
   if (own) cudaStreamDestroy(s);
   return BD_OK;
 }

@@ -331,15 +331,28 @@ static double band_entries(const MatDesc &hd, int t0, int ke, int cend) {
   return (double)(a * (a + 1) / 2 + b * k + (long long)(br.nv - br.ni) * k);
 }
 
+// Few matrices (kAheadCount at most) leave the chip idle in the chain of a block's panels (a diagonal
+// block is one CTA for 32 us, its rows a few CTAs for 22).  There the trailing update is cut in two:
+// first the columns of the next outer block, then, beside that block's panels on a second stream, the
+// columns right of it, on kAheadSms fewer CTAs so that the panels find free SMs.  The two sides share
+// no column, and the digit planes of the panels' own updates take half of the workspace.  A Jacobian
+// of the masked shell (coarse matrix of 2,618 unknowns) takes 3 % less, of the 128x128x32 slab too.
+constexpr int kAheadCount = 8, kAheadSms = 24;
+
 template <typename T>
 void engine_partial_cholesky(const EngineShape &sh, const MatDesc *d_desc, T *base, int *d_err, cudaStream_t s,
-                             T *store, ProfHook *prof, int tc, const SliceWs &ws) {
+                             T *store, ProfHook *prof, int tc, const SliceWs &ws, const LookAhead *ahead) {
   if (sh.count == 0) return;
   constexpr bool f64 = std::is_same<T, double>::value;
   const bool narrow = f64 || tc == 2;  // 64-column panels solved on the tensor cores
   const int PW = narrow ? kPanel64 : kPW;
   T *pinv = static_cast<T *>(ws.pinv);
   const int ob = std::max(kPW, (sh.ob / kPW) * kPW);  // outer block: columns per long-K trailing update
+  SliceWs half[2] = {ws, ws};                         // planes of the trailing updates, of the panels ahead
+  half[0].bytes = half[1].bytes = (ws.bytes / 2) & ~(size_t)4095;
+  half[1].mem = ws.mem + half[0].bytes;
+  const bool look = ahead && (f64 || tc) && sh.count <= kAheadCount && sh.max_e > ob &&
+                    slice_fits<T>(sh.count, sh.max_m, std::max(ob, PW), half[0]);
   // host copies of the descriptors' sizes and bands: the grids cover the rows and columns
   // the band lets an update reach (the kernels apply the same limits per matrix)
   std::vector<MatDesc> hd(sh.count);
@@ -350,7 +363,8 @@ void engine_partial_cholesky(const EngineShape &sh, const MatDesc *d_desc, T *ba
     if (!sh.id0.empty()) hd[b].id0 = sh.id0[b];
     if (!sh.ifirst.empty()) hd[b].ifirst = sh.ifirst[b];
   }
-  for (int K0 = 0; K0 < sh.max_e; K0 += ob) {
+  // the panels of the outer block from K0 on
+  auto block = [&](int K0, cudaStream_t q, const SliceWs &w_s) {
     const int K1 = K0 + ob;
     for (int k0 = K0; k0 < std::min(K1, sh.max_e); k0 += PW) {
       int max_below = 0, max_cols = 0;
@@ -365,31 +379,35 @@ void engine_partial_cholesky(const EngineShape &sh, const MatDesc *d_desc, T *ba
         fl_panel += (double)w * w * w / 3.0 + (double)below * w * w;
         fl_in += 2.0 * w * band_entries(hd[b], k0 + w, k0 + w, cend);
       }
-      if (prof) prof->begin(PROF_PANEL, s);
+      if (prof) prof->begin(PROF_PANEL, q);
       if (narrow) {
-        launch_diag<T>(d_desc, base, k0, sh.count, d_err, store, pinv, s);
-        launch_update<T>(d_desc, base, Upd64{3, k0, 0, PW, 0, 0}, max_below, PW, sh.count, ws, d_err, s, pinv);
+        launch_diag<T>(d_desc, base, k0, sh.count, d_err, store, pinv, q);
+        launch_update<T>(d_desc, base, Upd64{3, k0, 0, PW, 0, 0}, max_below, PW, sh.count, w_s, d_err, q, pinv);
       } else if constexpr (!f64) {
-        launch_diag128(d_desc, base, k0, sh.count, d_err, store, s);
+        launch_diag128(d_desc, base, k0, sh.count, d_err, store, q);
         if (max_below > 0) {
-          k_panel_rows<<<dim3(ceil_div(max_below, kPanelRB), sh.count), 256, kPanelSmem, s>>>(d_desc, base, k0);
+          k_panel_rows<<<dim3(ceil_div(max_below, kPanelRB), sh.count), 256, kPanelSmem, q>>>(d_desc, base, k0);
           count_launch();
         }
       }
-      if (prof) prof->end(PROF_PANEL, s, fl_panel, 0.0);
+      if (prof) prof->end(PROF_PANEL, q, fl_panel, 0.0);
       // the rest of the outer block: rows [k0 + w, m), columns [k0 + w, min(K1, e)); timed
       // with the panels (the long-K class holds only the trailing updates)
       if (max_below > 0 && max_cols > 0) {
-        if (prof) prof->begin(PROF_PANEL, s);
+        if (prof) prof->begin(PROF_PANEL, q);
         if constexpr (f64) {
-          launch_update<T>(d_desc, base, Upd64{0, k0, K1, PW, 0, 0}, max_below, max_cols, sh.count, ws, d_err, s);
+          launch_update<T>(d_desc, base, Upd64{0, k0, K1, PW, 0, 0}, max_below, max_cols, sh.count, w_s, d_err, q);
         } else {
-          if (tc) launch_update<T>(d_desc, base, Upd64{0, k0, K1, PW, 0, 0}, max_below, max_cols, sh.count, ws, d_err, s);
-          else launch_rankk(d_desc, base, 0, k0, K0, K1, max_below, max_cols, sh.count, s);
+          if (tc) launch_update<T>(d_desc, base, Upd64{0, k0, K1, PW, 0, 0}, max_below, max_cols, sh.count, w_s, d_err, q);
+          else launch_rankk(d_desc, base, 0, k0, K0, K1, max_below, max_cols, sh.count, q);
         }
-        if (prof) prof->end(PROF_PANEL, s, fl_in, 0.0);
+        if (prof) prof->end(PROF_PANEL, q, fl_in, 0.0);
       }
     }
+  };
+  block(0, s, ws);
+  for (int K0 = 0; K0 < sh.max_e; K0 += ob) {
+    const int K1 = K0 + ob;
     // outer update of the trailing columns [K1, e) with the finished outer panel
     int max_rows = 0, max_cols = 0;
     double fl = 0.0, by = 0.0;
@@ -402,16 +420,33 @@ void engine_partial_cholesky(const EngineShape &sh, const MatDesc *d_desc, T *ba
       fl += 2.0 * ob * ent;
       by += sizeof(T) * (2.0 * ent + (double)ob * rows);
     }
-    if (max_rows > 0 && max_cols > 0) {
+    const bool update = max_rows > 0 && max_cols > 0;
+    const Upd64 u{2, K0, K1, PW, K0, K1};
+    if (update && look) {
+      if (prof) prof->begin(PROF_RANKK, s);
+      launch_update<T>(d_desc, base, u, max_rows, max_cols, sh.count, half[0], d_err, s, nullptr,
+                       UpdPart{0, ob / kUpdN, false, 0});
+      cudaEventRecord(ahead->cols, s);
+      cudaStreamWaitEvent(ahead->s, ahead->cols, 0);
+      launch_update<T>(d_desc, base, u, max_rows, max_cols, sh.count, half[0], d_err, s, nullptr,
+                       UpdPart{ob / kUpdN, -1, true, kUpdCtas - kAheadSms});
+      if (prof) prof->end(PROF_RANKK, s, fl, by);
+      block(K1, ahead->s, half[1]);
+      cudaEventRecord(ahead->panels, ahead->s);
+      cudaStreamWaitEvent(s, ahead->panels, 0);
+      continue;
+    }
+    if (update) {
       if (prof) prof->begin(PROF_RANKK, s);
       if constexpr (f64) {
-        launch_update<T>(d_desc, base, Upd64{2, K0, K1, PW, K0, K1}, max_rows, max_cols, sh.count, ws, d_err, s);
+        launch_update<T>(d_desc, base, u, max_rows, max_cols, sh.count, ws, d_err, s);
       } else {
-        if (tc) launch_update<T>(d_desc, base, Upd64{2, K0, K1, PW, K0, K1}, max_rows, max_cols, sh.count, ws, d_err, s);
+        if (tc) launch_update<T>(d_desc, base, u, max_rows, max_cols, sh.count, ws, d_err, s);
         else launch_rankk(d_desc, base, 2, 0, K0, K1, max_rows, max_cols, sh.count, s);
       }
       if (prof) prof->end(PROF_RANKK, s, fl, by);
     }
+    if (K1 < sh.max_e) block(K1, s, ws);
   }
   int max_t = 0;
   double fl = 0.0, by = 0.0;
@@ -1392,7 +1427,7 @@ bool dense_configure() {
 
 #define BD_INST(T)                                                                                              \
   template void engine_partial_cholesky<T>(const EngineShape &, const MatDesc *, T *, int *, cudaStream_t,    \
-                                           T *, ProfHook *, int, const SliceWs &);                                              \
+                                           T *, ProfHook *, int, const SliceWs &, const LookAhead *);                                              \
   template void launch_gemv<T>(int, int, int, const GemvDesc *, const T *, const double *, const int *,        \
                                double *, double, const int *, cudaStream_t);                                   \
   template void launch_symv_rows<T>(int, const T *, int, const double *, double *, int, const int *,           \

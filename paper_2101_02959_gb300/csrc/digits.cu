@@ -60,7 +60,7 @@ template <typename T> constexpr int update_smem() {
   return Dig<T>::Stages * stage_bytes<T>() + kDrain * epi_bytes<T>() + 1024;
 }
 constexpr uint32_t kTmemCols = 512;
-constexpr int kSms = 152;
+constexpr int kSms = kUpdCtas;
 constexpr int kExNan = 1 << 20;    // exponent mark of a row that holds an infinity or a NaN
 
 // Rows, columns and K range of an update.
@@ -380,7 +380,7 @@ __global__ void __launch_bounds__(kUThreads, 1) k_update(const MatDesc *__restri
       const long long idx = blockIdx.x + (32LL * k + lane) * gridDim.x;
       Tile t;
       const bool valid = idx < total && make_tile(desc, out, u, (int)(idx / per), (int)(idx % per) / nct,
-                                                  (int)(idx % per) % nct, N, t);
+                                                  u.ct0 + (int)(idx % per) % nct, N, t);
       const unsigned m = __ballot_sync(0xffffffffu, valid);
       if (valid) ring[slot][__popc(m & ((1u << lane) - 1u))] = t;
       const bool last = blockIdx.x + 32LL * (k + 1) * gridDim.x >= total;
@@ -894,11 +894,16 @@ size_t slice_bytes(int count, int max_rows, int max_e) {
   return (size_t)std::max(1, count) * (rows_bytes<T>(max_rows, std::min(std::max(max_e, 1), kSliceK)) + inv_bytes<T>());
 }
 
+template <typename T>
+bool slice_fits(int count, int max_rows, int cols, const SliceWs &ws) {
+  return cols <= kSliceK && ws.bytes / (rows_bytes<T>(max_rows, cols) + inv_bytes<T>()) >= (size_t)count;
+}
+
 // Runs of matrices whose planes fit the workspace; the final update (mode 1) also in runs of
 // kSliceK columns (each run rounds C once more, so they are long).
 template <typename T>
 void launch_update(const MatDesc *d_desc, T *base, Upd64 u, int max_rows, int max_cols, int count,
-                   const SliceWs &ws, int *err, cudaStream_t s, const T *pinv) {
+                   const SliceWs &ws, int *err, cudaStream_t s, const T *pinv, const UpdPart &part) {
   if (max_rows <= 0 || max_cols <= 0 || count <= 0) return;
   using C = Dig<T>;
   const bool panel = u.mode == 0 || u.mode == 3;
@@ -906,7 +911,9 @@ void launch_update(const MatDesc *d_desc, T *base, Upd64 u, int max_rows, int ma
   const int kmax = std::min(zz - za, kSliceK), nrb = pad_rows(max_rows) / 64;
   const int run = (int)std::max<size_t>(
       1, std::min<size_t>((size_t)count, ws.bytes / (rows_bytes<T>(max_rows, kmax) + inv_bytes<T>())));
-  const int nrt = ceil_div(max_rows, kUM), nct = ceil_div(max_cols, C::N), rpc = 256 / (C::Grp / 8);
+  const int nrt = ceil_div(max_rows, kUM), rpc = 256 / (C::Grp / 8), rest = ceil_div(max_cols, C::N) - part.ct0;
+  const int nct = part.nct < 0 ? rest : std::min(rest, part.nct), ctas = part.ctas > 0 ? part.ctas : kSms;
+  if (nct <= 0) return;
   unsigned char *sl = ws.mem, *slb = sl + (size_t)run * planes_bytes<T>(nrb * 64, kmax);
   int *ex = reinterpret_cast<int *>(slb + (size_t)run * planes_bytes<T>(C::N, kPanel64));
   int *exb = ex + (size_t)run * ceil_div(kmax, C::Grp) * nrb * 64;
@@ -916,10 +923,13 @@ void launch_update(const MatDesc *d_desc, T *base, Upd64 u, int max_rows, int ma
       Upd64 q = u;
       q.ka = ka;
       q.kz = std::min(zz, ka + kSliceK);
+      q.ct0 = part.ct0;
       const int kw = q.kz - ka, nkc = ceil_div(kw, kUK), ng = ceil_div(kw, C::Grp);
       const Planes pa{sl, ex, nrb, nkc, ng}, pi{slb, exb, C::N / 64, kPanel64 / kUK, 1};
-      k_slice<T><<<dim3(nrb * 64 / rpc, ng, nb), 256, 0, s>>>(d_desc + b0, base, q, nullptr, sl, ex, nrb, nkc, ng);
-      count_launch();
+      if (!part.sliced) {
+        k_slice<T><<<dim3(nrb * 64 / rpc, ng, nb), 256, 0, s>>>(d_desc + b0, base, q, nullptr, sl, ex, nrb, nkc, ng);
+        count_launch();
+      }
       if (u.mode == 3) {
         const T *pv = pinv + (size_t)b0 * u.pw * u.pw;
         k_slice<T><<<dim3(C::N / rpc, 1, nb), 256, 0, s>>>(d_desc + b0, base, q, pv, slb, exb, C::N / 64,
@@ -927,7 +937,7 @@ void launch_update(const MatDesc *d_desc, T *base, Upd64 u, int max_rows, int ma
         count_launch();
       }
       const int per = nrt * nct, total = per * nb;
-      k_update<T><<<std::min(total, kSms), kUThreads, update_smem<T>(), s>>>(d_desc + b0, d_desc + b0, base, q, pa,
+      k_update<T><<<std::min(total, ctas), kUThreads, update_smem<T>(), s>>>(d_desc + b0, d_desc + b0, base, q, pa,
                                                                             u.mode == 3 ? pi : pa, nct, per, total, err);
       count_launch();
     }
@@ -969,7 +979,8 @@ void launch_product(const MatDesc *d_a, const T *A, const MatDesc *d_b, const T 
   template void launch_diag<T>(const MatDesc *, T *, int, int, int *, T *, T *, cudaStream_t);               \
   template size_t slice_bytes<T>(int, int, int);                                                             \
   template void launch_update<T>(const MatDesc *, T *, Upd64, int, int, int, const SliceWs &, int *,       \
-                                 cudaStream_t, const T *);                                                  \
+                                 cudaStream_t, const T *, const UpdPart &);                                 \
+  template bool slice_fits<T>(int, int, int, const SliceWs &);                                               \
   template size_t product_bytes<T>(int, int);                                                                \
   template void launch_product<T>(const MatDesc *, const T *, const MatDesc *, const T *, const MatDesc *, T *, int, \
                                   int, const SliceWs &, int *, cudaStream_t);

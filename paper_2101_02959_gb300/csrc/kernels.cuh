@@ -76,9 +76,19 @@ void launch_sum_partials(int nblk, const double *partial, double *out, cudaStrea
 
 // digits.cu -- rank-k updates and panel solves on the tensor cores by exact digit products.
 constexpr int kPanel64 = 64;   // panel width where the panels too are solved that way
+constexpr int kUpdN = 64;       // columns of an update's tile
+constexpr int kUpdCtas = 152;   // its persistent CTAs, one per SM
 constexpr int kSliceK = 1024;  // columns whose digit planes the workspace holds at a time
 struct Upd64 {                 // one update over a batch (modes as in digits.cu); pw: panel width
   int mode, K0, K1, pw, ka, kz;
+  int ct0 = 0;                 // first of the launch's column tiles
+};
+// Part of an update: its column tiles [ct0, ct0 + nct) (nct < 0: to the end), the digit planes of an
+// earlier part of the same update reused when `sliced`, on at most `ctas` CTAs (0: all SMs).
+struct UpdPart {
+  int ct0 = 0, nct = -1;
+  bool sliced = false;
+  int ctas = 0;
 };
 struct SliceWs {               // workspace: digit planes and row exponents; a panel inverse per matrix
   unsigned char *mem = nullptr;
@@ -106,9 +116,13 @@ struct EngineShape {
 // block's width).  tc: 0 SIMT (FP32 only), 1 the updates on the tensor cores (digits.cu), 2 also the
 // panels, 64 columns wide (always in FP64).
 constexpr int kEnginePanel = 128;
+struct LookAhead {  // second stream and events of the panels worked ahead of an update's rest
+  cudaStream_t s = nullptr;
+  cudaEvent_t cols = nullptr, panels = nullptr;
+};
 template <typename T>
 void engine_partial_cholesky(const EngineShape &sh, const MatDesc *d_desc, T *base, int *d_err, cudaStream_t s,
-                             T *store, ProfHook *prof, int tc, const SliceWs &ws);
+                             T *store, ProfHook *prof, int tc, const SliceWs &ws, const LookAhead *ahead = nullptr);
 
 bool dense_configure();
 size_t dense_smem_limit();  // bytes of shared memory the dense kernels may stage per CTA
@@ -120,7 +134,10 @@ template <typename T>
 size_t slice_bytes(int count, int max_rows, int max_e);
 template <typename T>
 void launch_update(const MatDesc *d_desc, T *base, Upd64 u, int max_rows, int max_cols, int count, const SliceWs &ws,
-                   int *err, cudaStream_t s, const T *pinv = nullptr);
+                   int *err, cudaStream_t s, const T *pinv = nullptr, const UpdPart &part = {});
+// the digit planes of `cols` columns of the whole batch fit the workspace at once
+template <typename T>
+bool slice_fits(int count, int max_rows, int cols, const SliceWs &ws);
 template <typename T>
 size_t product_bytes(int count, int max_n);
 template <typename T>
