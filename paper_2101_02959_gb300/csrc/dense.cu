@@ -44,18 +44,22 @@ template <> struct Vec16<double> {
 };
 
 // ---- rows below a 128-column panel: L_21 = A_21 L_11^-T (FP32) ----------------------
-// The diagonal block is factored already (k_diag128).  RB rows per CTA, staged in shared memory; 32
-// columns at a time: one thread per row solves x L_bb^T = a, then all threads apply the rank-32 update
-// to the remaining columns (4 x 4 register tiles over a transposed copy of the solved columns), reading
-// the finished L_11 one 32-column slice at a time.  Rows: those the band lets the panel reach.
+// The diagonal block is factored already and its 32 x 32 diagonal blocks inverted (k_diag128).  RB rows
+// per CTA, staged in shared memory; 32 columns at a time: multiplied by that inverse (4 x 4 tiles),
+// then a rank-32 update of the remaining columns (4 x 4 tiles over transposed copies of the solved
+// columns and of L_11's, the next 32 columns of L_11 on their way meanwhile).  Rows: those the band lets
+// the panel reach.  A chain of latencies: one thread per row substituted here before (22 us for
+// the 2,490 rows of a coarse panel on 20 CTAs; 11 us on 78 CTAs of 32 rows now).
 constexpr int kPW = kEnginePanel;  // panel width
 constexpr int kLDP = kPW + 4;      // row stride of the staged panel (16-byte aligned rows)
-constexpr int kPanelRB = 128, kPanelNR = kPW + kPanelRB;
-constexpr size_t kPanelSmem = sizeof(float) * ((size_t)kPanelRB * kLDP + 32 * kPanelNR + 32 * 32 + 32);
+constexpr int kLDY = 36;
+template <int RB>
+constexpr size_t panel_smem() { return sizeof(float) * ((size_t)RB * kLDP + 32 * (kPW + RB) + 32 * kLDY); }
 
+template <int RB>
 __global__ void __launch_bounds__(256, 2) k_panel_rows(const MatDesc *__restrict__ desc, float *__restrict__ base,
-                                                       int K0) {
-  constexpr int RB = kPanelRB, NR = kPanelNR, VPP = kPW / 4;  // VPP: vectors per staged row
+                                                       int K0, const float *__restrict__ pinv) {
+  constexpr int NR = kPW + RB, VPP = kPW / 4;  // VPP: vectors per staged row
   const MatDesc d = desc[blockIdx.y];
   if (K0 >= d.e) return;
   const int w = min(kPW, d.e - K0);
@@ -67,92 +71,100 @@ __global__ void __launch_bounds__(256, 2) k_panel_rows(const MatDesc *__restrict
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float *P = reinterpret_cast<float *>(smem_raw);  // [RB][kLDP] own rows
   float *PT = P + RB * kLDP;                       // [32][NR]: 32 columns, transposed (L_11 rows, then own)
-  float *Lt = PT + 32 * NR;                        // [32][32]: Lt[c][t] = L_bb[t][c]
-  float *rd = Lt + 32 * 32;                        // [32]: 1 / L_bb[c][c]
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  float *Yt = PT + 32 * NR;                        // [32][kLDY]: Yt[k][c] = (L_bb^-1)[c][k]
+  const int tid = threadIdx.x;
+  // L_11 below the sub-block (columns [c0, c0 + 32) of rows [c0 + 32, w): three vectors a thread) and
+  // the sub-block's inverse (one)
+  float4 lv[3], yv;
+  auto fetch = [&](int bq) {
+    const int c0 = 32 * bq;
+#pragma unroll
+    for (int u = 0; u < 3; ++u) {
+      const int idx = tid + 256 * u, p = c0 + 32 + idx / 8;
+      lv[u] = p < w ? *reinterpret_cast<const float4 *>(A + (long long)(K0 + p) * d.ld + K0 + c0 + (idx % 8) * 4) : float4{};
+    }
+    yv = *reinterpret_cast<const float4 *>(pinv + ((long long)blockIdx.y * 4 + bq) * 1024 + tid * 4);
+  };
+  fetch(0);
   // stage: kBatch vector loads in flight per thread and batch
-  constexpr int kVec = RB * VPP, kBatch = 8;
+  constexpr int kVec = RB * VPP, kBatch = kVec / 256 < 8 ? kVec / 256 : 8;
   for (int base_i = 0; base_i < kVec; base_i += 256 * kBatch) {
     float4 buf[kBatch];
 #pragma unroll
     for (int u = 0; u < kBatch; ++u) {
       const int idx = base_i + tid + 256 * u, sr = idx / VPP, cv = idx % VPP;
-      const bool ok = idx < kVec && cv * 4 < w && sr < nrows;
+      const bool ok = cv * 4 < w && sr < nrows;
       buf[u] = ok ? *reinterpret_cast<const float4 *>(A + (long long)br.row(v0 + sr) * d.ld + K0 + cv * 4) : float4{};
     }
 #pragma unroll
     for (int u = 0; u < kBatch; ++u) {
       const int idx = base_i + tid + 256 * u, sr = idx / VPP, cv = idx % VPP;
-      if (idx < kVec) {
-        float4 o = buf[u];
-        if (cv * 4 + 1 >= w) o.y = 0.f;
-        if (cv * 4 + 2 >= w) o.z = 0.f;
-        if (cv * 4 + 3 >= w) o.w = 0.f;
-        *reinterpret_cast<float4 *>(P + sr * kLDP + cv * 4) = o;
-      }
+      float4 o = buf[u];
+      if (cv * 4 + 1 >= w) o.y = 0.f;
+      if (cv * 4 + 2 >= w) o.z = 0.f;
+      if (cv * 4 + 3 >= w) o.w = 0.f;
+      *reinterpret_cast<float4 *>(P + sr * kLDP + cv * 4) = o;
     }
   }
-  const int nbk = ceil_div(w, 32);
+  const int nbk = ceil_div(w, 32), nr4 = (nrows + 3) / 4;
   for (int bq = 0; bq < nbk; ++bq) {
-    const int c0 = 32 * bq, wb = min(32, w - c0);
-    const int nbelow = max(0, w - c0 - 32);  // L_11 rows below the sub-block
+    const int c0 = 32 * bq;
     __syncthreads();
-    if (wid == 0) {
-      const float *src = A + (long long)(K0 + c0 + (lane < wb ? lane : 0)) * d.ld + K0 + c0;
-      float dg = 1.f;
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const float4 v = lane < wb && i * 4 <= lane ? *reinterpret_cast<const float4 *>(src + i * 4) : float4{};
+    for (int u = 0; u < 3; ++u) {
+      const int idx = tid + 256 * u, p = c0 + 32 + idx / 8, cv = (idx % 8) * 4;
+      if (p < kPW) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) PT[(cv + q) * NR + p] = Vec16<float>::get(lv[u], q);
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) Yt[((tid & 7) * 4 + q) * kLDY + (tid >> 3)] = Vec16<float>::get(yv, q);
+    if (bq + 1 < nbk) fetch(bq + 1);
+    __syncthreads();
+    // x = a Y^T: four rows RB / 4 apart (consecutive threads read consecutive rows) by four columns a thread
+    constexpr int RS = RB / 4;
+    const int r0 = tid % RS, j0 = 4 * (tid / RS);
+    const bool mine = j0 < 32;
+    float x[4][4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) x[i][j] = 0.f;
+    if (mine) {
+#pragma unroll
+      for (int k = 0; k < 32; k += 4) {
+        float4 av[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) av[i] = *reinterpret_cast<const float4 *>(P + (r0 + RS * i) * kLDP + c0 + k);
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-          const int t = i * 4 + q;
-          const float e = (lane < wb && t <= lane) ? Vec16<float>::get(v, q) : (t == lane ? 1.f : 0.f);
-          if (t == lane) dg = e;
-          Lt[t * 32 + lane] = e;
-        }
-      }
-      rd[lane] = 1.f / dg;
-    } else {
-      // the finished L_11 rows below the sub-block, columns [c0, c0 + 32), transposed
-      for (int idx = tid - 32; idx < nbelow * 8; idx += 256 - 32) {
-        const int r = idx / 8, cv = idx % 8, p = c0 + 32 + r;
-        const float4 v = *reinterpret_cast<const float4 *>(A + (long long)(K0 + p) * d.ld + K0 + c0 + cv * 4);
+          const float4 y = *reinterpret_cast<const float4 *>(Yt + (k + q) * kLDY + j0);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) PT[(cv * 4 + q) * NR + p] = Vec16<float>::get(v, q);
-      }
-    }
-    __syncthreads();
-    if (tid < nrows) {
-      float x[32];
-      float *src = P + tid * kLDP + c0;
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const float4 v = *reinterpret_cast<const float4 *>(src + i * 4);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) x[i * 4 + q] = Vec16<float>::get(v, q);
-      }
-#pragma unroll
-      for (int c = 0; c < 32; ++c) {
-        x[c] *= rd[c];
-#pragma unroll
-        for (int i = (c + 1) / 4; i < 8; ++i) {
-          const float4 lv = *reinterpret_cast<const float4 *>(&Lt[c * 32 + i * 4]);
-#pragma unroll
-          for (int q = 0; q < 4; ++q)
-            if (i * 4 + q > c) x[i * 4 + q] -= Vec16<float>::get(lv, q) * x[c];
+          for (int i = 0; i < 4; ++i) {
+            const float e = Vec16<float>::get(av[i], q);
+            x[i][0] += e * y.x;
+            x[i][1] += e * y.y;
+            x[i][2] += e * y.z;
+            x[i][3] += e * y.w;
+          }
         }
       }
 #pragma unroll
-      for (int i = 0; i < 8; ++i)
-        *reinterpret_cast<float4 *>(src + i * 4) = make_float4(x[4 * i], x[4 * i + 1], x[4 * i + 2], x[4 * i + 3]);
+      for (int j = 0; j < 4; ++j)
 #pragma unroll
-      for (int t = 0; t < 32; ++t) PT[t * NR + kPW + tid] = x[t];
+        for (int i = 0; i < 4; ++i) PT[(j0 + j) * NR + kPW + r0 + RS * i] = x[i][j];
     }
     __syncthreads();
+    if (mine) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        *reinterpret_cast<float4 *>(P + (r0 + RS * i) * kLDP + c0 + j0) = make_float4(x[i][0], x[i][1], x[i][2], x[i][3]);
+    }
     // rank-32 update of the panel columns [c0 + 32, w), 4 x 4 tiles
     const int jb = c0 + 32, ncol = w - jb;
     if (ncol > 0) {
-      const int nr4 = (nrows + 3) / 4, nc4 = (ncol + 3) / 4;
+      const int nc4 = (ncol + 3) / 4;
       for (int mt = tid; mt < nr4 * nc4; mt += 256) {
         const int r0 = 4 * (mt / nc4), j0 = jb + 4 * (mt % nc4);
         float acc[4][4];
@@ -310,6 +322,19 @@ __global__ void __launch_bounds__(256) k_rankk128(const MatDesc *__restrict__ de
   }
 }
 
+// 128 rows per CTA share one copy of L_11; with fewer than two such CTAs an SM, 32 rows.  The shell's Jacobians
+// (a batch of 502 and a coarse matrix) take 68.9 ms so, 72.2 with 128 rows everywhere and 72.0 with 32;
+// the 128x128x32 slab's (1,024 matrices) 41.4, 41.5 and 45.3.
+static void launch_panel_rows(const MatDesc *d_desc, float *base, int K0, int max_below, int count, const float *pinv,
+                              cudaStream_t s) {
+  if (max_below <= 0) return;
+  if (ceil_div(max_below, 128) * (long long)count >= 2 * kUpdCtas)
+    k_panel_rows<128><<<dim3(ceil_div(max_below, 128), count), 256, panel_smem<128>(), s>>>(d_desc, base, K0, pinv);
+  else
+    k_panel_rows<32><<<dim3(ceil_div(max_below, 32), count), 256, panel_smem<32>(), s>>>(d_desc, base, K0, pinv);
+  count_launch();
+}
+
 static void launch_rankk(const MatDesc *d_desc, float *base, int mode, int k0, int K0, int K1, int max_rows,
                          int max_cols, int count, cudaStream_t s) {
   const int nrt = ceil_div(max_rows, kTB2), nct = ceil_div(max_cols, kTB2);
@@ -332,7 +357,7 @@ static double band_entries(const MatDesc &hd, int t0, int ke, int cend) {
 }
 
 // Few matrices (kAheadCount at most) leave the chip idle in the chain of a block's panels (a diagonal
-// block is one CTA for 32 us, its rows a few CTAs for 22).  There the trailing update is cut in two:
+// block is one CTA for 32 us, its rows a few CTAs for 11).  There the trailing update is cut in two:
 // first the columns of the next outer block, then, beside that block's panels on a second stream, the
 // columns right of it, on kAheadSms fewer CTAs so that the panels find free SMs.  The two sides share
 // no column, and the digit planes of the panels' own updates take half of the workspace.  A Jacobian
@@ -384,11 +409,8 @@ void engine_partial_cholesky(const EngineShape &sh, const MatDesc *d_desc, T *ba
         launch_diag<T>(d_desc, base, k0, sh.count, d_err, store, pinv, q);
         launch_update<T>(d_desc, base, Upd64{3, k0, 0, PW, 0, 0}, max_below, PW, sh.count, w_s, d_err, q, pinv);
       } else if constexpr (!f64) {
-        launch_diag128(d_desc, base, k0, sh.count, d_err, store, q);
-        if (max_below > 0) {
-          k_panel_rows<<<dim3(ceil_div(max_below, kPanelRB), sh.count), 256, kPanelSmem, q>>>(d_desc, base, k0);
-          count_launch();
-        }
+        launch_diag128(d_desc, base, k0, sh.count, d_err, store, pinv, q);
+        launch_panel_rows(d_desc, base, k0, max_below, sh.count, pinv, q);
       }
       if (prof) prof->end(PROF_PANEL, q, fl_panel, 0.0);
       // the rest of the outer block: rows [k0 + w, m), columns [k0 + w, min(K1, e)); timed
@@ -1407,7 +1429,8 @@ size_t dense_smem_limit() { return 200 * 1024; }
 bool dense_configure() {
   const int lim = (int)dense_smem_limit();
   bool ok = true;
-  ok &= cudaFuncSetAttribute(k_panel_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPanelSmem) == cudaSuccess;
+  ok &= cudaFuncSetAttribute(k_panel_rows<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)panel_smem<128>()) == cudaSuccess;
+  ok &= cudaFuncSetAttribute(k_panel_rows<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)panel_smem<32>()) == cudaSuccess;
   ok &= cudaFuncSetAttribute(k_trsv<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim) == cudaSuccess;
   ok &= cudaFuncSetAttribute(k_trsv<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim) == cudaSuccess;
   ok &= cudaFuncSetAttribute(k_gemv<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim) == cudaSuccess;

@@ -749,12 +749,13 @@ __global__ void __launch_bounds__(256) k_diag(const MatDesc *__restrict__ desc, 
 // One CTA per matrix, 32 columns at a time: factor and inverse as above, the block's rows below by
 // that inverse (warp = four columns, lane = row), rank-32 update of the rest (4 x 4 tiles a thread).
 // A latency chain of 128 pivots: 44 us with one warp factoring and one thread per row substituting,
-// 33 us here; a coarse matrix of 2,600 unknowns runs 21 of these one after another.
+// 33 us here.  The inverses of the four 32 x 32 diagonal blocks go to pinv.  A coarse matrix of 2,600 unknowns runs 21 of these one after another.
 constexpr int kWP = kEnginePanel, kWLD = kWP + 1;
 constexpr size_t kDiag128Smem = sizeof(float) * (size_t)kWP * kWLD;
 
 __global__ void __launch_bounds__(256) k_diag128(const MatDesc *__restrict__ desc, float *__restrict__ base, int K0,
-                                                 int *__restrict__ err, float *__restrict__ store) {
+                                                 int *__restrict__ err, float *__restrict__ store,
+                                                 float *__restrict__ pinv) {
   const MatDesc d = desc[blockIdx.x];
   if (K0 >= d.e) return;
   const int w = min(kWP, d.e - K0);
@@ -785,7 +786,12 @@ __global__ void __launch_bounds__(256) k_diag128(const MatDesc *__restrict__ des
     if (warp < 4) ldl_inv32<kWLD, 33>(P + o * kWLD + o, Y, warp, lane, Lc, piv, bad);
     __syncthreads();
     float *sb = store + ((long long)d.dblk + K0 / kNB + h) * kNB * kNB;
-    for (int q = tid; q < 1024; q += 256) sb[q] = P[(o + (q >> 5)) * kWLD + o + (q & 31)];
+    float *inv = pinv + ((long long)blockIdx.x * 4 + h) * 1024;  // for the rows below the panel
+    for (int q = tid; q < 1024; q += 256) {
+      const int i = q >> 5, j = q & 31;
+      sb[q] = P[(o + i) * kWLD + o + j];
+      inv[q] = j <= i ? Y[i * 33 + j] : 0.f;
+    }
     if (h + 1 == nbk) break;
     const int nrb = nbk - h - 1;  // 32-row blocks below
     float x[3][4];
@@ -852,8 +858,9 @@ __global__ void __launch_bounds__(256) k_diag128(const MatDesc *__restrict__ des
     for (int j = lane; j <= r; j += 32) A[(long long)r * d.ld + j] = P[r * kWLD + j];
 }
 
-void launch_diag128(const MatDesc *d_desc, float *base, int K0, int count, int *err, float *store, cudaStream_t s) {
-  k_diag128<<<count, 256, kDiag128Smem, s>>>(d_desc, base, K0, err, store);
+void launch_diag128(const MatDesc *d_desc, float *base, int K0, int count, int *err, float *store, float *pinv,
+                    cudaStream_t s) {
+  k_diag128<<<count, 256, kDiag128Smem, s>>>(d_desc, base, K0, err, store, pinv);
   count_launch();
 }
 

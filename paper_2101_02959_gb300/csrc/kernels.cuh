@@ -145,7 +145,8 @@ void launch_product(const MatDesc *d_a, const T *A, const MatDesc *d_b, const T 
                     int max_n, const SliceWs &ws, int *err, cudaStream_t s);
 template <typename T>
 void launch_diag(const MatDesc *d_desc, T *base, int K0, int count, int *err, T *store, T *pinv, cudaStream_t s);
-void launch_diag128(const MatDesc *d_desc, float *base, int K0, int count, int *err, float *store, cudaStream_t s);
+void launch_diag128(const MatDesc *d_desc, float *base, int K0, int count, int *err, float *store, float *pinv,
+                    cudaStream_t s);
 
 // The same products for many small matrices: one CTA per task over all its rows (columns)
 template <typename T>

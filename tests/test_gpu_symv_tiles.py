@@ -18,7 +18,7 @@ pytestmark = pytest.mark.gpu
 # over many CTAs) and 256 (a few CTAs a matrix)
 @pytest.mark.parametrize("subs,s", [((2, 2, 2), (1, 1, 1)), ((2, 2, 2), (2, 2, 1)), ((2, 2, 2), (2, 2, 2)),
                                     ((2, 2, 2), (3, 2, 2)), ((2, 2, 2), (5, 5, 5)), ((2, 2, 2), (9, 7, 1)),
-                                    ((2, 1, 1), (4, 4, 4)), ((8, 8, 4), (2, 2, 2))])
+                                    ((2, 1, 1), (4, 4, 4)), ((8, 8, 4), (2, 2, 2)), ((2, 2, 2), (7, 7, 7))])
 def test_mixed_schur_operator_at_tile_edges(subs, s):
     from paper_2101_02959_gb300 import binding, build
     build.build()
