@@ -266,8 +266,8 @@ void coarse_refine64(int np, const T *x0, int ld0, const double *C, double *X, d
 //
 // One cluster of eight CTAs, each with an eighth of the rows, one warp per row; every CTA keeps whole
 // copies of the vectors, which the owners write into all of them.  On one SM the products are bound by
-// its FP64 rate (2 multiply-adds a clock: 35 us for np = 270); spread over eight SMs the launch takes
-// COARSE_AFTER.
+// its FP64 rate (2 multiply-adds a clock); spread over eight SMs the launch takes 14.9 us instead of 37 on
+// the 32x32x16 slab (np = 102).
 constexpr int kCoCta = 8;
 __device__ __forceinline__ void cluster_sync() {
   asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -858,16 +858,21 @@ void launch_small_gemm(int ntasks, int max_n, const GemmTask *tasks, const T *A,
   count_launch();
 }
 
+// Threads per block of the Krylov row loops on the fixed reduction grid: bound by the chain of loads of a
+// row (ptr, idx, value), so the blocks grow until a thread has one row.  The 318,000 interface rows of the
+// 128x128x32 slab: 173.0 ms a step with 256 threads, 170.0 so; up to 77,824 rows nothing changes.
+static int row_threads(int n) { return n <= 256 * kRedBlocks ? 256 : n <= 512 * kRedBlocks ? 512 : 1024; }
+
 void launch_gather_sum_dot(int n, const int *ptr, const int *idx, const double *src, double *y, int zero,
                            const DotFuse &f, cudaStream_t s) {
   if (n == 0) return;
-  launch_pdl(k_gather_sum_dot, std::min(ceil_div(n, 256), kRedBlocks), 256, 0, s, n, ptr, idx, src, y, zero, f);
+  launch_pdl(k_gather_sum_dot, std::min(ceil_div(n, 256), kRedBlocks), row_threads(n), 0, s, n, ptr, idx, src, y, zero, f);
   count_launch();
 }
 void launch_spmv_dot(int n, const int *ptr, const int *col, const double *val, const double *x, double *y, int zero,
                      const DotFuse &f, cudaStream_t s) {
   if (n == 0) return;
-  launch_pdl(k_spmv_dot, std::min(ceil_div(n, 256), kRedBlocks), 256, 0, s, n, ptr, col, val, x, y, zero, f);
+  launch_pdl(k_spmv_dot, std::min(ceil_div(n, 256), kRedBlocks), row_threads(n), 0, s, n, ptr, col, val, x, y, zero, f);
   count_launch();
 }
 void launch_spmv(int n, const int *ptr, const int *col, const double *val, const double *x, double *y, int zero,
@@ -980,11 +985,11 @@ void launch_pcg_beta(KrylovState *ks, const double *dots, double *hb, cudaStream
 }
 void launch_pcg_xr(int n, const KrylovState *ks, const double *p, const double *q, double *x, double *r,
                    cudaStream_t s) {
-  launch_pdl(k_pcg_xr, std::max(1, std::min(ceil_div(n, 256), kRedBlocks)), 256, 0, s, n, ks, p, q, x, r);
+  launch_pdl(k_pcg_xr, std::max(1, std::min(ceil_div(n, 256), kRedBlocks)), row_threads(n), 0, s, n, ks, p, q, x, r);
   count_launch();
 }
 void launch_pcg_p(int n, const KrylovState *ks, const double *z, double *p, cudaStream_t s) {
-  launch_pdl(k_pcg_p, std::max(1, std::min(ceil_div(n, 256), kRedBlocks)), 256, 0, s, n, ks, z, p);
+  launch_pdl(k_pcg_p, std::max(1, std::min(ceil_div(n, 256), kRedBlocks)), row_threads(n), 0, s, n, ks, z, p);
   count_launch();
 }
 void launch_pcg_dot_step(int n, int which, const double *a0, const double *b0, const double *a1, const double *b1,
