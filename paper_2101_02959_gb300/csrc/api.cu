@@ -1482,7 +1482,7 @@ int solve_t(bd_handle &h, Dense<T> &D, const double *fi, const double *fe, doubl
   launch_trsv<T>(h.nsub, h.shK.max_e, h.d_Kdesc, h.d_vec_off_I, D.K, D.LdK, h.d_fI, h.d_yI, false, s);
   h.prof.end(PROF_TRSV, s, 0.0, 0.0);
   launch_gemv<T>(h.gv_lgi.n, h.gv_lgi.max_rows, h.gv_lgi.max_cols, h.gv_lgi.d, D.K, h.d_yI, nullptr, h.d_yloc, 1.0,
-                 nullptr, s);
+                 nullptr, s, h.d_Kdesc);
   launch_gather_pairs(h.nif / 2, h.d_iface_node, fi, fe, h.d_fG, 1.0, nullptr, s);
   int reason;
   if (h.opt.method == BD_BDDC) {
@@ -1526,7 +1526,7 @@ int solve_t(bd_handle &h, Dense<T> &D, const double *fi, const double *fe, doubl
   }
   // interior recovery: u_I = L_II^-T (y_I - L_GI^T u_G)
   launch_gemv_t<T>(h.gv_lgit.n, h.gv_lgit.max_rows, h.gv_lgit.max_cols, h.gv_lgit.d, D.K, h.d_uG, h.d_R, h.d_yI, -1.0,
-                   nullptr, s);
+                   nullptr, s, nullptr, h.d_Kdesc);
   h.prof.begin(PROF_TRSV, s);
   launch_trsv<T>(h.nsub, h.shK.max_e, h.d_Kdesc, h.d_vec_off_I, D.K, D.LdK, h.d_yI, h.d_fI, true, s);
   h.prof.end(PROF_TRSV, s, 0.0, 0.0);
@@ -1578,7 +1578,7 @@ void guess_interior_t(bd_handle &h, Dense<T> &D, int) {
   launch_gather_pairs(h.nint_nodes, h.d_int_node, h.d_ri, h.d_re, h.d_fI, -1.0, nullptr, s);
   launch_trsv<T>(h.nsub, h.shK.max_e, h.d_Kdesc, h.d_vec_off_I, D.K, D.LdK, h.d_fI, h.d_yI, false, s);
   launch_gemv_t<T>(h.gv_lgit.n, h.gv_lgit.max_rows, h.gv_lgit.max_cols, h.gv_lgit.d, D.K, h.d_dG, h.d_R, h.d_yI, -1.0,
-                   nullptr, s);
+                   nullptr, s, nullptr, h.d_Kdesc);
   launch_trsv<T>(h.nsub, h.shK.max_e, h.d_Kdesc, h.d_vec_off_I, D.K, D.LdK, h.d_yI, h.d_fI, true, s);
   launch_scatter_pairs(h.nint_nodes, h.d_int_node, h.d_fI, h.d_gi, h.d_ge, s);
   launch_scatter_pairs(h.nif / 2, h.d_iface_node, h.d_dG, h.d_gi, h.d_ge, s);

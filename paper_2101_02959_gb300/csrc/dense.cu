@@ -502,21 +502,25 @@ void engine_partial_cholesky(const EngineShape &sh, const MatDesc *d_desc, T *ba
 
 // ---- batched GEMV ------------------------------------------------------------
 // One CTA (8 warps) per (task, block of kGemvRows rows): each warp owns two rows
-// with independent accumulators; x is staged in shared memory.
+// with independent accumulators; x is staged in shared memory.  prof (interface rows of the local
+// factors only): row g of matrix b is zero left of prof[b].ifirst[g], non-decreasing, and not read there
+// (the 128x128x32 slab's 1,024 matrices: 382 -> 271 us).
 constexpr int kGemvRows = 16;
 
 template <typename T>
 __global__ void __launch_bounds__(256) k_gemv(const GemvDesc *__restrict__ tasks, const T *__restrict__ A,
                                               const double *__restrict__ x, const int *__restrict__ xidx,
-                                              double *__restrict__ y, double alpha, const int *__restrict__ done) {
+                                              double *__restrict__ y, double alpha, const int *__restrict__ done,
+                                              const MatDesc *__restrict__ prof) {
   pdl_wait();
   if (done && *done) return;
   const GemvDesc t = tasks[blockIdx.y];
   const int rbeg = blockIdx.x * kGemvRows;
   if (rbeg >= t.rows) return;
+  const int first = prof && prof[blockIdx.y].ifirst ? prof[blockIdx.y].ifirst[rbeg] & ~63 : 0;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T *xs = reinterpret_cast<T *>(smem_raw);
-  for (int c = threadIdx.x; c < t.cols; c += blockDim.x)
+  for (int c = first + threadIdx.x; c < t.cols; c += blockDim.x)
     xs[c] = (T)((t.flags & 1) ? x[xidx[t.x_off + c]] : x[t.x_off + c]);
   __syncthreads();
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -525,7 +529,7 @@ __global__ void __launch_bounds__(256) k_gemv(const GemvDesc *__restrict__ tasks
   const T *row0 = A + t.a_off + (long long)(v0 ? r0 : rbeg) * t.ld;
   const T *row1 = A + t.a_off + (long long)(v1 ? r1 : rbeg) * t.ld;
   T a0 = T(0), a1 = T(0), b0 = T(0), b1 = T(0);
-  int c = lane;
+  int c = first + lane;
   for (; c + 32 < t.cols; c += 64) {
     const T x0 = xs[c], x1 = xs[c + 32];
     a0 += row0[c] * x0;
@@ -1003,45 +1007,63 @@ void launch_symv_fix(int ntasks, int max_n, const SymvTask *d_tasks, const int2 
   count_launch();
 }
 
-// y[a] = (acc ? y[a] : 0) + alpha sum_p A[p][a] x[p]: one CTA per (task, 32 columns);
-// x may instead be a sparse product evaluated while staging (csr.ptr set).
-// lane = column (coalesced rows), the 8 warps split the rows with 4 loads in flight
-// each and add up their partial sums in shared memory in a fixed order.
+// y[a] = (acc ? y[a] : 0) + alpha sum_p A[p][a] x[p]: one CTA per (task, 64 columns);
+// x may instead be a sparse product evaluated while staging (csr.ptr set).  A lane takes two
+// columns (coalesced rows), the 8 warps split the rows with 8 loads in flight each and add up their
+// partial sums in shared memory in a fixed order.  prof as in k_gemv: the rows that reach the CTA's
+// columns come first, and only they are read.  Bound by HBM: 780 us for the interface rows of the
+// 128x128x32 slab's 1,024 matrices before (all rows, four loads in flight, x staged per 32 columns), 364 us now.
+constexpr int kGemvTCols = 64;
 template <typename T>
 __global__ void __launch_bounds__(256) k_gemv_t(const GemvDesc *__restrict__ tasks, const T *__restrict__ A,
                                                 const double *__restrict__ x, const int *__restrict__ xidx,
                                                 double *__restrict__ y, double alpha, const int *__restrict__ done,
-                                                const CsrIn csr) {
+                                                const CsrIn csr, const MatDesc *__restrict__ prof) {
   if (done && *done) return;
   const GemvDesc t = tasks[blockIdx.y];
-  const int c0 = blockIdx.x * 32;
+  const int c0 = blockIdx.x * kGemvTCols;
   if (c0 >= t.cols) return;
+  const int rows = prof ? min(t.rows, profile_rows(prof[blockIdx.y], c0 + kGemvTCols)) : t.rows;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T *xs = reinterpret_cast<T *>(smem_raw);
-  __shared__ T part[8][33];
-  for (int p = threadIdx.x; p < t.rows; p += blockDim.x)
+  __shared__ T part[8][kGemvTCols];
+  for (int p = threadIdx.x; p < rows; p += blockDim.x)
     xs[p] = (T)(csr.ptr ? csr_row(csr, t.x_off + p) : (t.flags & 1) ? x[xidx[t.x_off + p]] : x[t.x_off + p]);
   __syncthreads();
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int a = c0 + lane;
-  const bool va = a < t.cols;
-  const T *col = A + t.a_off + (va ? a : c0);
+  const T *col0 = A + t.a_off + min(c0 + lane, t.cols - 1), *col1 = A + t.a_off + min(c0 + 32 + lane, t.cols - 1);
   const long long ld = t.ld;
-  T a0 = T(0), a1 = T(0), a2 = T(0), a3 = T(0);
-  int p = wid;
-  for (; p + 24 < t.rows; p += 32) {
-    a0 += col[p * ld] * xs[p];
-    a1 += col[(p + 8) * ld] * xs[p + 8];
-    a2 += col[(p + 16) * ld] * xs[p + 16];
-    a3 += col[(p + 24) * ld] * xs[p + 24];
+  T a0 = T(0), a1 = T(0), b0 = T(0), b1 = T(0);
+  for (int p = wid; p < rows; p += 32) {
+    T u[4], v[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int r = min(p + 8 * q, rows - 1);
+      u[q] = col0[r * ld];
+      v[q] = col1[r * ld];
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      if (p + 8 * q < rows) {
+        const T xv = xs[p + 8 * q];
+        if (q & 1) {
+          a1 += u[q] * xv;
+          b1 += v[q] * xv;
+        } else {
+          a0 += u[q] * xv;
+          b0 += v[q] * xv;
+        }
+      }
+    }
   }
-  for (; p < t.rows; p += 8) a0 += col[p * ld] * xs[p];
-  part[wid][lane] = (a0 + a1) + (a2 + a3);
+  part[wid][lane] = a0 + a1;
+  part[wid][32 + lane] = b0 + b1;
   __syncthreads();
-  if (wid == 0 && va) {
+  const int a = c0 + threadIdx.x;
+  if (threadIdx.x < kGemvTCols && a < t.cols) {
     T sum = T(0);
 #pragma unroll
-    for (int k = 0; k < 8; ++k) sum += part[k][lane];
+    for (int k = 0; k < 8; ++k) sum += part[k][threadIdx.x];
     const double v = alpha * (double)sum;
     y[t.y_off + a] = (t.flags & 2) ? y[t.y_off + a] + v : v;
   }
@@ -1252,21 +1274,22 @@ void launch_symv_rows(int n, const T *A, int ld, const double *x, double *y, int
 
 template <typename T>
 void launch_gemv(int ntasks, int max_rows, int max_cols, const GemvDesc *d_tasks, const T *A, const double *x,
-                 const int *xidx, double *y, double alpha, const int *done, cudaStream_t s) {
+                 const int *xidx, double *y, double alpha, const int *done, cudaStream_t s, const MatDesc *prof) {
   if (ntasks == 0 || max_rows == 0) return;
   dim3 g(ceil_div(max_rows, kGemvRows), ntasks);
   const size_t sm = sizeof(T) * (size_t)std::max(1, max_cols);
-  launch_pdl(k_gemv<T>, g, 256, sm, s, d_tasks, A, x, xidx, y, alpha, done);
+  launch_pdl(k_gemv<T>, g, 256, sm, s, d_tasks, A, x, xidx, y, alpha, done, prof);
   count_launch();
 }
 
 template <typename T>
 void launch_gemv_t(int ntasks, int max_rows, int max_cols, const GemvDesc *d_tasks, const T *A, const double *x,
-                   const int *xidx, double *y, double alpha, const int *done, cudaStream_t s, const CsrIn *csr) {
+                   const int *xidx, double *y, double alpha, const int *done, cudaStream_t s, const CsrIn *csr,
+                   const MatDesc *prof) {
   if (ntasks == 0 || max_cols == 0) return;
-  dim3 g(ceil_div(max_cols, 32), ntasks);
+  dim3 g(ceil_div(max_cols, kGemvTCols), ntasks);
   const size_t sm = sizeof(T) * (size_t)std::max(1, max_rows);
-  k_gemv_t<T><<<g, 256, sm, s>>>(d_tasks, A, x, xidx, y, alpha, done, csr ? *csr : CsrIn{});
+  k_gemv_t<T><<<g, 256, sm, s>>>(d_tasks, A, x, xidx, y, alpha, done, csr ? *csr : CsrIn{}, prof);
   count_launch();
 }
 
@@ -1452,7 +1475,7 @@ bool dense_configure() {
   template void engine_partial_cholesky<T>(const EngineShape &, const MatDesc *, T *, int *, cudaStream_t,    \
                                            T *, ProfHook *, int, const SliceWs &, const LookAhead *);                                              \
   template void launch_gemv<T>(int, int, int, const GemvDesc *, const T *, const double *, const int *,        \
-                               double *, double, const int *, cudaStream_t);                                   \
+                               double *, double, const int *, cudaStream_t, const MatDesc *);                  \
   template void launch_symv_rows<T>(int, const T *, int, const double *, double *, int, const int *,           \
                                     cudaStream_t);                                                             \
   template size_t symv_smem<T>(int);                                                                           \
@@ -1462,7 +1485,7 @@ bool dense_configure() {
   template void launch_gemv_t_task<T>(int, int, int, const GemvDesc *, const T *, const double *, const int *, \
                                       double *, double, const int *, cudaStream_t, const CsrIn *);             \
   template void launch_gemv_t<T>(int, int, int, const GemvDesc *, const T *, const double *, const int *,      \
-                                 double *, double, const int *, cudaStream_t, const CsrIn *);                  \
+                                 double *, double, const int *, cudaStream_t, const CsrIn *, const MatDesc *);                  \
   template void launch_trsv<T>(int, int, const MatDesc *, const int *, const T *, const T *, const double *,   \
                                double *, bool, cudaStream_t);
 BD_INST(float)
