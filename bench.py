@@ -303,15 +303,10 @@ def explicit_values_per_sub(n_gamma, n_delta, n_primal):
 # with the first 16 hex digits of the sha256 of the kernel's source text: a figure stands only
 # while that text is unchanged, and is reported as null otherwise.
 TRAFFIC = {
-    "k_rankk_tc": {"bytes_per_launch": None, "sha": None, "file": "tc.cu",
-                   "span": ("__global__ void __launch_bounds__(128, 3) k_rankk_tc(",
-                            "static constexpr int kTcSmem")},
-    # DRAM bytes per library byte (a capture of three launches on the 32x32x16 slab): the operator
-    # and local-solve launches read their matrices once; scaled to a launch by its own bytes
     # DRAM bytes per library byte of the symmetric operator and local-solve products (a capture of
     # four launches on the 4x4x4-subdomain cube at H/h = 8, 0.5 GB of operators: larger than L2)
-    "k_symv_batched": {"dram_per_library_byte": 1.069, "sha": "00ea69ed6e692111", "file": "dense.cu",
-                       "span": ("__global__ void __launch_bounds__(256) k_symv_batched(",
+    "k_symv_batched": {"dram_per_library_byte": 1.070, "sha": "1d81a88213d3927a", "file": "dense.cu",
+                       "span": ("__global__ void __launch_bounds__(256, 2) k_symv_batched(",
                                 "template <typename T>\nsize_t symv_smem(")},
 }
 
@@ -347,6 +342,14 @@ def device_fp32_peak(dev=0):
     return sms * 128 * 2 * mhz * 1e6 / 1e12, f"derived: {sms} SMs (device) x 128 FP32 lanes x 2 flop x {mhz:.0f} MHz"
 
 
+def digit_peak(pk, products):
+    """Peak of the exact digit products: the measured sustained bf16 rate over the products per
+    multiplication (6 for FP32 operands, 34 for FP64)."""
+    src = "bf16_tflops_sustained"
+    return (pk.get(src, 1700.0) / products,
+            f"{'of measured' if src in pk else 'of fallback'}: bf16 sustained / {products} digit products")
+
+
 def equivalent_sides(sub_nodes):
     """H/h of a box subdomain with the same node count as each subdomain ((k + 1)^3 nodes): exact
     for box subdomains, an equivalent size for the pieces of a masked grid."""
@@ -356,7 +359,7 @@ def equivalent_sides(sub_nodes):
 def roofline(prof, regions, w, precision, tc_used, sub_nodes, sub_explicit=None):
     """The dominant part of a step against its roofline, with the method's ALGORITHMIC work:
     the factorisation kernels (panel + rank-k classes) per Jacobian against the tensor pipe
-    (3xTF32) / FP32 / FP64 peak, or the Krylov local-solve GEMVs per iteration against HBM.
+    (exact bf16 digit products) or the FP32 SIMT peak, or the Krylov local-solve GEMVs per iteration against HBM.
     Both figures are returned; `roofline` is the one that takes more of the step."""
     pk = peaks()
     ks = equivalent_sides(sub_nodes)
@@ -376,26 +379,22 @@ def roofline(prof, regions, w, precision, tc_used, sub_nodes, sub_explicit=None)
         if f_capped:  # as for the Krylov bytes below: a fragment's factors cost less than the box's
             algo = lib
         if precision == "mixed" and tc_used:
-            src = "bf16_tflops_sustained" if "bf16_tflops_sustained" in pk else None
-            peak = (pk[src] if src else 1700.0) * 1.1 / 2.25 / 3.0
-            psrc = ("of measured: bf16_tflops_sustained x 1.1/2.25 (tf32) / 3 (hi/lo split)" if src
-                    else "of fallback: 1.7 PF bf16 sustained x 1.1/2.25 / 3")
+            peak, psrc = digit_peak(pk, 6)
             bound = "tensor"
         elif precision == "mixed":
             peak, psrc = device_fp32_peak()
             bound = "alu"
         else:
-            peak, psrc = 1.25, "nominal GB300 FP64 (recipe table)"
-            bound = "alu"
+            peak, psrc = digit_peak(pk, 34)
+            bound = "tensor"
         ach = algo / (f_ms * 1e-3) / 1e12
         out["factorisation"] = {
             "bound": bound, "achieved": ach, "peak": peak, "unit": "TFLOP/s", "frac": ach / peak,
-            "traffic": traffic("k_rankk_tc") if tc_used else None,
+            "traffic": None,
             "traffic_note": ("null: the factorisation is a class of launches of several kernels and shapes; "
-                             "no per-launch DRAM count stands for it (the tensor-core kernel's own capture "
-                             "is summarised in the profiles)"),
-            "kernel": ("k_rankk_tc (or k_rankk128 without tensor cores) + k_bigpanel (+ k_diag_inverse with the "
-                       "tensor-core panel solve): the factorisation launches of a Jacobian"),
+                             "no per-launch DRAM count stands for it"),
+            "kernel": ("k_slice + k_update (k_rankk128 without tensor cores) + k_diag128 + k_panel_rows (k_diag in "
+                       "FP64 and with the tensor-core panels): the factorisation launches of a Jacobian"),
             "peak_source": psrc, "launches": f_launch, "avg_launch_us": f_ms * 1e3 / f_launch,
             "ms_per_jacobian": f_ms / n_jac,
             "algorithmic_flops_per_jacobian": algo / n_jac, "library_flops_per_jacobian": lib / n_jac,
@@ -609,7 +608,7 @@ def main():
         "metric": METRIC, "value": ms, "unit": "ms/time step", "n_gpus": world, "steps": K,
         "warmup": args.warmup, "ms_per_step": ms, "higher_is_better": False, "scaling": "weak",
         "vs_baseline": None,
-        "dtype": "f32 local factors (tf32 tensor cores) + f64 Krylov/Newton/coarse solve" if args.precision == "mixed"
+        "dtype": "f32 local factors (exact bf16 digit products) + f64 Krylov/Newton/coarse solve" if args.precision == "mixed"
         else "f64", "data": "synthetic",
         "config": {"workload": describe(w, nsub), "unknowns": 2 * r["N"], "subdomains": nsub,
                    "method": f"{args.method}-{args.scaling}", "krylov": "pcg", "precision": args.precision,

@@ -158,9 +158,10 @@ typedef struct {
   int learned_guess, mlp_train_steps, mlp_warmup, mlp_epochs;
   double mlp_lr;
   /* BD_MIXED only: 1 = the rank-k Schur updates of the factorisations run on
-   * the tensor cores (tcgen05, TF32 split in hi + lo parts, FP32 accumulation);
-   * 2 = also the rows below every 128-column panel, solved as one tensor-core
-   * product with the inverse of the panel's factored diagonal block */
+   * the tensor cores (tcgen05) as exact products of bf16 digits, at FP32 rounding;
+   * 2 = also the panels, 64 columns wide, whose rows are one tensor-core product
+   * with the inverse of the panel's factored diagonal block.  BD_FP64 always does
+   * both, with the digits of FP64 */
   int use_tensor_cores;
   /* 1 = chord Newton: factorise the Jacobian at the first Newton iterate of a
    * time step and reuse it for the later iterations of that step (every iterate
