@@ -337,7 +337,10 @@ struct bd_handle {
   double *d_uh1i, *d_uh1e, *d_uh2i, *d_uh2e, *d_gi, *d_ge;
   double rtol_scale = 1.0;
   // factorisation tuning (bidomain_autotune): outer panel width, batch groups, tensor cores
-  int tune_ob = 256, tune_groups = 1;
+  // columns of an outer block: 128 with the updates on the tensor cores, which spares in-block updates of
+  // few tiles (Jacobians of the H/h = 12 cube in FP64 61.8 -> 57.9 ms, of the masked shell's mixed step
+  // 68.4 -> 66.6), 256 SIMT (128x128x32 slab: 219 ms a step, 220 with 128)
+  int tune_ob = 128, tune_groups = 1;
   int tune_panel_tc = 0;  // 1: panel solves on the tensor cores too (tensor cores on)
   cudaGraphExec_t pcg_exec[2] = {nullptr, nullptr};  // captured PCG chunk per method
   size_t pcg_nodes[2] = {0, 0};
@@ -1972,6 +1975,7 @@ int bidomain_setup(const bd_mesh *mesh, const bd_conductivity *cond, const bd_io
     ck(cudaEventCreateWithFlags(&h->ev_join, cudaEventDisableTiming), "event");
     if (h->opt.precision != BD_MIXED) h->opt.use_tensor_cores = 0;
     h->tune_panel_tc = h->opt.use_tensor_cores == 2 ? 1 : 0;
+    if (h->opt.precision == BD_MIXED && !h->opt.use_tensor_cores) h->tune_ob = 256;
     if (h->opt.learned_guess && !gemm_tc_configure()) {
       g_last_error = "tensor-core GEMM configuration failed";
       return BD_ERR_CUDA;
