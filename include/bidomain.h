@@ -312,10 +312,10 @@ int bidomain_coarse_solve(bd_handle *h, const double *c, double *z, int nref);
  * Times the whole factorisation sequence of bidomain_linearize (CUDA events,
  * best of two after a warm-up) at the current Jacobian for every combination of
  * outer block width {128, 256, 512} (columns per long-K trailing update; panels
- * are 128 columns), number of subdomain groups the batch is factorised in
+ * are 128 columns, 64 where their rows go to the tensor cores), number of subdomain groups the batch is factorised in
  * {1, 2, 4} and, in BD_MIXED, the arithmetic: SIMT FP32 (tensor_cores = 0), the
  * rank-k updates on the tensor cores (1), or also the rows below every panel solved on
- * the tensor cores as one product with the inverse of the 128 x 128 diagonal block (2);
+ * the tensor cores as one product with the inverse of the 64 x 64 diagonal block (2);
  * keeps the fastest for the handle and leaves the Jacobian factorised with it.
  * Requires bidomain_linearize (or a step) first.  Results are identical up to rounding
  * for every choice. */
