@@ -20,6 +20,7 @@
 
 #include "bidomain.h"
 #include "dd_kernels.cuh"
+#include "digit_ws.h"
 #include "mlp.cuh"
 #include "plan.h"
 

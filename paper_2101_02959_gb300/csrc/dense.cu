@@ -13,6 +13,7 @@
 #include <type_traits>
 #include <vector>
 
+#include "digit_ws.h"
 #include "kernels.cuh"
 
 namespace bd {

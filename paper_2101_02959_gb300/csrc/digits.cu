@@ -29,7 +29,10 @@
 // accumulators' low bits; a time step solved until the FP64 residual stops falling takes 10 Newton
 // iterations instead of 32 (13 with SIMT FP32).
 #include <algorithm>
+#include <stdexcept>
+#include <string>
 
+#include "digit_ws.h"
 #include "kernels.cuh"
 #include "tc_ptx.cuh"
 
@@ -40,16 +43,16 @@ namespace {
 template <typename T> struct Dig;
 template <> struct Dig<double> {
   // digits, weights, K group, tile columns, pipeline stages, columns of an epilogue pass
-  static constexpr int D = 7, W = 8, Grp = 128, N = 64, Stages = 2, Epi = 8;
+  static constexpr int D = DigitDims<double>::D, W = 8, Grp = DigitDims<double>::Grp, N = kUpdN, Stages = 2, Epi = 8;
   static constexpr int ExMin = 60 - 1022;  // smallest row exponent (keeps the scale factor finite)
 };
 template <> struct Dig<float> {
-  static constexpr int D = 3, W = 3, Grp = 64, N = 64, Stages = 4, Epi = 16;
+  static constexpr int D = DigitDims<float>::D, W = 3, Grp = DigitDims<float>::Grp, N = kUpdN, Stages = 4, Epi = 16;
   static constexpr int ExMin = 30 - 126;
 };
-constexpr int kUM = 128;           // tile rows
-constexpr int kUK = 32;            // K elements per pipeline stage (one 64-byte row of bf16)
-constexpr int kBlkBytes = 64 * kUK * 2;  // one digit plane of 64 rows x 32 columns
+constexpr int kUM = kUpdM;         // tile rows
+constexpr int kUK = kUpdK;         // K elements per pipeline stage
+constexpr int kBlkBytes = kDigitBlk;
 template <typename T> constexpr int a_bytes() { return Dig<T>::D * 2 * kBlkBytes; }
 template <typename T> constexpr int stage_bytes() { return a_bytes<T>() + Dig<T>::D * (Dig<T>::N / 64) * kBlkBytes; }
 // warps 0-15 drain the accumulators and write C, 16 loads, 17 issues the MMAs, 18 lists the tiles
@@ -880,30 +883,18 @@ bool digits_configure() {
          cudaFuncSetAttribute(k_diag128, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kDiag128Smem) == cudaSuccess;
 }
 
-// Workspace of the digit planes of one matrix (rows x cols) and of a panel inverse.
-template <typename T>
-static size_t planes_bytes(int rows, int cols) {
-  return (size_t)ceil_div(cols, kUK) * Dig<T>::D * ceil_div(rows, 64) * kBlkBytes;
-}
-static int pad_rows(int rows) { return ceil_div(std::max(rows, 1), kUM) * kUM; }
-template <typename T>
-static size_t rows_bytes(int rows, int cols) {
-  return planes_bytes<T>(pad_rows(rows), cols) + (size_t)ceil_div(cols, Dig<T>::Grp) * pad_rows(rows) * sizeof(int);
-}
-template <typename T>
-static size_t inv_bytes() {
-  return planes_bytes<T>(Dig<T>::N, kPanel64) + Dig<T>::N * sizeof(int);
-}
-static_assert(kPanel64 == 64, "a panel inverse is one scaling group");
-
-template <typename T>
-size_t slice_bytes(int count, int max_rows, int max_e) {
-  return (size_t)std::max(1, count) * (rows_bytes<T>(max_rows, std::min(std::max(max_e, 1), kSliceK)) + inv_bytes<T>());
+// A launch that the workspace cannot hold is refused (an error of the sizes computed at setup).
+static int ws_run(size_t ws_bytes, size_t one, int count) {
+  const int run = digit_run(ws_bytes, one, count);
+  if (run < 1)
+    throw std::length_error("digit workspace of " + std::to_string(ws_bytes) + " bytes, " + std::to_string(one) +
+                            " needed for one matrix");
+  return run;
 }
 
 template <typename T>
 bool slice_fits(int count, int max_rows, int cols, const SliceWs &ws) {
-  return cols <= kSliceK && ws.bytes / (rows_bytes<T>(max_rows, cols) + inv_bytes<T>()) >= (size_t)count;
+  return cols <= kSliceK && upd_layout<T>(count, max_rows, cols).bytes <= ws.bytes;
 }
 
 // Runs of matrices whose planes fit the workspace; the final update (mode 1) also in runs of
@@ -915,15 +906,14 @@ void launch_update(const MatDesc *d_desc, T *base, Upd64 u, int max_rows, int ma
   using C = Dig<T>;
   const bool panel = u.mode == 0 || u.mode == 3;
   const int za = panel ? u.K0 : u.ka, zz = panel ? u.K0 + u.pw : u.kz;
-  const int kmax = std::min(zz - za, kSliceK), nrb = pad_rows(max_rows) / 64;
-  const int run = (int)std::max<size_t>(
-      1, std::min<size_t>((size_t)count, ws.bytes / (rows_bytes<T>(max_rows, kmax) + inv_bytes<T>())));
+  const int kmax = std::min(zz - za, kSliceK), nrb = digit_rows(max_rows) / 64;
+  const int run = ws_run(ws.bytes, upd_layout<T>(1, max_rows, kmax).bytes, count);
   const int nrt = ceil_div(max_rows, kUM), rpc = 256 / (C::Grp / 8), rest = ceil_div(max_cols, C::N) - part.ct0;
   const int nct = part.nct < 0 ? rest : std::min(rest, part.nct), ctas = part.ctas > 0 ? part.ctas : kSms;
   if (nct <= 0) return;
-  unsigned char *sl = ws.mem, *slb = sl + (size_t)run * planes_bytes<T>(nrb * 64, kmax);
-  int *ex = reinterpret_cast<int *>(slb + (size_t)run * planes_bytes<T>(C::N, kPanel64));
-  int *exb = ex + (size_t)run * ceil_div(kmax, C::Grp) * nrb * 64;
+  const UpdLayout lay = upd_layout<T>(run, max_rows, kmax);
+  unsigned char *sl = ws.mem, *slb = sl + lay.inv;
+  int *ex = reinterpret_cast<int *>(sl + lay.ex), *exb = reinterpret_cast<int *>(sl + lay.ex_inv);
   for (int b0 = 0; b0 < count; b0 += run) {
     const int nb = std::min(run, count - b0);
     for (int ka = za; ka < zz; ka += kSliceK) {
@@ -951,11 +941,6 @@ void launch_update(const MatDesc *d_desc, T *base, Upd64 u, int max_rows, int ma
   }
 }
 
-template <typename T>
-size_t product_bytes(int count, int max_n) {
-  return 2 * (size_t)std::max(1, count) * rows_bytes<T>(max_n, std::max(max_n, 1));
-}
-
 // C = A B^T for `count` pairs of n x n matrices (n = desc.m = desc.e; the same n in all three
 // descriptors of a pair), in runs of pairs whose planes fit the workspace.
 template <typename T>
@@ -963,10 +948,10 @@ void launch_product(const MatDesc *d_a, const T *A, const MatDesc *d_b, const T 
                     int max_n, const SliceWs &ws, int *err, cudaStream_t s) {
   if (count <= 0 || max_n <= 0) return;
   using C = Dig<T>;
-  const int nrb = pad_rows(max_n) / 64, nkc = ceil_div(max_n, kUK), ng = ceil_div(max_n, C::Grp);
-  const int run = (int)std::max<size_t>(1, std::min<size_t>((size_t)count, ws.bytes / product_bytes<T>(1, max_n)));
+  const int nrb = digit_rows(max_n) / 64, nkc = ceil_div(max_n, kUK), ng = ceil_div(max_n, C::Grp);
+  const int run = ws_run(ws.bytes, product_bytes<T>(1, max_n), count);
   const int nrt = ceil_div(max_n, kUM), nct = ceil_div(max_n, C::N), rpc = 256 / (C::Grp / 8);
-  const size_t planes = (size_t)run * planes_bytes<T>(nrb * 64, max_n);
+  const size_t planes = (size_t)run * digit_planes<T>(nrb * 64, max_n);
   unsigned char *sl[2] = {ws.mem, ws.mem + planes};
   int *ex[2] = {reinterpret_cast<int *>(ws.mem + 2 * planes), nullptr};
   ex[1] = ex[0] + (size_t)run * ng * nrb * 64;
@@ -984,11 +969,9 @@ void launch_product(const MatDesc *d_a, const T *A, const MatDesc *d_b, const T 
 
 #define BD_DIG_INST(T)                                                                                       \
   template void launch_diag<T>(const MatDesc *, T *, int, int, int *, T *, T *, cudaStream_t);               \
-  template size_t slice_bytes<T>(int, int, int);                                                             \
   template void launch_update<T>(const MatDesc *, T *, Upd64, int, int, int, const SliceWs &, int *,       \
                                  cudaStream_t, const T *, const UpdPart &);                                 \
   template bool slice_fits<T>(int, int, int, const SliceWs &);                                               \
-  template size_t product_bytes<T>(int, int);                                                                \
   template void launch_product<T>(const MatDesc *, const T *, const MatDesc *, const T *, const MatDesc *, T *, int, \
                                   int, const SliceWs &, int *, cudaStream_t);
 BD_DIG_INST(float)

@@ -75,10 +75,7 @@ void launch_gauge_shift(int n, double *ui, double *ue, const double *scal, cudaS
 void launch_sum_partials(int nblk, const double *partial, double *out, cudaStream_t s);
 
 // digits.cu -- rank-k updates and panel solves on the tensor cores by exact digit products.
-constexpr int kPanel64 = 64;   // panel width where the panels too are solved that way
-constexpr int kUpdN = 64;       // columns of an update's tile
-constexpr int kUpdCtas = 152;   // its persistent CTAs, one per SM
-constexpr int kSliceK = 1024;  // columns whose digit planes the workspace holds at a time
+constexpr int kUpdCtas = 152;   // persistent CTAs of an update, one per SM
 struct Upd64 {                 // one update over a batch (modes as in digits.cu); pw: panel width
   int mode, K0, K1, pw, ka, kz;
   int ct0 = 0;                 // first of the launch's column tiles
@@ -129,17 +126,12 @@ size_t dense_smem_limit();  // bytes of shared memory the dense kernels may stag
 
 // digits.cu
 bool digits_configure();
-// workspace of `count` matrices of max_rows rows and max_e eliminated columns at once
-template <typename T>
-size_t slice_bytes(int count, int max_rows, int max_e);
 template <typename T>
 void launch_update(const MatDesc *d_desc, T *base, Upd64 u, int max_rows, int max_cols, int count, const SliceWs &ws,
                    int *err, cudaStream_t s, const T *pinv = nullptr, const UpdPart &part = {});
 // the digit planes of `cols` columns of the whole batch fit the workspace at once
 template <typename T>
 bool slice_fits(int count, int max_rows, int cols, const SliceWs &ws);
-template <typename T>
-size_t product_bytes(int count, int max_n);
 template <typename T>
 void launch_product(const MatDesc *d_a, const T *A, const MatDesc *d_b, const T *B, const MatDesc *d_c, T *C, int count,
                     int max_n, const SliceWs &ws, int *err, cudaStream_t s);
