@@ -808,18 +808,22 @@ void launch_symv_batched(int ntasks, int max_n, const SymvTask *d_tasks, const f
 // then four 32 x 32 -> 64-bit integer multiply-adds per entry, exact, and two FP64 instructions per
 // row and tile.  Packed tiles in the order of k_symv_batched; the same parts, partial vectors
 // and fixed orders.
-__device__ __forceinline__ int2 fix_split(double x, double scale) {  // scale = 2^(55 - e), |x| < 2^e
-  const long long X = __double2ll_rn(x * scale);
-  const int lo = (int)(X & ((1 << 28) - 1)), l = lo - ((lo >> 27) << 28);
-  return make_int2((int)((X - l) >> 28), l);
-}
 __device__ __forceinline__ double pow2(int e) {  // 2^e, e clamped to the normal range
   return __hiloint2double((max(min(e, 1023), -1022) + 1023) << 20, 0);
 }
+// v 2^e, by two factors where 2^e is no normal number (one range test that all lanes share)
+__device__ __forceinline__ double scale2(double v, int e) {
+  if (e < -1022 || e > 1023) return v * pow2(e / 2) * pow2(e - e / 2);
+  return v * pow2(e);
+}
+__device__ __forceinline__ int2 fix_split(double x, int e) {  // |x| < 2^e
+  const long long X = __double2ll_rn(scale2(x, 55 - e));
+  const int lo = (int)(X & ((1 << 28) - 1)), l = lo - ((lo >> 27) << 28);
+  return make_int2((int)((X - l) >> 28), l);
+}
 constexpr int kFixNan = 1 << 20;  // exponent of a tile or segment that holds an infinity or a NaN
-constexpr int kFixMin = -900;     // smallest exponent (keeps the scale factor finite)
 __device__ __forceinline__ int fix_exp(int mag) {  // from the largest top word of the magnitudes
-  return mag >= 0x7ff00000 ? kFixNan : max((mag >> 20) - 1022, kFixMin);
+  return mag >= 0x7ff00000 ? kFixNan : (mag >> 20) - 1022;
 }
 
 // One tile per CTA, grid-stride over a matrix's tiles: task.a_off -> packed tile task.f_off + s.
@@ -849,12 +853,11 @@ __global__ void __launch_bounds__(256) k_fix_tiles(const FixTask *__restrict__ t
     for (int q = 0; q < 8; ++q) mag = max(mag, smax[q]);
     __syncthreads();
     const int e = fix_exp(mag);
-    const double scale = e == kFixNan ? 0.0 : pow2(55 - e);
     if (tid == 0) ex[t.f_off + s] = e;
     int2 *out = tiles + (t.f_off + s) * 1024;
 #pragma unroll
     for (int q = 0; q < 4; ++q)
-      out[(warp + 8 * q) * 32 + lane] = e == kFixNan ? make_int2(0, 0) : fix_split(v[q], scale);
+      out[(warp + 8 * q) * 32 + lane] = e == kFixNan ? make_int2(0, 0) : fix_split(v[q], e);
   }
 }
 
@@ -881,7 +884,7 @@ __global__ void __launch_bounds__(256) k_symv_fix(const SymvTask *__restrict__ t
     const int c = 32 * b + lane;
     const double v = c < n ? ((t.flags & 1) ? x[xidx[t.x_off + c]] : x[t.x_off + c]) : 0.0;
     const int e = fix_exp(__reduce_max_sync(0xffffffffu, __double2hiint(v) & 0x7fffffff));
-    xs[c] = e == kFixNan ? make_int2(0, 0) : fix_split(v, pow2(55 - e));
+    xs[c] = e == kFixNan ? make_int2(0, 0) : fix_split(v, e);
     if (lane == 0) xe[b] = e;
   }
   for (int c = tid; c < 8 * np; c += 256) part[c] = 0.0;
@@ -907,7 +910,7 @@ __global__ void __launch_bounds__(256) k_symv_fix(const SymvTask *__restrict__ t
   auto value = [](long long hh, long long m, long long ll, int ea, int eb) {
     m += (ll + (1 << 27)) >> 28;
     const double v = fma(__ll2double_rn(hh), 268435456.0, __ll2double_rn(m));
-    return (ea == kFixNan || eb == kFixNan) ? __hiloint2double(0x7ff80000, 0) : v * pow2(ea + eb - 82);
+    return (ea == kFixNan || eb == kFixNan) ? __hiloint2double(0x7ff80000, 0) : scale2(v, ea + eb - 82);
   };
   if (s0 < s1) load(s0);
   double racc = 0.0;  // row sums of the current block row

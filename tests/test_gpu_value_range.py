@@ -1,0 +1,36 @@
+"""Operators at the ends of the number range: scaling the data by a power of two scales the result by
+one and changes nothing else, as long as the numbers stay normal.
+"""
+import numpy as np
+import pytest
+
+import synth
+
+pytestmark = pytest.mark.gpu
+
+
+def _solver(w, scale=1.0, **opt):
+    """The cube's problem with every entry of its matrices times `scale`."""
+    from paper_2101_02959_gb300 import binding, build
+    build.build()
+    ionic = dict(synth.IONIC, **{k: synth.IONIC[k] * scale for k in ("G", "eta1", "chi_cm")})
+    return binding.Solver(w, tuple(v * scale for v in synth.SIGMA_I), tuple(v * scale for v in synth.SIGMA_E), ionic,
+                          synth.TAU, **opt)
+
+
+def test_operator_of_small_and_large_vectors():
+    """FP64: the products' fixed-point segments keep all their bits down to the smallest vectors whose
+    result is normal (entries of S_hat are 1e-8 .. 1e-3 here).  Bar 1e-13: 32 x 434 terms of 2^-53 a row
+    sum, and nothing that depends on the scale; the first results that round to subnormals lie below
+    2^-990."""
+    w = synth.workload("cube8ve")
+    s = _solver(w, precision="fp64")
+    ui, ue, wv = synth.initial_state(s.N, 5)
+    s.linearize(ui, ue, wv)
+    x = synth.random_vector(s.sizes["n_iface"], 6)
+    ref = s.schur_apply(x)
+    for k in (-970, -950, -930, -900, -500, 500, 900, 1000):
+        y = np.ldexp(s.schur_apply(np.ldexp(x, k)), -k)
+        assert np.linalg.norm(y - ref) < 1e-13 * np.linalg.norm(ref), k
+    assert not s.schur_apply(np.zeros_like(x)).any()
+    s.close()
