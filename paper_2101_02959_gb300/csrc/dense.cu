@@ -821,7 +821,9 @@ __device__ __forceinline__ int2 fix_split(double x, int e) {  // |x| < 2^e
   const int lo = (int)(X & ((1 << 28) - 1)), l = lo - ((lo >> 27) << 28);
   return make_int2((int)((X - l) >> 28), l);
 }
-constexpr int kFixNan = 1 << 20;  // exponent of a tile or segment that holds an infinity or a NaN
+// exponent of a tile or segment that holds an infinity or a NaN; such a segment of x keeps the FP64
+// numbers themselves, and its products are those of fix_plain
+constexpr int kFixNan = 1 << 20;
 __device__ __forceinline__ int fix_exp(int mag) {  // from the largest top word of the magnitudes
   return mag >= 0x7ff00000 ? kFixNan : (mag >> 20) - 1022;
 }
@@ -863,6 +865,17 @@ __global__ void __launch_bounds__(256) k_fix_tiles(const FixTask *__restrict__ t
 
 __device__ __forceinline__ void mad_wide(long long &acc, int a, int b) { acc += (long long)a * b; }
 
+// sum of the products of 32 entries of a tile (exponent e) with a segment of FP64 numbers: infinities
+// keep their signs as in a plain sum
+__device__ __noinline__ double fix_plain(const int2 *a, int stride, const int2 *x, int e) {
+  double s = 0.0;
+  for (int c = 0; c < 32; ++c) {
+    const int2 t = a[c * stride];
+    s += scale2(fma((double)t.x, 268435456.0, (double)t.y), e - 55) * __hiloint2double(x[c].y, x[c].x);
+  }
+  return s;
+}
+
 __global__ void __launch_bounds__(256) k_symv_fix(const SymvTask *__restrict__ tasks, const int2 *__restrict__ tiles,
                                                   const int *__restrict__ ex, const double *__restrict__ x,
                                                   const int *__restrict__ xidx, double *__restrict__ y, double alpha,
@@ -884,7 +897,7 @@ __global__ void __launch_bounds__(256) k_symv_fix(const SymvTask *__restrict__ t
     const int c = 32 * b + lane;
     const double v = c < n ? ((t.flags & 1) ? x[xidx[t.x_off + c]] : x[t.x_off + c]) : 0.0;
     const int e = fix_exp(__reduce_max_sync(0xffffffffu, __double2hiint(v) & 0x7fffffff));
-    xs[c] = e == kFixNan ? make_int2(0, 0) : fix_split(v, e);
+    xs[c] = e == kFixNan ? make_int2(__double2loint(v), __double2hiint(v)) : fix_split(v, e);
     if (lane == 0) xe[b] = e;
   }
   for (int c = tid; c < 8 * np; c += 256) part[c] = 0.0;
@@ -907,10 +920,12 @@ __global__ void __launch_bounds__(256) k_symv_fix(const SymvTask *__restrict__ t
     e1 = et[s];
   };
   // sum of 32 products as FP64: (h h) 2^56 + (h l + l h) 2^28 + l l, the low part rounded to 2^28
-  auto value = [](long long hh, long long m, long long ll, int ea, int eb) {
+  auto value = [&](long long hh, long long m, long long ll, int ea, const int2 *a, int stride, int seg) {
+    const int eb = xe[seg];
+    if (ea == kFixNan) return __hiloint2double(0x7ff80000, 0);
+    if (eb == kFixNan) return fix_plain(a, stride, xs + 32 * seg, ea);
     m += (ll + (1 << 27)) >> 28;
-    const double v = fma(__ll2double_rn(hh), 268435456.0, __ll2double_rn(m));
-    return (ea == kFixNan || eb == kFixNan) ? __hiloint2double(0x7ff80000, 0) : scale2(v, ea + eb - 82);
+    return scale2(fma(__ll2double_rn(hh), 268435456.0, __ll2double_rn(m)), ea + eb - 82);
   };
   if (s0 < s1) load(s0);
   double racc = 0.0;  // row sums of the current block row
@@ -934,7 +949,7 @@ __global__ void __launch_bounds__(256) k_symv_fix(const SymvTask *__restrict__ t
       mad_wide(m, a.y, b.x);
       mad_wide(ll, a.y, b.y);
     }
-    racc += value(hh, m, ll, e, xe[cj]);
+    racc += value(hh, m, ll, e, tile + lane * 33, 1, cj);
     if (cj < ci) {
       hh = m = ll = 0;
 #pragma unroll 8
@@ -945,7 +960,7 @@ __global__ void __launch_bounds__(256) k_symv_fix(const SymvTask *__restrict__ t
         mad_wide(m, a.y, b.x);
         mad_wide(ll, a.y, b.y);
       }
-      mine[32 * cj + lane] += value(hh, m, ll, e, xe[ci]);
+      mine[32 * cj + lane] += value(hh, m, ll, e, tile + lane, 33, ci);
     }
     if (I != ci || s + 1 == s1) {
       mine[32 * ci + lane] += racc;

@@ -34,3 +34,40 @@ def test_operator_of_small_and_large_vectors():
         assert np.linalg.norm(y - ref) < 1e-13 * np.linalg.norm(ref), k
     assert not s.schur_apply(np.zeros_like(x)).any()
     s.close()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("bad", [np.inf, -np.inf, np.nan])
+def test_infinite_and_nan_entries(precision, bad):
+    """One entry that is no finite number: the rows that one subdomain alone couples to it follow the
+    sign of their entry of S_hat, rows of subdomains that do not hold it stay as they are."""
+    from conftest import oracle_problem
+    prob = oracle_problem("cube8ve")
+    part, dofs = prob.part, prob.dofs
+    s = _solver(synth.workload("cube8ve"), precision=precision)
+    ui, ue, wv = synth.initial_state(s.N, 5)
+    s.linearize(ui, ue, wv)
+    face = next(c for c in range(part.n_cls) if len(part.cls_subs[c]) == 2)
+    g = 2 * dofs.gnode_to_iface[part.cls_nodes[face][0]]
+    e = np.zeros(s.sizes["n_iface"])
+    e[g] = 1.0
+    col = s.schur_apply(e)
+    x = synth.random_vector(e.size, 6)
+    x[g] = 0.0
+    rest = s.schur_apply(x)
+    x[g] = bad
+    y = s.schur_apply(x)
+    gauge = 2 * dofs.gnode_to_iface[part.gauge_node] + 1
+    seen = 0
+    for c in range(part.n_cls):
+        shared = len(set(part.cls_subs[c]) & set(part.cls_subs[face]))
+        rows = np.concatenate([[2 * dofs.gnode_to_iface[n], 2 * dofs.gnode_to_iface[n] + 1] for n in part.cls_nodes[c]])
+        rows = rows[rows != gauge]
+        if shared == 0:
+            assert np.array_equal(y[rows], rest[rows])
+        elif shared == 1:
+            seen += len(rows)
+            assert (col[rows] != 0.0).all()
+            assert np.array_equal(y[rows], col[rows] * bad, equal_nan=True)
+    assert seen > 100
+    s.close()
