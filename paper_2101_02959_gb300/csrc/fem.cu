@@ -332,8 +332,9 @@ __global__ void __launch_bounds__(256, 3) k_residual(
     const double a = fma(p.tau, Ai, q), c = fma(p.tau, Ae, -q);
     ri[x] = a;
     re[x] = c;
-    // d/dv (G v (1 - a v)(1 - b v) + eta1 v w) = G + v (2 g1 + 3 g2 v) + eta1 w
-    if (factor) factor[x] = fma(p.tau, fma(v, fma(v, p.g2, p.g1), p.G) + p.eta1 * w, p.chi_cm);
+    // d/dv (G v (1 - a v)(1 - b v) + eta1 v w) = (G + g1 v) + g2 v^2 + eta1 w, in this order: v = +inf
+    // gives a NaN (g1 < 0 < g2), which the factorisation refuses, and not a pivot of +inf
+    if (factor) factor[x] = fma(p.tau, fma(p.g2, v * v, fma(p.g1, v, p.G)) + p.eta1 * w, p.chi_cm);
     if (ui_out) { ui_out[x] = xi; ue_out[x] = xe; }
     acc += a * a + c * c;
   }

@@ -71,3 +71,21 @@ def test_infinite_and_nan_entries(precision, bad):
             assert np.array_equal(y[rows], col[rows] * bad, equal_nan=True)
     assert seen > 100
     s.close()
+
+
+@pytest.mark.parametrize("precision,tc", [("fp64", 0), ("mixed", 0), ("mixed", 1), ("mixed", 2)])
+@pytest.mark.parametrize("bad", [np.inf, np.nan])
+def test_state_that_is_no_finite_number_is_refused(precision, tc, bad):
+    """A Jacobian at a state with an infinity or a NaN, at the one interior vertex (whose rows only the
+    coarse matrix factorises) and inside a subdomain."""
+    from paper_2101_02959_gb300 import binding
+    s = _solver(synth.workload("cube8ve"), precision=precision, use_tensor_cores=tc)
+    ui, ue, wv = synth.initial_state(s.N, 5)
+    for node in (s.N // 2, 2 * 81 + 2 * 9 + 2):
+        u = ui.copy()
+        u[node] = bad
+        with pytest.raises(binding.BidomainError) as err:
+            s.linearize(u, ue, wv)
+        assert err.value.code == -2  # BD_ERR_NOT_SPD
+    s.linearize(ui, ue, wv)  # the handle goes on
+    s.close()
