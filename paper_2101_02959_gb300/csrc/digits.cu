@@ -44,11 +44,11 @@ template <typename T> struct Dig;
 template <> struct Dig<double> {
   // digits, weights, K group, tile columns, pipeline stages, columns of an epilogue pass
   static constexpr int D = DigitDims<double>::D, W = 8, Grp = DigitDims<double>::Grp, N = kUpdN, Stages = 2, Epi = 8;
-  static constexpr int ExMin = 60 - 1022;  // smallest row exponent (keeps the scale factor finite)
+  static constexpr int ExLow = 60 - 1022;  // below it a row is lifted first (keeps the scale factor finite)
 };
 template <> struct Dig<float> {
   static constexpr int D = DigitDims<float>::D, W = 3, Grp = DigitDims<float>::Grp, N = kUpdN, Stages = 4, Epi = 16;
-  static constexpr int ExMin = 30 - 126;
+  static constexpr int ExLow = 30 - 126;
 };
 constexpr int kUM = kUpdM;         // tile rows
 constexpr int kUK = kUpdK;         // K elements per pipeline stage
@@ -177,11 +177,17 @@ __global__ void __launch_bounds__(256) k_slice(const MatDesc *__restrict__ desc,
 #pragma unroll
   for (int o = TM / 2; o > 0; o >>= 1) mag = max(mag, __shfl_xor_sync(0xffffffffu, mag, o));
   const bool bad = mag_bad(T(0), mag);
-  const int e = max(mag_exp(T(0), mag), C::ExMin);  // every |x| < 2^e
+  const int e = mag > 0 ? mag_exp(T(0), mag) : 0;  // every |x| < 2^e
   if (t == 0) ex[((long long)b * ng + g) * (nrb * 64) + v] = bad ? kExNan : e;
   const int kc = g * (C::Grp / kUK) + (t >> 2);
   if (k0 + (t >> 2) * kUK >= r.ke) return;
-  const T scale = fix_scale(T(0), e);
+  int up = 0;
+  if (e < C::ExLow) {  // a row of very small entries, exact times 2^60
+    up = 60;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) x[q] *= T(1ll << 60);
+  }
+  const T scale = fix_scale(T(0), max(e + up, C::ExLow));
   uint32_t pk[C::D][4];
 #pragma unroll
   for (int q = 0; q < 8; q += 2) {
@@ -250,7 +256,7 @@ struct Planes {
 
 // Reads one group's accumulators (CPW columns from taddr) and adds sum_w B^(2D-w) P_w 2^(er + ec) to
 // acc; the accumulator of weight w is released on bfree + 8 w once read.
-__device__ __forceinline__ void drain(uint32_t taddr, uint32_t bfree, int lane, int er, const int *ecol,
+__device__ __forceinline__ void drain(uint32_t taddr, uint32_t bfree, int lane, int er, const int *ecol, bool,
                                       double (&acc)[16]) {
   long long I[16];
   // the 64-bit sum in steps of three weights, 256 (256 P_w + P_(w+1)) + P_(w+2)
@@ -296,10 +302,12 @@ __device__ __forceinline__ void drain(uint32_t taddr, uint32_t bfree, int lane, 
     acc[q] = fma(__ll2double_rn(I[q]), sc, acc[q]);
   }
 }
-__device__ __forceinline__ float half_scale(int e) {  // 2^(e - 17), NaN for a marked row
-  return e == kExNan ? __int_as_float(0x7fc00000) : __int_as_float((e - 17 + 127) << 23);
+__device__ __forceinline__ float half_scale(int e) {  // 2^(e - 17), subnormal below e = -109; NaN for a marked row
+  return e == kExNan ? __int_as_float(0x7fc00000) : __int_as_float(e >= -109 ? (e - 17 + 127) << 23 : 1 << (e + 132));
 }
-__device__ __forceinline__ void drain(uint32_t taddr, uint32_t bfree, int lane, int er, const int *ecol,
+// low: a row or column of the warp lies below 2^-46, where the factor 2^(er + ec - 34) of all products may
+// be no normal number
+__device__ __forceinline__ void drain(uint32_t taddr, uint32_t bfree, int lane, int er, const int *ecol, bool low,
                                       float (&acc)[Dig<float>::N / 4]) {
   constexpr int N = Dig<float>::N, NH = N / 64;
   const float fr = half_scale(er);
@@ -316,11 +324,23 @@ __device__ __forceinline__ void drain(uint32_t taddr, uint32_t bfree, int lane, 
       if (lane < 3) tcp::mbar_arrive(bfree + 8 * lane);
     }
     // unit of weight 4: 2^(er + ec - 52) 512^2 = 2^(er - 17) 2^(ec - 17)
+    float p[16];
 #pragma unroll
-    for (int q = 0; q < 16; ++q) {
-      const float p = fmaf(fmaf(__uint_as_float(t2[q]), 512.f, __uint_as_float(t3[q])), 512.f, __uint_as_float(t4[q]));
-      acc[16 * hf + q] = fmaf(p, fr * __int_as_float(ecol[16 * hf + q]), acc[16 * hf + q]);
+    for (int q = 0; q < 16; ++q)
+      p[q] = fmaf(fmaf(__uint_as_float(t2[q]), 512.f, __uint_as_float(t3[q])), 512.f, __uint_as_float(t4[q]));
+    float f2 = fr;
+    if (low) {
+      // a small row's factor on the sum, a large one's on the column's: no partial product leaves the
+      // range that the result has
+      const bool small = er < 0 || er == kExNan;
+      const float f1 = small ? fr : 1.f / 65536.f;
+      f2 = small ? 1.f : __int_as_float((er - 1 + 127) << 23);
+#pragma unroll
+      for (int q = 0; q < 16; ++q) p[q] *= f1;
     }
+#pragma unroll
+    for (int q = 0; q < 16; ++q)
+      acc[16 * hf + q] = fmaf(p[q], f2 * __int_as_float(ecol[16 * hf + q]), acc[16 * hf + q]);
   }
 }
 
@@ -507,6 +527,7 @@ __global__ void __launch_bounds__(kUThreads, 1) k_update(const MatDesc *__restri
         int er1 = exr[(long long)g0 * rstep], ec1 = exc[(long long)g0 * cstep];
         for (int g = g0; g < g1; ++g, ++G) {
           const int er = er1;
+          const bool low = sizeof(T) == 4 && __any_sync(0xffffffffu, er < -46 || ec1 < -46);
           ecol[lane % CPW] = sizeof(T) == 8 ? ec1 : __float_as_int(half_scale(ec1));
           __syncwarp();
           if (g + 1 < g1) {
@@ -515,7 +536,7 @@ __global__ void __launch_bounds__(kUThreads, 1) k_update(const MatDesc *__restri
           }
           ok = ok && tcp::mbar_wait(bacc, G & 1);
           tcp::fence_after();
-          drain(taddr, bfree, lane, er, ecol, acc);
+          drain(taddr, bfree, lane, er, ecol, low, acc);
           __syncwarp();
         }
         if (!ok) break;

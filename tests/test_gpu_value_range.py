@@ -89,3 +89,23 @@ def test_state_that_is_no_finite_number_is_refused(precision, tc, bad):
         assert err.value.code == -2  # BD_ERR_NOT_SPD
     s.linearize(ui, ue, wv)  # the handle goes on
     s.close()
+
+
+@pytest.mark.parametrize("tc", [0, 1, 2])
+def test_mixed_operators_of_small_and_large_matrices(tc):
+    """All matrices times a power of two (entries of K are 2^-45 .. 2^-17 before).  Bars: the operator
+    1e-6, the preconditioners 1e-5.  At the ends of the range the smallest couplings turn subnormal, at
+    2^-23 or less of their row's largest entry, one FP32 rounding (6e-8) in the operator, times a
+    condition of 1e2 in the preconditioners."""
+    out = {}
+    for k in (0, -90, -80, -60, 60, 100, 124, 130):
+        s = _solver(synth.workload("cube8ve"), 2.0 ** k, precision="mixed", use_tensor_cores=tc)
+        ui, ue, wv = synth.initial_state(s.N, 5)
+        s.linearize(ui, ue, wv)
+        x = synth.random_vector(s.sizes["n_iface"], 6)
+        lam = synth.random_vector(s.sizes["n_lambda"], 7)
+        out[k] = (np.ldexp(s.schur_apply(x), -k), np.ldexp(s.bddc_apply(x), k), np.ldexp(s.fetidp_apply(lam), -k))
+        s.close()
+    for k, got in out.items():
+        for y, ref, bar in zip(got, out[0], (1e-6, 1e-5, 1e-5)):
+            assert np.linalg.norm(y - ref) < bar * np.linalg.norm(ref), k
