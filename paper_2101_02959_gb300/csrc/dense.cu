@@ -811,7 +811,7 @@ void launch_symv_batched(int ntasks, int max_n, const SymvTask *d_tasks, const f
 __device__ __forceinline__ double pow2(int e) {  // 2^e, e clamped to the normal range
   return __hiloint2double((max(min(e, 1023), -1022) + 1023) << 20, 0);
 }
-// v 2^e, by two factors where 2^e is no normal number (one range test that all lanes share)
+// v 2^e, by two factors where 2^e is no normal number
 __device__ __forceinline__ double scale2(double v, int e) {
   if (e < -1022 || e > 1023) return v * pow2(e / 2) * pow2(e - e / 2);
   return v * pow2(e);
@@ -822,7 +822,7 @@ __device__ __forceinline__ int2 fix_split(double x, int e) {  // |x| < 2^e
   return make_int2((int)((X - l) >> 28), l);
 }
 // exponent of a tile or segment that holds an infinity or a NaN; such a segment of x keeps the FP64
-// numbers themselves, and its products are those of fix_plain
+// numbers themselves, and its products are those of fix_special
 constexpr int kFixNan = 1 << 20;
 __device__ __forceinline__ int fix_exp(int mag) {  // from the largest top word of the magnitudes
   return mag >= 0x7ff00000 ? kFixNan : (mag >> 20) - 1022;
@@ -865,13 +865,17 @@ __global__ void __launch_bounds__(256) k_fix_tiles(const FixTask *__restrict__ t
 
 __device__ __forceinline__ void mad_wide(long long &acc, int a, int b) { acc += (long long)a * b; }
 
-// sum of the products of 32 entries of a tile (exponent e) with a segment of FP64 numbers: infinities
-// keep their signs as in a plain sum
-__device__ __noinline__ double fix_plain(const int2 *a, int stride, const int2 *x, int e) {
+// 32 products of a tile (exponent ea) with a segment (eb) where 2^(ea + eb - 82) is no normal number or one
+// of the two is marked; v: their fixed-point sum.  A marked segment holds FP64 numbers: a plain sum, in
+// which infinities keep their signs.
+__device__ __forceinline__ double fix_special(const int2 *a, int stride, const int2 *x, int ea, int eb, double v) {
+  if (ea == kFixNan) return __hiloint2double(0x7ff80000, 0);
+  if (eb != kFixNan) return scale2(v, ea + eb - 82);
   double s = 0.0;
+#pragma unroll 1
   for (int c = 0; c < 32; ++c) {
     const int2 t = a[c * stride];
-    s += scale2(fma((double)t.x, 268435456.0, (double)t.y), e - 55) * __hiloint2double(x[c].y, x[c].x);
+    s += scale2(fma((double)t.x, 268435456.0, (double)t.y), ea - 55) * __hiloint2double(x[c].y, x[c].x);
   }
   return s;
 }
@@ -921,11 +925,12 @@ __global__ void __launch_bounds__(256) k_symv_fix(const SymvTask *__restrict__ t
   };
   // sum of 32 products as FP64: (h h) 2^56 + (h l + l h) 2^28 + l l, the low part rounded to 2^28
   auto value = [&](long long hh, long long m, long long ll, int ea, const int2 *a, int stride, int seg) {
-    const int eb = xe[seg];
-    if (ea == kFixNan) return __hiloint2double(0x7ff80000, 0);
-    if (eb == kFixNan) return fix_plain(a, stride, xs + 32 * seg, ea);
+    const int eb = xe[seg], s = ea + eb - 82;
     m += (ll + (1 << 27)) >> 28;
-    return scale2(fma(__ll2double_rn(hh), 268435456.0, __ll2double_rn(m)), ea + eb - 82);
+    const double v = fma(__ll2double_rn(hh), 268435456.0, __ll2double_rn(m));
+    // one test for all that is rare, shared by the warp
+    if ((unsigned)(s + 1022) > 2045u) return fix_special(a, stride, xs + 32 * seg, ea, eb, v);
+    return v * __hiloint2double((s + 1023) << 20, 0);
   };
   if (s0 < s1) load(s0);
   double racc = 0.0;  // row sums of the current block row
