@@ -109,3 +109,19 @@ def test_mixed_operators_of_small_and_large_matrices(tc):
     for k, got in out.items():
         for y, ref, bar in zip(got, out[0], (1e-6, 1e-5, 1e-5)):
             assert np.linalg.norm(y - ref) < bar * np.linalg.norm(ref), k
+
+
+@pytest.mark.parametrize("tc", [0, 1, 2])
+def test_mixed_pivots_in_the_last_binades(tc):
+    """Pivots of the local and coarse matrices between 2^126 and the end of FP32's range (bars as above:
+    the inverses' smallest entries are subnormal)."""
+    out = []
+    for k in (0, 138):
+        s = _solver(synth.workload("cube8ve"), 2.0 ** k, precision="mixed", use_tensor_cores=tc)
+        ui, ue, wv = synth.initial_state(s.N, 5)
+        s.linearize(ui, ue, wv)
+        x = synth.random_vector(s.sizes["n_iface"], 6)
+        out.append((np.ldexp(s.schur_apply(x), -k), np.ldexp(s.bddc_apply(x), k)))
+        s.close()
+    for ref, y, bar in zip(*out, (1e-6, 1e-5)):
+        assert np.linalg.norm(y - ref) < bar * np.linalg.norm(ref)
