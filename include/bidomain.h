@@ -236,6 +236,10 @@ int bd_options_default(bd_options *opt);
  * cudaStream_t (NULL = the library creates its own).  tau in ms. */
 int bidomain_setup(const bd_mesh *mesh, const bd_conductivity *cond, const bd_ionic *ionic,
                    double tau, const bd_options *opt, void *stream, bd_handle **out);
+/* The handle's stream (a cudaStream_t): the one passed to bidomain_setup or the
+ * library's own, which lives until bidomain_destroy.  A caller that prepares device
+ * buffers on another stream orders them against this one (NULL for h == NULL). */
+void *bidomain_stream(const bd_handle *h);
 int bidomain_sizes(const bd_handle *h, bd_sizes *out);
 int bidomain_index_sets(const bd_handle *h, int which, int64_t *out, int64_t cap, int64_t *len);
 

@@ -30,7 +30,7 @@ IDX = dict(ELEM_SUB=0, NODE_MULT=1, IFACE_NODES=2, CLS_TYPE=3, CLS_PTR=4, CLS_NO
            SUB_DUAL=13, SUB_PRIMAL_PTR=14, SUB_PRIMAL=15, GAUGE=16)
 
 EXPORTED = ["bd_plan_create", "bd_plan_sizes", "bd_plan_index_sets", "bd_plan_destroy", "bd_options_default",
-            "bidomain_setup", "bidomain_sizes", "bidomain_index_sets", "bidomain_set_state",
+            "bidomain_setup", "bidomain_stream", "bidomain_sizes", "bidomain_index_sets", "bidomain_set_state",
             "bidomain_get_state", "bidomain_step", "bidomain_gating", "bidomain_residual", "bidomain_linearize",
             "schur_apply", "bddc_apply", "fetidp_apply", "fetidp_operator", "krylov_solve", "bidomain_profile",
             "bidomain_profile_read", "bidomain_launch_count", "schur_apply_noalloc", "bidomain_mlp_sizes",
@@ -113,6 +113,7 @@ def load(build_if_missing: bool = False):
         "bd_options_default": (I, [C.POINTER(BdOptions)]),
         "bidomain_setup": (I, [C.POINTER(BdMesh), C.POINTER(BdConductivity), C.POINTER(BdIonic), D,
                                C.POINTER(BdOptions), P, C.POINTER(P)]),
+        "bidomain_stream": (P, [P]),
         "bidomain_sizes": (I, [P, C.POINTER(BdSizes)]),
         "bidomain_index_sets": (I, [P, I, P, C.c_int64, C.POINTER(C.c_int64)]),
         "bidomain_set_state": (I, [P, P, P, P, D, I]),
@@ -220,13 +221,6 @@ def _ptr(a, n=None):
     return a.data_ptr(), 1
 
 
-def _same_kind(ref, n):
-    if isinstance(ref, np.ndarray):
-        return np.zeros(n)
-    import torch
-    return torch.zeros(n, dtype=torch.float64, device=ref.device)
-
-
 class Plan:
     """Host-only index sets of a mesh and partition (no GPU needed)."""
 
@@ -293,6 +287,25 @@ class Solver:
         self._check(lib.bidomain_sizes(self._h, C.byref(s)), "bidomain_sizes")
         self.sizes = {k: getattr(s, k) for k, _ in BdSizes._fields_}
         self.N = self.sizes["n_node"]
+        self._stream = lib.bidomain_stream(self._h) or 0
+        self._torch_stream = None
+
+    def _same_kind(self, ref, n):
+        """A zeroed result array where `ref` lives.  On the device it is allocated and filled on the
+        handle's stream, ahead of the call's kernels: on torch's current stream, when that is another
+        one, the fill could run after them, or earlier work there still use the memory."""
+        if isinstance(ref, np.ndarray):
+            return np.zeros(n)
+        import torch
+        cur = torch.cuda.current_stream(ref.device)
+        if cur.cuda_stream == self._stream:
+            return torch.zeros(n, dtype=torch.float64, device=ref.device)
+        if self._torch_stream is None:
+            self._torch_stream = torch.cuda.ExternalStream(self._stream, device=ref.device)
+        with torch.cuda.stream(self._torch_stream):
+            out = torch.zeros(n, dtype=torch.float64, device=ref.device)
+        out.record_stream(cur)  # the caller reads it there: not reused before that work is done
+        return out
 
     def _check(self, code, where):
         _check(code, where, getattr(self, "_h", None))
@@ -314,7 +327,7 @@ class Solver:
 
     def get_state(self, like=None):
         like = np.zeros(1) if like is None else like
-        ui, ue, w = (_same_kind(like, self.N) for _ in range(3))
+        ui, ue, w = (self._same_kind(like, self.N) for _ in range(3))
         t = C.c_double()
         d = _ptr(ui)[1]
         self._check(self._lib.bidomain_get_state(self._h, _ptr(ui)[0], _ptr(ue)[0], _ptr(w)[0], C.byref(t), d),
@@ -338,13 +351,13 @@ class Solver:
         return out
 
     def gating(self, ui, ue, w):
-        out = _same_kind(ui, self.N)
+        out = self._same_kind(ui, self.N)
         (a, d), (b, _), (c, _), (o, _) = _ptr(ui, self.N), _ptr(ue, self.N), _ptr(w, self.N), _ptr(out, self.N)
         self._check(self._lib.bidomain_gating(self._h, a, b, c, o, d), "bidomain_gating")
         return out
 
     def residual(self, stim, t_next, ui, ue, w_next, ui_n, ue_n):
-        out = _same_kind(ui, 2 * self.N)
+        out = self._same_kind(ui, 2 * self.N)
         ps = [_ptr(x, self.N) for x in (ui, ue, w_next, ui_n, ue_n)]
         s = _stim(stim)
         self._check(self._lib.bidomain_residual(self._h, None if s is None else C.byref(s), float(t_next),
@@ -356,7 +369,7 @@ class Solver:
         self._check(self._lib.bidomain_linearize(self._h, a, b, c, d), "bidomain_linearize")
 
     def _apply(self, fn, x, n, name):
-        out = _same_kind(x, n)
+        out = self._same_kind(x, n)
         p, d = _ptr(x, n)
         self._check(fn(self._h, p, _ptr(out)[0], d), name)
         return out
@@ -447,7 +460,7 @@ class Solver:
         return z
 
     def krylov_solve(self, f):
-        out = _same_kind(f, 2 * self.N)
+        out = self._same_kind(f, 2 * self.N)
         st = BdSolveStats()
         p, d = _ptr(f, 2 * self.N)
         code = self._lib.krylov_solve(self._h, p, _ptr(out)[0], d, C.byref(st))

@@ -1995,6 +1995,8 @@ int bidomain_setup(const bd_mesh *mesh, const bd_conductivity *cond, const bd_io
   });
 }
 
+void *bidomain_stream(const bd_handle *h) { return h ? (void *)h->s : nullptr; }
+
 int bidomain_sizes(const bd_handle *h, bd_sizes *out) {
   if (!h || !out) return BD_ERR_ARG;
   return fill_sizes(h->plan, out);
