@@ -297,14 +297,14 @@ class Solver:
         if isinstance(ref, np.ndarray):
             return np.zeros(n)
         import torch
-        cur = torch.cuda.current_stream(ref.device)
-        if cur.cuda_stream == self._stream:
+        # (the raw handle: 0.1 us, torch.cuda.current_stream 1.9 us of a call of 48)
+        if not ref.is_cuda or torch._C._cuda_getCurrentRawStream(ref.device.index) == self._stream:
             return torch.zeros(n, dtype=torch.float64, device=ref.device)
         if self._torch_stream is None:
             self._torch_stream = torch.cuda.ExternalStream(self._stream, device=ref.device)
         with torch.cuda.stream(self._torch_stream):
             out = torch.zeros(n, dtype=torch.float64, device=ref.device)
-        out.record_stream(cur)  # the caller reads it there: not reused before that work is done
+        out.record_stream(torch.cuda.current_stream(ref.device))  # not reused before the caller's work
         return out
 
     def _check(self, code, where):
