@@ -1033,7 +1033,9 @@ void setup_handle(bd_handle &h) {
     };
     h.sv_schur = sset(s_schur);
     h.sv_local = sset(s_local);
-    h.sv_sdd = sset(s_sdd);
+    // S_DeltaDelta serves the FETI-DP preconditioner alone: BDDC handles apply it from the FP64 matrices
+    // (fetidp_apply may be called on any handle) and hold no packed copy
+    if (h.mixed() || h.opt.method == BD_FETIDP) h.sv_sdd = sset(s_sdd);
     // bytes read by the products of one application (the profile's library bytes)
     if (h.sv_schur.n) {
       h.gemv_schur_bytes = 0.0;
