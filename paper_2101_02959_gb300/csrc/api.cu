@@ -20,6 +20,7 @@
 
 #include "bidomain.h"
 #include "dd_kernels.cuh"
+#include "dev_mem.h"
 #include "digit_ws.h"
 #include "mlp.cuh"
 #include "plan.h"
@@ -28,38 +29,10 @@ using namespace bd;
 
 namespace {
 
-struct Status : std::runtime_error {
-  int code;
-  Status(int c, const std::string &m) : std::runtime_error(m), code(c) {}
-};
-
-void ck(cudaError_t e, const char *what) {
-  if (e == cudaErrorMemoryAllocation) throw Status(BD_ERR_NOMEM, what);
-  if (e != cudaSuccess) throw Status(BD_ERR_CUDA, std::string(what) + ": " + cudaGetErrorString(e));
-}
-
-struct DevMem {
-  std::vector<void *> ptrs;
-  template <class X>
-  X *alloc(size_t n) {
-    void *p = nullptr;
-    ck(cudaMalloc(&p, std::max<size_t>(n, 1) * sizeof(X)), "cudaMalloc");
-    ptrs.push_back(p);
-    return static_cast<X *>(p);
-  }
-  template <class X>
-  X *upload(const std::vector<X> &v, cudaStream_t s) {
-    X *p = alloc<X>(v.size());
-    if (!v.empty()) ck(cudaMemcpyAsync(p, v.data(), v.size() * sizeof(X), cudaMemcpyHostToDevice, s), "upload");
-    return p;
-  }
-  ~DevMem() {
-    for (void *p : ptrs) cudaFree(p);
-  }
-};
-
-// workspace of the tensor-core updates
+// workspace of the tensor-core updates: at most so much, less where the device has less
 constexpr size_t kWsCap64 = (size_t)1 << 30, kWsCap32 = (size_t)512 << 20, kWsCapCls = (size_t)256 << 20;
+// left free by what a handle can do without (kernels loaded on first use, captured graphs, events)
+constexpr size_t kSpareBytes = (size_t)256 << 20;
 
 // order from which a deluxe product runs on the tensor cores: FP64 n = 242 took 10.2 ms per Jacobian in
 // SIMT and about 1 ms so; below, a 128 x 64 tile is mostly padding
@@ -101,6 +74,7 @@ struct SymvSet {  // batched symmetric GEMV tasks; n = 0 when their shared memor
   int nfix = 0;
   int2 *tiles = nullptr;
   int *ex = nullptr;
+  long long ntiles = 0;
 };
 void launch_symv(const SymvSet &g, const float *A, const double *x, const int *xidx, double *y, const int *done,
                  cudaStream_t s) {
@@ -297,6 +271,7 @@ struct bd_handle {
   SymvSet sv_schur, sv_local, sv_sdd;  // sv_sdd: the FETI-DP preconditioner's S_DeltaDelta
   // tensor-core factorisation: digit planes of the updates, inverses of the panels' diagonal blocks
   SliceWs ws, ws_cls;  // ws_cls: of the deluxe classes, factorised on the second stream
+  size_t ws_least = 0, ws_want = 0, cls_least = 0, cls_want = 0;  // bytes of one matrix, of whole batches
   // D_C^(j) products: blocks of order kProductMin and more on the tensor cores (FP64, or tensor cores on)
   GemmTask *d_gemm = nullptr, *d_gemm_small = nullptr;
   int n_gemm = 0, n_gemm_small = 0, max_small = 0, n_prod = 0, max_prod = 0;
@@ -500,6 +475,28 @@ void mlp_train_once(bd_handle &h, bool want_loss) {
 // ---------------------------------------------------------------------------
 // setup
 // ---------------------------------------------------------------------------
+// Digit workspaces.  SIMT handles have none until bidomain_autotune tries the tensor cores.
+void alloc_ws(bd_handle &h) {
+  h.ws.mem = h.mem.between(h.ws_least, h.ws_want, kSpareBytes, &h.ws.bytes);
+  h.ws_cls.mem = h.mem.between(h.cls_least, h.cls_want, kSpareBytes, &h.ws_cls.bytes);
+}
+void free_ws(bd_handle &h) {
+  for (SliceWs *w : {&h.ws, &h.ws_cls}) {
+    h.mem.release(w->mem);
+    w->mem = nullptr;
+    w->bytes = 0;
+  }
+}
+// Packed tiles of a set; where the device has no room for them the products are those of k_gemv.
+void alloc_tiles(bd_handle &h, SymvSet &g) {
+  if (!g.ntiles) return;
+  g.tiles = h.mem.optional<int2>((size_t)g.ntiles * 1024, kSpareBytes);
+  g.ex = g.tiles ? h.mem.optional<int>(g.ntiles, kSpareBytes) : nullptr;
+  if (g.ex) return;
+  h.mem.release(g.tiles);
+  g = SymvSet{};
+}
+
 void setup_handle(bd_handle &h) {
   Plan &p = h.plan;
   cudaStream_t s = h.s;
@@ -875,7 +872,7 @@ void setup_handle(bd_handle &h) {
     h.d_Codesc = m.upload(std::vector<MatDesc>{co}, s);
     h.shCo = EngineShape{1, np, 2 * np, {2 * np}, {np}};
     h.shCo.id0 = {np};
-    {  // (in mixed precision the autotuner may turn the tensor cores on)
+    {  // workspace sizes; the memory itself last of all (alloc_ws)
       size_t want = 0, one = 0;
       int most = 1;
       for (const EngineShape *q : {&h.shK, &h.shA, &h.shCo}) {
@@ -886,8 +883,8 @@ void setup_handle(bd_handle &h) {
         one = std::max(one, need(1));
         most = std::max(most, q->count);
       }
-      h.ws.bytes = std::max(one, std::min(want, h.mixed() ? kWsCap32 : kWsCap64));
-      h.ws.mem = m.alloc<unsigned char>(h.ws.bytes);
+      h.ws_least = one;
+      h.ws_want = std::max(one, std::min(want, h.mixed() ? kWsCap32 : kWsCap64));
       const size_t inv = (size_t)kPanel64 * kPanel64 * (h.mixed() ? sizeof(float) : sizeof(double));
       h.ws.pinv = m.alloc<unsigned char>(most * inv);
       // the deluxe classes' factorisation and products run beside the local Neumann factorisation
@@ -895,8 +892,8 @@ void setup_handle(bd_handle &h) {
         return h.mixed() ? std::max(slice_bytes<float>(n, h.shC.max_m, h.shC.max_e), product_bytes<float>(n, h.max_prod))
                          : std::max(slice_bytes<double>(n, h.shC.max_m, h.shC.max_e), product_bytes<double>(n, h.max_prod));
       };
-      h.ws_cls.bytes = std::max(cls(1), std::min(cls(std::max(h.shC.count, h.n_prod)), kWsCapCls));
-      h.ws_cls.mem = m.alloc<unsigned char>(h.ws_cls.bytes);
+      h.cls_least = cls(1);
+      h.cls_want = std::max(cls(1), std::min(cls(std::max(h.shC.count, h.n_prod)), kWsCapCls));
       h.ws_cls.pinv = m.alloc<unsigned char>(std::max(h.shC.count, 1) * inv);
     }
     // sparse pattern of S_PP: the (p, q) pairs that some subdomain couples, with the
@@ -1017,8 +1014,7 @@ void setup_handle(bd_handle &h) {
         }
         g.fix = m.upload(fix, s);
         g.nfix = (int)fix.size();
-        g.tiles = m.alloc<int2>((size_t)off * 1024);
-        g.ex = m.alloc<int>(off);
+        g.ntiles = off;  // the tiles themselves: alloc_tiles
       }
       const int occ = h.mixed() ? symv_occupancy<float>(g.max_n) : symv_occupancy<double>(g.max_n);
       int rows = 0, ctrs = 0;
@@ -1036,16 +1032,6 @@ void setup_handle(bd_handle &h) {
     // S_DeltaDelta serves the FETI-DP preconditioner alone: BDDC handles apply it from the FP64 matrices
     // (fetidp_apply may be called on any handle) and hold no packed copy
     if (h.mixed() || h.opt.method == BD_FETIDP) h.sv_sdd = sset(s_sdd);
-    // bytes read by the products of one application (the profile's library bytes)
-    if (h.sv_schur.n) {
-      h.gemv_schur_bytes = 0.0;
-      for (auto &t : s_schur) h.gemv_schur_bytes += (double)sym_tile_entries(t.n);
-    }
-    if (h.sv_local.n) {
-      h.gemv_local_bytes = 0.0;
-      for (auto &t : s_local) h.gemv_local_bytes += (double)sym_tile_entries(t.n);
-      for (auto &t : g_psi) h.gemv_local_bytes += (double)t.rows * t.cols;
-    }
   }
   h.gv_psit = gset(g_psit);
   h.gv_sdd = gset(g_sdd);
@@ -1145,6 +1131,19 @@ void setup_handle(bd_handle &h) {
   const int io = std::max({2 * N, h.nif, h.nlam});
   for (int i = 0; i < 6; ++i) h.d_io[i] = m.alloc<double>(io);
   if (h.opt.learned_guess) setup_mlp(h);
+  // what a handle can do with less of comes last: planes of fewer matrices at a time, no packed tiles
+  if (!h.mixed() || h.tc()) alloc_ws(h);
+  for (SymvSet *g : {&h.sv_schur, &h.sv_local, &h.sv_sdd}) alloc_tiles(h, *g);
+  // bytes read by the products of one application (the profile's library bytes)
+  if (h.sv_schur.n) {
+    h.gemv_schur_bytes = 0.0;
+    for (auto &t : s_schur) h.gemv_schur_bytes += (double)sym_tile_entries(t.n);
+  }
+  if (h.sv_local.n) {
+    h.gemv_local_bytes = 0.0;
+    for (auto &t : s_local) h.gemv_local_bytes += (double)sym_tile_entries(t.n);
+    for (auto &t : g_psi) h.gemv_local_bytes += (double)t.rows * t.cols;
+  }
   ck(cudaStreamSynchronize(s), "setup");
 }
 
@@ -2290,11 +2289,22 @@ int bidomain_autotune(bd_handle *h, bd_tune_result *out) {
       }
       return best;
     };
+    bool planes = true;  // SIMT handles hold no workspace: for the trials, and longer if they choose it
+    const bool lent = h->mixed() && !h->ws.mem;
+    if (lent) {
+      try {
+        alloc_ws(*h);
+      } catch (const Status &e) {
+        if (e.code != BD_ERR_NOMEM) throw;
+        free_ws(*h);
+        planes = false;
+      }
+    }
     const float base_ms = time_it();
     float best_ms = base_ms;
     int best_ob = ob0, best_g = g0, best_tc = tc0, n = 0;
     for (int tc : {0, 1, 2}) {
-      if (tc && !h->mixed()) continue;
+      if (tc && (!h->mixed() || !planes)) continue;
       for (int ob : {128, 256, 512})
         for (int g : {1, 2, 4}) {
           set_tc(tc);
@@ -2310,6 +2320,10 @@ int bidomain_autotune(bd_handle *h, bd_tune_result *out) {
     h->tune_groups = best_g;
     linearize(*h);
     h->prof.on = prof_on;
+    if (lent && !best_tc) {
+      ck(cudaStreamSynchronize(s), "sync");
+      free_ws(*h);
+    }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     int st = h->check_err();
