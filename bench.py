@@ -443,7 +443,8 @@ def roofline(prof, regions, w, precision, tc_used, sub_nodes, sub_explicit=None)
     dom = max(out, key=lambda c: (prof["panel"]["ms"] + prof["rankk"]["ms"]) if c == "factorisation"
               else prof["gemv"]["ms"])
     r = dict(out[dom])
-    r["measured_in"] = "profiled pass: per-launch CUDA events on the library stream"
+    r["measured_in"] = ("profiled pass: per-launch CUDA events on the library stream, the factorisation's launches "
+                        "one after another (the timed steps overlap some of them)")
     others = {c: v for c, v in out.items() if c != dom}
     return r, others
 

@@ -395,7 +395,9 @@ int schur_apply_noalloc(bd_handle *h, const double *x, double *y);
 /* enable = 1 records a CUDA event pair on the handle's stream around every
  * launch of the kernel classes and around every region above (and clears the
  * totals); enable = 2 records the regions only; 0 stops recording.  Per-launch
- * events are not recorded inside captured CUDA graphs. */
+ * events are not recorded inside captured CUDA graphs.  With 1, the launches of
+ * a Jacobian run one after another on the handle's stream, so that the classes'
+ * times add up; with 0 and 2 some of them overlap on streams of the handle. */
 int bidomain_profile(bd_handle *h, int enable);
 /* out[4] = {launches, total milliseconds, algorithmic flops, algorithmic bytes}
  * summed over the launches of class `which` since profiling was enabled.

@@ -323,6 +323,9 @@ struct bd_handle {
   double gemv_schur_flops = 0, gemv_schur_bytes = 0, gemv_local_flops = 0, gemv_local_bytes = 0;
 
   bool mixed() const { return opt.precision == BD_MIXED; }
+  // the kernel classes are timed one launch after another: their times add up to what the stream took
+  bool serial() const { return prof.on == 1; }
+  const LookAhead *look_ahead() const { return serial() ? nullptr : &ahead; }
   int tc() const { return opt.use_tensor_cores ? 1 + tune_panel_tc : 0; }
   int check_err() {
     int e = 0;
@@ -1169,7 +1172,7 @@ void run_engine_groups(bd_handle &h, const EngineShape &all, const MatDesc *d_de
       g.max_m = std::max(g.max_m, all.m[q]);
       g.max_e = std::max(g.max_e, all.e[q]);
     }
-    engine_partial_cholesky<T>(g, d_desc + a, base, h.d_err, h.s, linv, &h.prof, h.tc(), h.ws, &h.ahead);
+    engine_partial_cholesky<T>(g, d_desc + a, base, h.d_err, h.s, linv, &h.prof, h.tc(), h.ws, h.look_ahead());
   }
 }
 
@@ -1195,7 +1198,7 @@ void linearize_t(bd_handle &h, Dense<T> &D, bool precond) {
   launch_copy<T, T>(h.cp_blk.n, h.cp_blk.max_elems, h.cp_blk.d, D.Aug, D.Blk, s);
   // the deluxe classes need only the blocks just copied: their factorisation and the products D_C^(j)
   // run on the second stream beside the local Neumann factorisation (each is a chain of short launches)
-  cudaStream_t s2 = h.s2;
+  cudaStream_t s2 = h.serial() ? s : h.s2;
   ck(cudaEventRecord(h.ev_fork, s), "record");
   ck(cudaStreamWaitEvent(s2, h.ev_fork, 0), "wait");
   launch_class_aug<T>(h.ncls, h.max_nc, h.d_cls, h.d_pairs, D.Blk, h.d_Cdesc, D.CA, s2);
@@ -1225,7 +1228,7 @@ void linearize_t(bd_handle &h, Dense<T> &D, bool precond) {
   {  // one large matrix: its trailing updates go to the tensor cores like the local ones
     EngineShape co = h.shCo;
     co.ob = h.tune_ob;
-    engine_partial_cholesky<T>(co, h.d_Codesc, D.Co, h.d_err, s, D.LdCo, &h.prof, h.tc(), h.ws, &h.ahead);
+    engine_partial_cholesky<T>(co, h.d_Codesc, D.Co, h.d_err, s, D.LdCo, &h.prof, h.tc(), h.ws, h.look_ahead());
   }
   launch_copy<T, T>(h.cp_coinv.n, h.cp_coinv.max_elems, h.cp_coinv.d, D.Co, D.CoInv, s);
   if (h.d_CoInv64) coarse_refine64<T>(h.np, D.CoInv, pad8(h.np), h.d_Co64d, h.d_CoInv64, h.d_CoW, h.d_CoY, s);
