@@ -74,7 +74,7 @@ struct SymvSet {  // batched symmetric GEMV tasks; n = 0 when their shared memor
   int nfix = 0;
   int2 *tiles = nullptr;
   int *ex = nullptr;
-  long long ntiles = 0;
+  long long ntiles = 0, nex = 0;  // exponents: of the tiles, then of the rows
 };
 void launch_symv(const SymvSet &g, const float *A, const double *x, const int *xidx, double *y, const int *done,
                  cudaStream_t s) {
@@ -494,7 +494,7 @@ void free_ws(bd_handle &h) {
 void alloc_tiles(bd_handle &h, SymvSet &g) {
   if (!g.ntiles) return;
   g.tiles = h.mem.optional<int2>((size_t)g.ntiles * 1024, kSpareBytes);
-  g.ex = g.tiles ? h.mem.optional<int>(g.ntiles, kSpareBytes) : nullptr;
+  g.ex = g.tiles ? h.mem.optional<int>(g.nex, kSpareBytes) : nullptr;
   if (g.ex) return;
   h.mem.release(g.tiles);
   g = SymvSet{};
@@ -1008,13 +1008,19 @@ void setup_handle(bd_handle &h) {
       std::vector<SymvTask> v = in;
       if (!h.mixed()) {
         std::vector<FixTask> fix;
-        long long off = 0;
+        long long off = 0, rows = 0;
         for (SymvTask &t : v) {
           const long long nb = ceil_div(t.n, 32);
           t.f_off = off;
-          fix.push_back(FixTask{t.a_off, off, t.ld, t.n});
+          t.d_off = rows;
           off += nb * (nb + 1) / 2;
+          rows += 32 * nb;
         }
+        for (SymvTask &t : v) {  // the diagonals' exponents behind the tiles'
+          t.d_off += off;
+          fix.push_back(FixTask{t.a_off, t.f_off, t.d_off, t.ld, t.n});
+        }
+        g.nex = off + rows;
         g.fix = m.upload(fix, s);
         g.nfix = (int)fix.size();
         g.ntiles = off;  // the tiles themselves: alloc_tiles

@@ -140,11 +140,11 @@ struct SymvTask {
   long long a_off, b_off;
   int ld, n, nb, x_off, y_off, yb_off, flags;
   int part = 0, nparts = 1, scr = 0, ctr = 0;
-  long long f_off = 0;  // FP64: first packed tile
+  long long f_off = 0, d_off = 0;  // FP64: first packed tile, first exponent of the diagonal scaling
 };
 // A symmetric matrix to be packed as fixed-point tiles (its lower block triangle).
 struct FixTask {
-  long long a_off, f_off;
+  long long a_off, f_off, d_off;
   int ld, n;
 };
 

@@ -802,12 +802,13 @@ void launch_symv_batched(int ntasks, int max_n, const SymvTask *d_tasks, const f
 // ---- FP64 symmetric products in integer arithmetic --------------------------------
 // The FP64 pipe (2 multiply-adds per SM and clock) cannot keep up with HBM: a symmetric product needs
 // 5.4 of them per SM and clock at the copy rate.  So the operators' lower block triangles are kept a
-// second time as 32 x 32 tiles of fixed-point numbers: every tile is scaled by a power of two and
-// rounded once to 55 bits, X = 2^28 h + l with |h|, |l| <= 2^27 (8 bytes, as the FP64 entry, error below
-// 2^-56 of the tile's largest entry); x likewise by segments of 32.  A tile's product with a segment is
-// then four 32 x 32 -> 64-bit integer multiply-adds per entry, exact, and two FP64 instructions per
-// row and tile.  Packed tiles in the order of k_symv_batched; the same parts, partial vectors
-// and fixed orders.
+// second time as 32 x 32 tiles of fixed-point numbers: A = D A' D with D the powers of two of the
+// diagonal's square roots, so that the positive definite A' has |A'_rc| <= 1 whatever the units or the
+// contrast of the two media; every tile of A' is rounded once to 55 bits below its power of two 2^e,
+// X = 2^28 h + l with |h|, |l| <= 2^27 (8 bytes, as the FP64 entry; error at most 2^(e - 56)); D x
+// likewise by segments of 32.  A tile's product with a segment is then four 32 x 32 -> 64-bit integer
+// multiply-adds per entry, exact, and two FP64 instructions per row and tile.  Packed tiles in the order
+// of k_symv_batched; the same parts, partial vectors and fixed orders.
 __device__ __forceinline__ double pow2(int e) {  // 2^e, e clamped to the normal range
   return __hiloint2double((max(min(e, 1023), -1022) + 1023) << 20, 0);
 }
@@ -824,8 +825,16 @@ __device__ __forceinline__ int2 fix_split(double x, int e) {  // |x| < 2^e
 // exponent of a tile or segment that holds an infinity or a NaN; such a segment of x keeps the FP64
 // numbers themselves, and its products are those of fix_special
 constexpr int kFixNan = 1 << 20;
-__device__ __forceinline__ int fix_exp(int mag) {  // from the largest top word of the magnitudes
-  return mag >= 0x7ff00000 ? kFixNan : (mag >> 20) - 1022;
+constexpr int kFixZero = -(1 << 20);
+// the exponent e of a number times 2^se, |v| 2^se < 2^e
+__device__ __forceinline__ int fix_exp(double v, int se) {
+  const int mag = __double2hiint(v) & 0x7fffffff;
+  return (mag | __double2loint(v)) == 0 ? kFixZero : mag >= 0x7ff00000 ? kFixNan : (mag >> 20) - 1022 + se;
+}
+// D's exponent from a diagonal entry: half of its own, rounded up
+__device__ __forceinline__ int fix_half(double v) {
+  const int e = fix_exp(v, 0);
+  return e == kFixZero || e == kFixNan ? 0 : (e + 1) >> 1;
 }
 
 // One tile per CTA, grid-stride over a matrix's tiles: task.a_off -> packed tile task.f_off + s.
@@ -833,33 +842,43 @@ __global__ void __launch_bounds__(256) k_fix_tiles(const FixTask *__restrict__ t
                                                    int2 *__restrict__ tiles, int *__restrict__ ex) {
   const FixTask t = tasks[blockIdx.y];
   const int nb = (t.n + 31) >> 5, ntiles = nb * (nb + 1) / 2;
-  __shared__ int smax[8];
+  __shared__ int smax[8], half[64];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   for (int s = blockIdx.x; s < ntiles; s += gridDim.x) {
     int I = (int)((sqrtf(8.f * s + 1.f) - 1.f) * 0.5f);
     while ((I + 1) * (I + 2) / 2 <= s) ++I;
     while (I * (I + 1) / 2 > s) --I;
     const int J = s - I * (I + 1) / 2;
+    if (tid < 64) {  // D of the tile's rows, then of its columns; a diagonal tile stores it
+      const int r = 32 * (tid < 32 ? I : J) + lane;
+      half[tid] = r < t.n ? fix_half(A[t.a_off + (long long)r * (t.ld + 1)]) : 0;
+      if (I == J && tid < 32) ex[t.d_off + r] = half[tid];
+    }
     double v[4];
-    int mag = 0;
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const int r = 32 * I + warp + 8 * q, c = 32 * J + lane;
       v[q] = r < t.n && c < t.n ? A[t.a_off + (long long)r * t.ld + c] : 0.0;
-      mag = max(mag, __double2hiint(v[q]) & 0x7fffffff);
     }
-    mag = __reduce_max_sync(0xffffffffu, mag);
-    if (lane == 0) smax[warp] = mag;
+    __syncthreads();
+    int e = kFixZero, se[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      se[q] = half[warp + 8 * q] + half[32 + lane];
+      e = max(e, fix_exp(v[q], -se[q]));
+    }
+    e = __reduce_max_sync(0xffffffffu, e);
+    if (lane == 0) smax[warp] = e;
     __syncthreads();
 #pragma unroll
-    for (int q = 0; q < 8; ++q) mag = max(mag, smax[q]);
+    for (int q = 0; q < 8; ++q) e = max(e, smax[q]);
     __syncthreads();
-    const int e = fix_exp(mag);
+    if (e == kFixZero) e = 0;
     if (tid == 0) ex[t.f_off + s] = e;
     int2 *out = tiles + (t.f_off + s) * 1024;
 #pragma unroll
     for (int q = 0; q < 4; ++q)
-      out[(warp + 8 * q) * 32 + lane] = e == kFixNan ? make_int2(0, 0) : fix_split(v[q], e);
+      out[(warp + 8 * q) * 32 + lane] = e == kFixNan ? make_int2(0, 0) : fix_split(v[q], e + se[q]);
   }
 }
 
@@ -897,11 +916,19 @@ __global__ void __launch_bounds__(256) k_symv_fix(const SymvTask *__restrict__ t
   int2 *stage = reinterpret_cast<int2 *>(xe + ((nb + 3) & ~3));  // [8][32][33]
   __shared__ int last;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int *dx = ex + t.d_off;  // exponents of D
   for (int b = warp; b < nb; b += 8) {
     const int c = 32 * b + lane;
     const double v = c < n ? ((t.flags & 1) ? x[xidx[t.x_off + c]] : x[t.x_off + c]) : 0.0;
-    const int e = fix_exp(__reduce_max_sync(0xffffffffu, __double2hiint(v) & 0x7fffffff));
-    xs[c] = e == kFixNan ? make_int2(__double2loint(v), __double2hiint(v)) : fix_split(v, e);
+    const int se = dx[c];
+    int e = __reduce_max_sync(0xffffffffu, fix_exp(v, se));
+    if (e == kFixZero) e = 0;
+    if (e == kFixNan) {
+      const double w = v * pow2(se);
+      xs[c] = make_int2(__double2loint(w), __double2hiint(w));
+    } else {
+      xs[c] = fix_split(v, e - se);
+    }
     if (lane == 0) xe[b] = e;
   }
   for (int c = tid; c < 8 * np; c += 256) part[c] = 0.0;
@@ -982,7 +1009,7 @@ __global__ void __launch_bounds__(256) k_symv_fix(const SymvTask *__restrict__ t
   };
   if (S == 1) {
     for (int r = tid; r < n; r += 256) {
-      const double o = alpha * column(r);
+      const double o = alpha * (column(r) * pow2(dx[r]));
       y[t.y_off + r] = (t.flags & 2) ? y[t.y_off + r] + o : o;
     }
     return;
@@ -999,7 +1026,7 @@ __global__ void __launch_bounds__(256) k_symv_fix(const SymvTask *__restrict__ t
   for (int r = tid; r < n; r += 256) {
     double v = __ldcg(sums + r);
     for (int q = 1; q < S; ++q) v += __ldcg(sums + (long long)q * ld_scr + r);
-    const double o = alpha * v;
+    const double o = alpha * (v * pow2(dx[r]));
     y[t.y_off + r] = (t.flags & 2) ? y[t.y_off + r] + o : o;
   }
   if (tid == 0) counter[t.ctr] = 0;  // ready for the next launch

@@ -125,3 +125,33 @@ def test_mixed_pivots_in_the_last_binades(tc):
         s.close()
     for ref, y, bar in zip(*out, (1e-6, 1e-5)):
         assert np.linalg.norm(y - ref) < bar * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("contrast", [1e2, 1e4, 1e6, 1e8, 1e-6])
+def test_operator_of_media_of_different_scale(contrast):
+    """FP64 with the extracellular conductivities times a contrast: tiles hold rows of both media, whose
+    entries differ by that factor.  The vector is scaled so that both media give terms of the same size;
+    bar 1e-12 for the rows of each medium by itself: 2^-53 times a condition of 1e3 of the scaled
+    matrices and a growth of ten.  (Entries cut to a common number of bits per tile lost 1e-17 x contrast
+    in the smaller medium's rows: 2e-10 at 1e8.)"""
+    from oracle import ionic
+    from oracle.bidomain import Problem
+    from oracle.dd import DDSolver
+    from paper_2101_02959_gb300 import binding, build
+    build.build()
+    w = synth.workload("cube8ve")
+    se = tuple(v * contrast for v in synth.SIGMA_E)
+    prob = Problem(w, synth.SIGMA_I, se, synth.IONIC, synth.TAU, synth.stimulus(w))
+    ui, ue, wv = synth.initial_state(prob.N, 5)
+    dd = DDSolver(prob)
+    dd.setup(prob.p["chi_cm"] + prob.tau * ionic.di_ion_dv(ui - ue, wv, prob.p))
+    x = synth.random_vector(prob.dofs.n_iface, 6)
+    x[1::2] /= max(contrast, 1.0) ** 0.5
+    x[dd.g_iface] = 0.0
+    ref = dd.schur_apply(x)
+    s = binding.Solver(w, synth.SIGMA_I, se, synth.IONIC, synth.TAU, precision="fp64")
+    s.linearize(ui, ue, wv)
+    y = s.schur_apply(x)
+    s.close()
+    for rows in (slice(0, None, 2), slice(1, None, 2)):
+        assert np.linalg.norm((y - ref)[rows]) < 1e-12 * np.linalg.norm(ref[rows])
