@@ -890,6 +890,7 @@ void setup_handle(bd_handle &h) {
       h.ws_want = std::max(one, std::min(want, h.mixed() ? kWsCap32 : kWsCap64));
       const size_t inv = (size_t)kPanel64 * kPanel64 * (h.mixed() ? sizeof(float) : sizeof(double));
       h.ws.pinv = m.alloc<unsigned char>(most * inv);
+      h.ws.pexp = m.alloc<int>((size_t)most * kPanelExp);
       // the deluxe classes' factorisation and products run beside the local Neumann factorisation
       auto cls = [&](int n) {
         return h.mixed() ? std::max(slice_bytes<float>(n, h.shC.max_m, h.shC.max_e), product_bytes<float>(n, h.max_prod))
@@ -898,6 +899,7 @@ void setup_handle(bd_handle &h) {
       h.cls_least = cls(1);
       h.cls_want = std::max(cls(1), std::min(cls(std::max(h.shC.count, h.n_prod)), kWsCapCls));
       h.ws_cls.pinv = m.alloc<unsigned char>(std::max(h.shC.count, 1) * inv);
+      h.ws_cls.pexp = m.alloc<int>((size_t)std::max(h.shC.count, 1) * kPanelExp);
     }
     // sparse pattern of S_PP: the (p, q) pairs that some subdomain couples, with the
     // offsets of their local contributions in the augmented matrices (subdomain order)

@@ -407,8 +407,8 @@ void engine_partial_cholesky(const EngineShape &sh, const MatDesc *d_desc, T *ba
       }
       if (prof) prof->begin(PROF_PANEL, q);
       if (narrow) {
-        launch_diag<T>(d_desc, base, k0, sh.count, d_err, store, pinv, q);
-        launch_update<T>(d_desc, base, Upd64{3, k0, 0, PW, 0, 0}, max_below, PW, sh.count, w_s, d_err, q, pinv);
+        launch_diag<T>(d_desc, base, k0, sh.count, d_err, store, w_s, q);
+        launch_update<T>(d_desc, base, Upd64{3, k0, 0, PW, 0, 0}, max_below, PW, sh.count, w_s, d_err, q);
       } else if constexpr (!f64) {
         launch_diag128(d_desc, base, k0, sh.count, d_err, store, pinv, q);
         launch_panel_rows(d_desc, base, k0, max_below, sh.count, pinv, q);
@@ -447,11 +447,11 @@ void engine_partial_cholesky(const EngineShape &sh, const MatDesc *d_desc, T *ba
     const Upd64 u{2, K0, K1, PW, K0, K1};
     if (update && look) {
       if (prof) prof->begin(PROF_RANKK, s);
-      launch_update<T>(d_desc, base, u, max_rows, max_cols, sh.count, half[0], d_err, s, nullptr,
+      launch_update<T>(d_desc, base, u, max_rows, max_cols, sh.count, half[0], d_err, s,
                        UpdPart{0, ob / kUpdN, false, 0});
       cudaEventRecord(ahead->cols, s);
       cudaStreamWaitEvent(ahead->s, ahead->cols, 0);
-      launch_update<T>(d_desc, base, u, max_rows, max_cols, sh.count, half[0], d_err, s, nullptr,
+      launch_update<T>(d_desc, base, u, max_rows, max_cols, sh.count, half[0], d_err, s,
                        UpdPart{ob / kUpdN, -1, true, kUpdCtas - kAheadSms});
       if (prof) prof->end(PROF_RANKK, s, fl, by);
       block(K1, ahead->s, half[1]);

@@ -7,6 +7,7 @@
 namespace bd {
 
 constexpr int kPanel64 = 64;   // panel width where the panels too are solved on the tensor cores
+constexpr int kPanelExp = 72;  // ints per matrix for the column exponents of a panel solve, and a flag
 constexpr int kUpdM = 128;     // rows of an update's tile
 constexpr int kUpdN = 64;      // its columns
 constexpr int kUpdK = 32;      // columns of K per digit block (one 64-byte row of bf16)

@@ -133,13 +133,39 @@ __device__ __forceinline__ bool mag_bad(float, int m) { return m >= 0x7f800000; 
 __device__ __forceinline__ double fix_scale(double, int e) { return __hiloint2double((1023 + 55 - e) << 20, 0); }
 __device__ __forceinline__ float fix_scale(float, int e) { return __int_as_float((127 + 26 - e) << 23); }
 
-// One team of Grp / 8 threads per row and group of columns, 8 columns a thread: the row's scale from
-// the largest magnitude of the group, then the digits of every entry.  Bound by memory (the planes
-// written are 14 and 6 bytes per entry) and, for FP64, by one multiply per entry.
+// Scaling of the columns of K in products of two different matrices: C = (A D) (B D^-1)^T with D powers of
+// two, so that entries of columns of different size (the two media) keep their bits below the row's
+// largest.  Panel solve: D from the diagonal of the block's inverse, as k_diag leaves it (kPanelExp ints
+// per matrix: the exponents, and 0 behind them where they differ by three or less and nothing is scaled:
+// FP64 multiplies on every entry cost the H/h = 12 cube 2 of 78 ms).  Plain product: from the square
+// roots of B's diagonal.
+template <typename T>
+struct ColScale {
+  const int *pexp = nullptr;      // panel solve
+  const T *B = nullptr;           // plain product, with B's descriptors
+  const MatDesc *desc = nullptr;
+  int sign = 1;                   // +1 for A, -1 for B
+};
+__device__ __forceinline__ double exp2i(double, int e) { return __hiloint2double((e + 1023) << 20, 0); }
+__device__ __forceinline__ float exp2i(float, int e) { return __int_as_float((e + 127) << 23); }
+template <typename T>
+__device__ __forceinline__ T col_factor(const ColScale<T> &c, int b, int k) {
+  int e = 0;
+  if (c.pexp) {
+    e = c.pexp[b * kPanelExp + k];
+  } else {
+    const T v = c.B[c.desc[b].off + (long long)k * (c.desc[b].ld + 1)];
+    const int m = mag_bits(v);
+    if (m > 0 && !mag_bad(v, m)) e = (mag_exp(v, m) + 1) >> 1;
+  }
+  constexpr int most = sizeof(T) == 8 ? 1000 : 120;
+  return exp2i(T(0), c.sign * max(-most, min(e, most)));
+}
+
 template <typename T>
 __global__ void __launch_bounds__(256) k_slice(const MatDesc *__restrict__ desc, const T *__restrict__ base,
                                                Upd64 u, const T *__restrict__ pinv, unsigned char *__restrict__ sl,
-                                               int *__restrict__ ex, int nrb, int nkc, int ng) {
+                                               int *__restrict__ ex, int nrb, int nkc, int ng, ColScale<T> cs) {
   using C = Dig<T>;
   constexpr int TM = C::Grp / 8, RPC = 256 / TM;  // threads of a team, rows per CTA
   const int b = blockIdx.z, g = blockIdx.y;
@@ -170,6 +196,11 @@ __global__ void __launch_bounds__(256) k_slice(const MatDesc *__restrict__ desc,
   } else {
 #pragma unroll
     for (int q = 0; q < 8; ++q) x[q] = (valid && k + q < r.ke) ? src[k + q] : T(0);
+  }
+  if (cs.pexp ? cs.pexp[b * kPanelExp + kPanel64] != 0 : cs.B != nullptr) {
+#pragma unroll
+    for (int q = 0; q < 8; ++q)
+      if (k + q < r.ke) x[q] *= col_factor(cs, b, k + q - r.kb);
   }
   int mag = 0;
 #pragma unroll
@@ -681,7 +712,8 @@ __device__ __forceinline__ void ldl_inv32(T *P, T *Y, int s, int lane, T (*Lc)[2
 
 template <typename T>
 __global__ void __launch_bounds__(256) k_diag(const MatDesc *__restrict__ desc, T *__restrict__ base, int K0,
-                                              int *__restrict__ err, T *__restrict__ store, T *__restrict__ pinv) {
+                                              int *__restrict__ err, T *__restrict__ store, T *__restrict__ pinv,
+                                              int *__restrict__ pexp) {
   const MatDesc d = desc[blockIdx.x];
   if (K0 >= d.e) return;
   const int w = min(kDP, d.e - K0);
@@ -767,6 +799,27 @@ __global__ void __launch_bounds__(256) k_diag(const MatDesc *__restrict__ desc, 
   __syncthreads();
   if (bad && lane == 0) atomicOr(err, DEV_ERR_NOT_SPD);
   T *out = pinv + (long long)blockIdx.x * kDP * kDP;
+  if (tid < 32) {  // exponents of the inverse's diagonal, for the column scaling of the panel solve
+    int e[2], lo = 1 << 20, hi = -(1 << 20);
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      const int i = lane + 32 * c;
+      const T y = Y[i * kDLD + i];
+      const int m = mag_bits(y);
+      const bool use = i < w && m > 0 && !mag_bad(y, m);
+      e[c] = use ? mag_exp(y, m) : 0;
+      if (use) {
+        lo = min(lo, e[c]);
+        hi = max(hi, e[c]);
+      }
+    }
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    int *pe = pexp + blockIdx.x * kPanelExp;
+    pe[lane] = e[0];
+    pe[lane + 32] = e[1];
+    if (lane == 0) pe[kPanel64] = hi - lo > 3;
+  }
 #pragma unroll 4
   for (int q = tid; q < kDP * kDP; q += 256) {
     const int i = q / kDP, j = q % kDP;
@@ -895,8 +948,9 @@ void launch_diag128(const MatDesc *d_desc, float *base, int K0, int count, int *
 }
 
 template <typename T>
-void launch_diag(const MatDesc *d_desc, T *base, int K0, int count, int *err, T *store, T *pinv, cudaStream_t s) {
-  k_diag<T><<<count, 256, diag_smem<T>(), s>>>(d_desc, base, K0, err, store, pinv);
+void launch_diag(const MatDesc *d_desc, T *base, int K0, int count, int *err, T *store, const SliceWs &ws,
+                 cudaStream_t s) {
+  k_diag<T><<<count, 256, diag_smem<T>(), s>>>(d_desc, base, K0, err, store, static_cast<T *>(ws.pinv), ws.pexp);
   count_launch();
 }
 
@@ -928,7 +982,7 @@ bool slice_fits(int count, int max_rows, int cols, const SliceWs &ws) {
 // kSliceK columns (each run rounds C once more, so they are long).
 template <typename T>
 void launch_update(const MatDesc *d_desc, T *base, Upd64 u, int max_rows, int max_cols, int count,
-                   const SliceWs &ws, int *err, cudaStream_t s, const T *pinv, const UpdPart &part) {
+                   const SliceWs &ws, int *err, cudaStream_t s, const UpdPart &part) {
   if (max_rows <= 0 || max_cols <= 0 || count <= 0) return;
   using C = Dig<T>;
   const bool panel = u.mode == 0 || u.mode == 3;
@@ -950,14 +1004,17 @@ void launch_update(const MatDesc *d_desc, T *base, Upd64 u, int max_rows, int ma
       q.ct0 = part.ct0;
       const int kw = q.kz - ka, nkc = ceil_div(kw, kUK), ng = ceil_div(kw, C::Grp);
       const Planes pa{sl, ex, nrb, nkc, ng}, pi{slb, exb, C::N / 64, kPanel64 / kUK, 1};
-      if (!part.sliced) {
-        k_slice<T><<<dim3(nrb * 64 / rpc, ng, nb), 256, 0, s>>>(d_desc + b0, base, q, nullptr, sl, ex, nrb, nkc, ng);
-        count_launch();
-      }
       if (u.mode == 3) {
-        const T *pv = pinv + (size_t)b0 * u.pw * u.pw;
+        const T *pv = static_cast<const T *>(ws.pinv) + (size_t)b0 * u.pw * u.pw;
+        const int *pe = ws.pexp + (size_t)b0 * kPanelExp;
+        k_slice<T><<<dim3(nrb * 64 / rpc, ng, nb), 256, 0, s>>>(d_desc + b0, base, q, nullptr, sl, ex, nrb, nkc, ng,
+                                                                     ColScale<T>{pe, nullptr, nullptr, 1});
         k_slice<T><<<dim3(C::N / rpc, 1, nb), 256, 0, s>>>(d_desc + b0, base, q, pv, slb, exb, C::N / 64,
-                                                         kPanel64 / kUK, 1);
+                                                               kPanel64 / kUK, 1, ColScale<T>{pe, nullptr, nullptr, -1});
+        count_launch(2);
+      } else if (!part.sliced) {
+        k_slice<T><<<dim3(nrb * 64 / rpc, ng, nb), 256, 0, s>>>(d_desc + b0, base, q, nullptr, sl, ex, nrb, nkc, ng,
+                                                                      ColScale<T>{});
         count_launch();
       }
       const int per = nrt * nct, total = per * nb;
@@ -985,8 +1042,10 @@ void launch_product(const MatDesc *d_a, const T *A, const MatDesc *d_b, const T 
   const Upd64 u{4, 0, 0, 0, 0, max_n};
   for (int b0 = 0; b0 < count; b0 += run) {
     const int nb = std::min(run, count - b0), per = nrt * nct, total = per * nb;
-    k_slice<T><<<dim3(nrb * 64 / rpc, ng, nb), 256, 0, s>>>(d_a + b0, A, u, nullptr, sl[0], ex[0], nrb, nkc, ng);
-    k_slice<T><<<dim3(nrb * 64 / rpc, ng, nb), 256, 0, s>>>(d_b + b0, B, u, nullptr, sl[1], ex[1], nrb, nkc, ng);
+    k_slice<T><<<dim3(nrb * 64 / rpc, ng, nb), 256, 0, s>>>(d_a + b0, A, u, nullptr, sl[0], ex[0], nrb, nkc, ng,
+                                                           ColScale<T>{nullptr, B, d_b + b0, 1});
+    k_slice<T><<<dim3(nrb * 64 / rpc, ng, nb), 256, 0, s>>>(d_b + b0, B, u, nullptr, sl[1], ex[1], nrb, nkc, ng,
+                                                           ColScale<T>{nullptr, B, d_b + b0, -1});
     k_update<T><<<std::min(total, kSms), kUThreads, update_smem<T>(), s>>>(
         d_a + b0, d_c + b0, Cm, u, Planes{sl[0], ex[0], nrb, nkc, ng}, Planes{sl[1], ex[1], nrb, nkc, ng}, nct, per, total,
         err);
@@ -995,9 +1054,9 @@ void launch_product(const MatDesc *d_a, const T *A, const MatDesc *d_b, const T 
 }
 
 #define BD_DIG_INST(T)                                                                                       \
-  template void launch_diag<T>(const MatDesc *, T *, int, int, int *, T *, T *, cudaStream_t);               \
+  template void launch_diag<T>(const MatDesc *, T *, int, int, int *, T *, const SliceWs &, cudaStream_t);   \
   template void launch_update<T>(const MatDesc *, T *, Upd64, int, int, int, const SliceWs &, int *,       \
-                                 cudaStream_t, const T *, const UpdPart &);                                 \
+                                 cudaStream_t, const UpdPart &);                                 \
   template bool slice_fits<T>(int, int, int, const SliceWs &);                                               \
   template void launch_product<T>(const MatDesc *, const T *, const MatDesc *, const T *, const MatDesc *, T *, int, \
                                   int, const SliceWs &, int *, cudaStream_t);

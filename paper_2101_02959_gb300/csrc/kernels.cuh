@@ -91,6 +91,7 @@ struct SliceWs {               // workspace: digit planes and row exponents; a p
   unsigned char *mem = nullptr;
   size_t bytes = 0;
   void *pinv = nullptr;
+  int *pexp = nullptr;         // exponents of its diagonal, kPanelExp ints per matrix
 };
 
 // dense.cu -- batched partial Cholesky: eliminates the first e columns of every
@@ -128,7 +129,7 @@ size_t dense_smem_limit();  // bytes of shared memory the dense kernels may stag
 bool digits_configure();
 template <typename T>
 void launch_update(const MatDesc *d_desc, T *base, Upd64 u, int max_rows, int max_cols, int count, const SliceWs &ws,
-                   int *err, cudaStream_t s, const T *pinv = nullptr, const UpdPart &part = {});
+                   int *err, cudaStream_t s, const UpdPart &part = {});
 // the digit planes of `cols` columns of the whole batch fit the workspace at once
 template <typename T>
 bool slice_fits(int count, int max_rows, int cols, const SliceWs &ws);
@@ -136,7 +137,7 @@ template <typename T>
 void launch_product(const MatDesc *d_a, const T *A, const MatDesc *d_b, const T *B, const MatDesc *d_c, T *C, int count,
                     int max_n, const SliceWs &ws, int *err, cudaStream_t s);
 template <typename T>
-void launch_diag(const MatDesc *d_desc, T *base, int K0, int count, int *err, T *store, T *pinv, cudaStream_t s);
+void launch_diag(const MatDesc *d_desc, T *base, int K0, int count, int *err, T *store, const SliceWs &ws, cudaStream_t s);
 void launch_diag128(const MatDesc *d_desc, float *base, int K0, int count, int *err, float *store, float *pinv,
                     cudaStream_t s);
 
