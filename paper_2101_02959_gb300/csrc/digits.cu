@@ -135,10 +135,12 @@ __device__ __forceinline__ float fix_scale(float, int e) { return __int_as_float
 
 // Scaling of the columns of K in products of two different matrices: C = (A D) (B D^-1)^T with D powers of
 // two, so that entries of columns of different size (the two media) keep their bits below the row's
-// largest.  Panel solve: D from the diagonal of the block's inverse, as k_diag leaves it (kPanelExp ints
-// per matrix: the exponents, and 0 behind them where they differ by three or less and nothing is scaled:
-// FP64 multiplies on every entry cost the H/h = 12 cube 2 of 78 ms).  Plain product: from the square
-// roots of B's diagonal.
+// largest.  Panel solve: D^-1 from the square roots of the block's diagonal before its factorisation, which
+// bound the entries of its columns (the pivots do not: where one is small because the block is nearly
+// singular, scaling by it takes the bits of all other columns), as k_diag leaves it: kPanelExp ints per
+// matrix, the exponents, and 0 behind them where they differ by three or less and nothing is scaled (FP64
+// multiplies on every entry cost the H/h = 12 cube 2 of 78 ms).  Plain product: the square roots of B's
+// diagonal.
 template <typename T>
 struct ColScale {
   const int *pexp = nullptr;      // panel solve
@@ -721,7 +723,7 @@ __global__ void __launch_bounds__(256) k_diag(const MatDesc *__restrict__ desc, 
   T *P = reinterpret_cast<T *>(smem_raw);  // [64][65] the block, lower, identity past w
   T *Y = P + kDP * kDLD;                        // [64][65] its inverse
   T *Tm = Y + kDP * kDLD;                       // [32][33]
-  __shared__ T Lc[4][2][32], piv[32];
+  __shared__ T Lc[4][2][32], piv[32], dg[kDP];  // dg: the diagonal before the factorisation
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   T *A = base + d.off + (long long)K0 * d.ld + K0;
   {
@@ -733,6 +735,7 @@ __global__ void __launch_bounds__(256) k_diag(const MatDesc *__restrict__ desc, 
     for (int q = 0; q < 16; ++q) {
       P[i * kDLD + j0 + q] = v[q];
       Y[i * kDLD + j0 + q] = T(0);
+      if (i == j0 + q) dg[i] = v[q];
     }
   }
   bool bad = false;
@@ -799,15 +802,14 @@ __global__ void __launch_bounds__(256) k_diag(const MatDesc *__restrict__ desc, 
   __syncthreads();
   if (bad && lane == 0) atomicOr(err, DEV_ERR_NOT_SPD);
   T *out = pinv + (long long)blockIdx.x * kDP * kDP;
-  if (tid < 32) {  // exponents of the inverse's diagonal, for the column scaling of the panel solve
+  if (tid < 32) {  // column scaling of the panel solve
     int e[2], lo = 1 << 20, hi = -(1 << 20);
 #pragma unroll
     for (int c = 0; c < 2; ++c) {
       const int i = lane + 32 * c;
-      const T y = Y[i * kDLD + i];
-      const int m = mag_bits(y);
-      const bool use = i < w && m > 0 && !mag_bad(y, m);
-      e[c] = use ? mag_exp(y, m) : 0;
+      const int m = mag_bits(dg[i]);
+      const bool use = i < w && m > 0 && !mag_bad(dg[i], m);
+      e[c] = use ? -((mag_exp(dg[i], m) + 1) >> 1) : 0;
       if (use) {
         lo = min(lo, e[c]);
         hi = max(hi, e[c]);

@@ -91,7 +91,7 @@ struct SliceWs {               // workspace: digit planes and row exponents; a p
   unsigned char *mem = nullptr;
   size_t bytes = 0;
   void *pinv = nullptr;
-  int *pexp = nullptr;         // exponents of its diagonal, kPanelExp ints per matrix
+  int *pexp = nullptr;         // column exponents of the panel solve, kPanelExp ints per matrix
 };
 
 // dense.cu -- batched partial Cholesky: eliminates the first e columns of every
