@@ -161,7 +161,10 @@ typedef struct {
    * the tensor cores (tcgen05) as exact products of bf16 digits, at FP32 rounding;
    * 2 = also the panels, 64 columns wide, whose rows are one tensor-core product
    * with the inverse of the panel's factored diagonal block.  BD_FP64 always does
-   * both, with the digits of FP64 */
+   * both, with the digits of FP64.  Entries are cut 26 bits (FP32) and 55 bits
+   * (FP64) below the power of two of their row's largest over 64 and 128 columns,
+   * FP64 operators 55 bits below that of a 32 x 32 tile scaled by the diagonal:
+   * the errors are those of a backward-stable sum, not of every entry by itself */
   int use_tensor_cores;
   /* 1 = chord Newton: factorise the Jacobian at the first Newton iterate of a
    * time step and reuse it for the later iterations of that step (every iterate

@@ -35,7 +35,7 @@ constexpr size_t kWsCap64 = (size_t)1 << 30, kWsCap32 = (size_t)512 << 20, kWsCa
 constexpr size_t kSpareBytes = (size_t)256 << 20;
 
 // order from which a deluxe product runs on the tensor cores: FP64 n = 242 took 10.2 ms per Jacobian in
-// SIMT and about 1 ms so; below, a 128 x 64 tile is mostly padding
+// SIMT and about 1 ms so; below, a 128 x 64 tile is mostly padding (orders between were not timed)
 constexpr int kProductMin = 48;
 
 inline int pad8(int n) { return (n + 7) & ~7; }

@@ -218,7 +218,7 @@ long long launch_count() { return g_launches.load(); }
 // mode 2 (outer):    rows [K1, m),   cols [K1, e),            K = [K0, K1)
 // mode 1 (final):    rows [e, m),    cols [e, m),             K = [0, e)
 // K is consumed in chunks of 16 with the next chunk prefetched into registers while the
-// current one is used.  (The FP64 updates run on the tensor cores, tc64.cu.)
+// current one is used.  (The FP64 updates run on the tensor cores, digits.cu.)
 constexpr int kTB2 = 128, kKC2 = 16;
 
 __global__ void __launch_bounds__(256) k_rankk128(const MatDesc *__restrict__ desc, float *__restrict__ base,
@@ -362,7 +362,9 @@ static double band_entries(const MatDesc &hd, int t0, int ke, int cend) {
 // first the columns of the next outer block, then, beside that block's panels on a second stream, the
 // columns right of it, on kAheadSms fewer CTAs so that the panels find free SMs.  The two sides share
 // no column, and the digit planes of the panels' own updates take half of the workspace.  A Jacobian
-// of the masked shell (coarse matrix of 2,618 unknowns) takes 3 % less, of the 128x128x32 slab too.
+// of the masked shell (coarse matrix of 2,618 unknowns) takes 3 % less, of the 128x128x32 slab too.  Both
+// constants come from these coarse matrices (40 SMs: the same); batches of 9 to about 100 matrices, whose
+// panels leave as many SMs idle, were not tried.
 constexpr int kAheadCount = 8, kAheadSms = 24;
 
 template <typename T>
@@ -732,7 +734,9 @@ size_t symv_smem(int max_n) {
 // partial-sum round trip and shorter prefetch runs), largest first, and the ones that would make up
 // a last, part-empty wave split over several CTAs.  Which ones and into how many parts is decided by
 // scheduling the CTAs on the slots with a cost of their tiles plus a fixed part (staging, reduction),
-// for every candidate.  1,024 matrices of order 772 on 456 slots: 3 waves of whole matrices, 2.3 so.
+// for every candidate.  1,024 matrices of order 772 on 304 slots (two CTAs an SM): 112 of them in halves,
+// three waves of whole matrices and one of halves instead of four.  The fixed parts were fitted when
+// three CTAs shared an SM and not again.
 std::vector<SymvTask> symv_plan(const std::vector<SymvTask> &tasks, int slots, int *scratch_rows, int *counters) {
   constexpr double kFix = 24.0, kSplitFix = 20.0;  // in tiles of 32 x 32
   const int n = (int)tasks.size();

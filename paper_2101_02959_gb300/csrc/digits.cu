@@ -8,13 +8,18 @@
 // holds exactly.  A product of two rows is sum_w B^{2D-w} P_w with P_w = sum_{s+t=w} sum_k d_s e_t; each
 // P_w is an integer below 2^24, so the FP32 accumulators of tcgen05.mma hold it exactly.
 //   FP64: B = 256, D = 7 (55 bits), groups of 128 columns (7 * 128 * 2^14 < 2^24), w = 2 .. 9, 34 of
-//   the 49 digit products; what is left out is below 2^-57 of the largest product, the operands'
-//   rounding below 2^-56 of the row's largest entry.  The P_w are combined as 64-bit integers,
-//   rounded once to FP64, scaled back and added in FP64.
+//   the 49 digit products.  With rows below 2^er and 2^ec over a group: an operand's rounding is at most
+//   2^(er - 56) (2^-55 of the row's largest entry), the digit products left out 2^-61 2^(er + ec) a column.
+//   The P_w are combined as 64-bit integers in units of weight 7, into which weights 8 and 9 are
+//   rounded (2^-55 2^(er + ec) a group), converted to FP64 with one rounding, scaled back and added.
 //   FP32: B = 512, D = 3 (26 bits), groups of 64 columns (3 * 64 * 2^16 < 2^24), w = 2 .. 4, 6 of the 9
-//   digit products, combined and added in FP32: one rounding per group where a chain of FP32
-//   multiply-adds has one per column and an FP32 accumulator of the tensor cores loses the low bits at
-//   every step.
+//   digit products: 2^(er - 27) for an operand, 2^-26 2^(er + ec) a column left out, combined and added
+//   in FP32: one rounding per group where a chain of FP32 multiply-adds has one per column and an FP32
+//   accumulator of the tensor cores loses the low bits at every step.
+// These are bounds below the rows' largest entries.  A Cholesky factor's rows are bounded by their
+// diagonals, so there they are those of any backward-stable sum; the products of two different matrices
+// scale the columns first (ColScale).  FP64 rows' products below 2^-968 are lost (matrices of entries
+// below 1e-290); FP32 keeps its whole range.
 //
 // Two kernels: k_slice writes the digit planes of the rows an update reads, in the order the
 // MMA kernel's shared-memory operands have, so that every operand tile is one contiguous bulk copy;
@@ -164,6 +169,10 @@ __device__ __forceinline__ T col_factor(const ColScale<T> &c, int b, int k) {
   return exp2i(T(0), c.sign * max(-most, min(e, most)));
 }
 
+// One team of Grp / 8 threads per row and group of columns, 8 columns a thread: the row's scale from
+// the largest magnitude of the group, then the digits of every entry.  The long-K launch of 32 matrices
+// of H/h = 8 moves 323 MB in 94 us (3.4 TB/s, most of it planes of 14 bytes per entry; the FP64 pipe is
+// 68 % busy with a multiply and a conversion per entry), in FP32 120 MB in 49 us.
 template <typename T>
 __global__ void __launch_bounds__(256) k_slice(const MatDesc *__restrict__ desc, const T *__restrict__ base,
                                                Upd64 u, const T *__restrict__ pinv, unsigned char *__restrict__ sl,
@@ -383,9 +392,12 @@ __device__ __forceinline__ void drain(uint32_t taddr, uint32_t bfree, int lane, 
 // accumulators after each group of columns and at a tile's end subtract the sums from C, while
 // loads and MMAs run on into the next group and tile; an accumulator is refilled as soon as it has
 // been read.  64 columns: eight FP64 accumulators fill tensor memory, and a wider FP32 tile measured
-// slower where the matrices are small (26 ms of updates against 35 on the masked shell).  Bound by
-// shared memory (an MMA takes 65 clocks, measured, where the tensor pipe needs 32, since A is read
-// again by every MMA) and, for short K, by reading and writing C between groups.
+// slower where the matrices are small (26 ms of updates against 35 on the masked shell).  Counters (32
+// matrices of H/h = 8): the long-K update takes 517 us in FP64 with the tensor pipe 18 % active, the FP64
+// pipe 38 % and DRAM at 13 %, 131 us in FP32 with 13 %, none and 10 %; short ones 4 to 7 % and 5 to 10 %.
+// So neither the tensor pipe nor memory bounds it: an MMA reads A again from shared memory, and between
+// groups the MMAs wait for the drain, which in FP64 does not fit its 96 registers (628 bytes of spill
+// stores a thread); for short K the reading and writing of C is added.
 template <typename T>
 __global__ void __launch_bounds__(kUThreads, 1) k_update(const MatDesc *__restrict__ desc,
                                                          const MatDesc *__restrict__ out, T *__restrict__ base, Upd64 u,
@@ -621,8 +633,8 @@ __global__ void __launch_bounds__(kUThreads, 1) k_update(const MatDesc *__restri
 // place, its 32 x 32 diagonal blocks to the block store and the inverse Y = L_11^-1 to pinv, so
 // the rows below become one product on the tensor cores.
 //
-// A warp issues one FP64 instruction in 64 clocks (measured, dependent or not) and the SM four of
-// them at a time, so the work is spread over the four schedulers: in ldl_inv32 warps 0-3 hold
+// A warp's FP64 instruction takes 64 clocks of its scheduler (2 multiply-adds a clock and SM), four warps
+// of an SM at a time (70 to 74 us a launch, the FP64 pipe 59 % busy on the SMs that have a matrix), so the work is spread over the four schedulers: in ldl_inv32 warps 0-3 hold
 // every fourth column of the block and of its inverse (lane = row) and eliminate one column a step,
 // root-free: the step's chain is one update, one reciprocal, one scaling, and the other updates run
 // beside it; the square roots of the 32 pivots are taken together at the end.
@@ -834,7 +846,8 @@ __global__ void __launch_bounds__(256) k_diag(const MatDesc *__restrict__ desc, 
 // One CTA per matrix, 32 columns at a time: factor and inverse as above, the block's rows below by
 // that inverse (warp = four columns, lane = row), rank-32 update of the rest (4 x 4 tiles a thread).
 // A latency chain of 128 pivots: 44 us with one warp factoring and one thread per row substituting,
-// 33 us here.  The inverses of the four 32 x 32 diagonal blocks go to pinv.  A coarse matrix of 2,600 unknowns runs 21 of these one after another.
+// 33 us here.  The inverses of the four 32 x 32 diagonal blocks go to pinv.  A coarse matrix of 2,600
+// unknowns runs 21 of these one after another.
 constexpr int kWP = kEnginePanel, kWLD = kWP + 1;
 constexpr size_t kDiag128Smem = sizeof(float) * (size_t)kWP * kWLD;
 

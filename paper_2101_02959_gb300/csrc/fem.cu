@@ -285,7 +285,7 @@ __global__ void k_trial(int n, const double *__restrict__ ui0, const double *__r
 // F(u) - G (Step 2) with the Jacobian factor chi Cm + tau dI/dv, and per-block
 // partial sums of ||F - G||^2.  One node per thread; the stencil's 27 slots in three batches of nine,
 // all loads of a batch in flight (a missing neighbour reads the node itself against its zero
-// coefficient).  Bound by FP64 instructions (64 clocks each per warp and scheduler: 54 stencil
+// coefficient).  Bound by FP64 instructions (2 multiply-adds a clock and SM: 54 stencil
 // multiply-adds and about 25 others) and HBM (656 bytes a node): 549,153 nodes take 82 us, 235 us
 // with divisions by the ionic parameters in the kernel, the trial point formed at every neighbour
 // and a grid that held a few loads in flight.

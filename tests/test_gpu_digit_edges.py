@@ -66,7 +66,7 @@ def test_deluxe_preconditioner(s, tc):
     assert np.max(np.abs(z - ref)) < bar * np.max(np.abs(ref))
 
 
-# 9.6e4 interface unknowns (512 threads a block) and 3.2e5 (1,024)
+# 9.8e4 interface unknowns (512 threads a block) and 3.2e5 (1,024)
 @pytest.mark.parametrize("n", [(64, 64, 40), (128, 128, 32)])
 def test_large_interfaces_under_both_krylov_methods(n):
     """PCG runs the row loops fused with its dots, GMRES the plain ones: the interface parts of the two
